@@ -29,6 +29,7 @@
 #include <vector>
 
 #include "eri_device.cuh"
+#include "eri_fixed.cuh"
 #include "eri_internal.h"
 #include "eri_tile.cuh"
 
@@ -59,7 +60,46 @@ struct PrepassArgs {
     const int32_t* shell_off;
     const double* exps;
     int* kmin;   // optional [2]: the smallest primitive-pair count K1 K2 over bra (ket) pairs
+    // optional [6]: the largest zeta_max / zeta_min of a bra (ket) pair (float
+    // bits), 1 if a primitive lies outside the fixed-point tile's range, the
+    // largest |coordinate| and the largest zeta of a bra (ket) pair (float bits)
+    int* spread;
+    const double* coefs;
 };
+
+// The fixed-point tile's range of primitives: exponents and coefficients far
+// from the ends of the FP64 range, and finite (the FP64 tile takes the rest).
+__device__ __forceinline__ bool fix_range(double z, double c)
+{
+    return z >= 1e-8 && z <= 1e8 && fabs(c) <= 1e30;
+}
+
+// zeta_max / zeta_min over the primitive pairs of shells s1, s2 (s2 < 0: the
+// unit function); *bad set where a primitive or centre is out of range, *far
+// raised to the largest |coordinate|, *zmax the largest zeta
+__device__ float pair_spread(const PrepassArgs& a, int s1, int s2, bool* bad, float* far, float* zmax)
+{
+    float lo = 0.f, hi = 0.f;
+    for (int c = 0; c < 2; ++c) {
+        const int s = c ? s2 : s1;
+        if (s < 0) continue;
+        float zl = 3e38f, zh = 0.f;
+        for (int i = a.shell_off[s]; i < a.shell_off[s] + a.shell_K[s]; ++i) {
+            *bad |= !fix_range(a.exps[i], a.coefs[i]);
+            zl = fminf(zl, (float)a.exps[i]);
+            zh = fmaxf(zh, (float)a.exps[i]);
+        }
+        for (int x = 0; x < 3; ++x) {
+            const double r = fabs(a.centres[3 * a.shell_atom[s] + x]);
+            *bad |= !(r <= 1e6);
+            *far = fmaxf(*far, __double2float_ru(r));
+        }
+        lo += zl;
+        hi += zh;
+    }
+    *zmax = hi;
+    return hi / lo;
+}
 
 // Copies the prepass results to mapped host memory.
 __global__ void info_to_host_kernel(const int* __restrict__ src, int n, int* dst)
@@ -120,6 +160,22 @@ __global__ void prepass_kernel(PrepassArgs a)
                 if (s1 >= 0 && s1 < a.nshell && (unit || (s2 >= 0 && s2 < a.nshell)))
                     kmin[side] = min(kmin[side], a.shell_K[s1] * (unit ? 1 : a.shell_K[s2]));
             }
+            if (a.spread) {
+                const int s1 = pr[2 * i], s2 = pr[2 * i + 1];
+                const bool unit = a.unit_b && side == 0;
+                if (s1 >= 0 && s1 < a.nshell && (unit || (s2 >= 0 && s2 < a.nshell))) {
+                    const int K1 = a.shell_K[s1], K2 = unit ? 1 : a.shell_K[s2];
+                    if (K1 >= 1 && K1 <= kKmax && K2 >= 1 && K2 <= kKmax) {
+                        bool bad = false;
+                        float far = 0.f, zmax;
+                        const float r = pair_spread(a, s1, unit ? -1 : s2, &bad, &far, &zmax);
+                        atomicMax(&a.spread[4 + side], __float_as_int(zmax));
+                        atomicMax(&a.spread[side], __float_as_int(r));  // r >= 1: int order = float order
+                        if (bad) a.spread[2] = 1;
+                        atomicMax(&a.spread[3], __float_as_int(far));
+                    }
+                }
+            }
             if (a.risk) {
                 const int s1 = pr[2 * i], s2 = pr[2 * i + 1];
                 if (s1 >= 0 && s1 < a.nshell && s2 >= 0 && s2 < a.nshell) {
@@ -173,6 +229,11 @@ struct PairArgs {
     int split;              // 1: E products stored as float pairs (hi, lo) in the double slots
     int hrr;                // 1: terms of E_{e,0}, |e| = l1..l1+l2 (horizontal-recursion form)
     const double* scale;    // [T] per-term factors (solid-harmonic side), or null
+    // fixed-point tile (never with ax): a pair's slots in descending order of
+    // zeta, ps holds FixPrim with coordinates in units of 2^-fx_f, and the E
+    // products carry a further zeta^(-1/2),
+    int fixed, fx_f;
+    double mu;              // and mu^(Hermite order) (eri_fixed.cuh)
 };
 
 constexpr int kEax = (kLmax + 3) * (kLmax + 3) * (2 * kLmax + 5);  // per-axis E table bound (adjoint shifts)
@@ -204,7 +265,12 @@ __global__ void pair_kernel_t(PairArgs a)
                 if (x0 != 0) continue;
                 a.zz[2 * g] = a.zz[2 * g + 1] = 1.0;
             } else {
-                for (int t = 0; t < a.T; ++t) a.E[((size_t)j * a.T + t) * a.KS + s] = 0.0;
+                for (int t = 0; t < a.T; ++t)
+                    a.E[a.fixed && !a.ket ? (size_t)g * a.T + t : ((size_t)j * a.T + t) * a.KS + s] = 0.0;
+            }
+            if (!RAISED && a.fixed) {
+                reinterpret_cast<FixPrim*>(a.ps)[g] = FixPrim{{0, 0, 0}, 1LL << 61, 1, 1.0f};
+                continue;
             }
             double* o = a.ps + (size_t)g * PS_N;
             o[PS_P] = 1.0;
@@ -219,6 +285,15 @@ __global__ void pair_kernel_t(PairArgs a)
         const double* B = s2 < 0 ? A : a.centres + 3 * a.shell_atom[s2];
         const double p = z1 + z2;
         const double invp = 1.0 / p;
+        int so = s;  // output slot
+        if (!RAISED && a.fixed) {
+            so = 0;
+            for (int x1 = 0; x1 < K1; ++x1)
+                for (int x2 = 0; x2 < K2; ++x2) {
+                    const double z = a.exps[a.shell_off[s1] + x1] + (s2 < 0 ? 0.0 : a.exps[a.shell_off[s2] + x2]);
+                    so += z > p || (z == p && x1 * K2 + x2 < s);
+                }
+        }
         const double inv2p = 0.5 * invp;
         double PA[3], PB[3], P[3], AB2 = 0.0;
         for (int x = 0; x < 3; ++x) {
@@ -234,7 +309,8 @@ __global__ void pair_kernel_t(PairArgs a)
         // bra and 1 / zeta_q on the ket: every E of the pair (per-axis tables
         // and products alike) carries it once, and [0]^(m) needs only the
         // quartet's 1/sqrt(zeta_p + zeta_q).
-        const double e00x = a.coefs[p1] * c2 * exp(-z1 * z2 * invp * AB2) * (a.ket ? invp : kTwoPi52 * invp);
+        double e00x = a.coefs[p1] * c2 * exp(-z1 * z2 * invp * AB2) * (a.ket ? invp : kTwoPi52 * invp);
+        if (!RAISED && a.fixed) e00x *= sqrt(invp);  // 1/sqrt(zeta_p + zeta_q) = sqrt(rho / (zeta_p zeta_q))
         const int ext = RAISED ? 2 : 0;
         // largest raised indices: the adjoint raises both by 2; the
         // horizontal-recursion form needs E_{i,0} for i <= l1 + l2
@@ -274,7 +350,9 @@ __global__ void pair_kernel_t(PairArgs a)
             a.zz[2 * g] = z1;
             a.zz[2 * g + 1] = z2;
         } else {
-            double* Eout = a.E + (size_t)j * a.T * a.KS + s;  // term t at Eout[t * KS]
+            // term t at Eout[t * es]: slot fastest, or (fixed-point bra) term fastest
+            const size_t es = a.fixed && !a.ket ? 1 : a.KS;
+            double* Eout = a.E + (a.fixed && !a.ket ? ((size_t)j * a.KS + so) * a.T : (size_t)j * a.T * a.KS + so);
             const int ntc = L12 + 1, n2c = a.hrr ? 1 : a.l2 + 1;  // dims the class-table indices use
             for (int t = 0; t < a.T; ++t) {
                 int idx[3], lq = 0;
@@ -287,13 +365,25 @@ __global__ void pair_kernel_t(PairArgs a)
                 double v = E[0][idx[0]] * E[NX > 1 ? 1 : 0][idx[1]] * E[NX > 2 ? 2 : 0][idx[2]];
                 if (a.scale) v *= a.scale[t];
                 if (a.ket && (lq & 1)) v = -v;
+                if (a.fixed)
+                    for (int x = 0; x < lq; ++x) v *= a.mu;
                 if (a.split)
-                    reinterpret_cast<float2*>(Eout)[(size_t)t * a.KS] = split_f64(v);
+                    reinterpret_cast<float2*>(Eout)[t * es] = split_f64(v);
                 else
-                    Eout[(size_t)t * a.KS] = v;
+                    Eout[t * es] = v;
             }
         }
-        double* o = a.ps + (size_t)g * PS_N;
+        if (!RAISED && a.fixed) {
+            FixPrim f;
+            for (int x = 0; x < 3; ++x) f.x[x] = fix_coordinate(P[x], a.fx_f);
+            // 1/zeta to 62 bits: the rounded reciprocal and its residual
+            fix_split_exponent(invp, &f.um, &f.ue);
+            f.um += (long long)(fma(-invp, p, 1.0) * (double)f.um);
+            f.zeta = (float)p;
+            reinterpret_cast<FixPrim*>(a.ps)[j * a.KS + so] = f;
+            continue;
+        }
+        double* o = a.ps + (size_t)(j * a.KS + so) * PS_N;
         o[PS_P] = p;
         o[PS_PX] = P[0];
         o[PS_PY] = P[1];
@@ -318,9 +408,11 @@ static const auto fwd_kernel_split = fwd_kernel_t<true, kNT>;
 // takes a 1 KB system reserve and a few bytes of static shared memory).
 static bool one_cta_per_sm(size_t bytes) { return 2 * (bytes + 1024 + 64) > (size_t)smem_per_sm(); }
 
-// The forward kernel for a precision and a CTA width (kNT or kNTWide).
+// The forward kernel for the transforms' arithmetic and a CTA width (kNT or kNTWide).
 static void (*fwd_kern(int split, int nt))(FwdArgs)
 {
+    if (split == XF_FIXED)
+        return nt == kNTWide ? fwd_fixed_kernel<kNTWide> : (nt == kNTSlim ? fwd_fixed_kernel<kNTSlim> : fwd_fixed_kernel<kNT>);
     if (nt == kNTWide) return split ? fwd_kernel_t<true, kNTWide> : fwd_kernel_t<false, kNTWide>;
     return split ? fwd_kernel_split : fwd_kernel;
 }
@@ -392,7 +484,7 @@ static void hrr_buffers(const ClassTables& ct, int TQ, size_t* A, size_t* B)
     }
 }
 
-bool tile_layout(const ClassTables& ct, int KB, int KK, int TQ, int IC, int e_smem, TilePlan* tp, int split)
+bool tile_layout(const ClassTables& ct, int KB, int KK, int TQ, int IC, int e_smem, TilePlan* tp, int split, int nt)
 {
     size_t off = 0;
     auto take = [&](size_t nd) {
@@ -406,6 +498,18 @@ bool tile_layout(const ClassTables& ct, int KB, int KK, int TQ, int IC, int e_sm
     tp->e_smem = e_smem;
     tp->sEbS = e_smem ? odd_up(KB * ct.Tab) : 0;
     tp->sEkS = e_smem ? odd_up(KK * ct.Tcd) : 0;
+    // the fixed-point tile: E staged, register accumulators, ket primitives
+    // in 16-byte pairs (rows of KS, quartets and rows an odd number of pairs apart)
+    const bool fixed = split == XF_FIXED;
+    const int nx = fixed ? IC : 1;  // X of a chunk's bra primitives, or of one
+    const int ps_n = fixed ? (int)(sizeof(FixPrim) / 8) : PS_N;
+    if (fixed && ct.L > kFixAuxLmax) return false;
+    if (fixed && !e_smem) return false;
+    const int KS = (KK + 1) & ~1;
+    if (fixed) {
+        tp->sEkS = r_row_stride(KS * ct.Tcd, 1);
+        tp->sEbS = odd_up(IC * ct.Tab);  // a chunk's bra primitives
+    }
     // the paired layout of the auxiliary integrals where the split form's
     // blocked ket stage packs two ket primitives per FP32 instruction, for
     // tiles that accumulate in memory: with register accumulators live
@@ -413,9 +517,10 @@ bool tile_layout(const ClassTables& ct, int KB, int KK, int TQ, int IC, int e_sm
     // on (ff|dd), K = 5: 1.27 times slower than the unpacked loop; (ff|ff),
     // K = 5, accumulating in memory: 1.06 times faster)
     const bool acc_regs = TQ * ct.nab * ct.ncd <= kNT * kNACC;
-    tp->r_pairs = split && split_block_width(ct.nhb - ct.pb0) && KK >= 2 && !acc_regs ? 1 : 0;
+    tp->r_pairs = split == XF_SPLIT && split_block_width(ct.nhb - ct.pb0) && KK >= 2 && !acc_regs ? 1 : 0;
     const int KKr = tp->r_pairs ? (KK + 1) & ~1 : KK;
-    size_t r_need = (size_t)r_row_stride(TQ * IC * KKr, tp->r_pairs) * ct.nhl;
+    size_t r_need = (size_t)(fixed ? r_row_stride(TQ * r_row_stride(IC * KS, 1), 1)
+                                   : r_row_stride(TQ * IC * KKr, tp->r_pairs)) * ct.nhl;
     size_t hA = 0, hB = 0;
     if (ct.hrr || ct.sph) {
         // the recursion (and solid-harmonic) buffers alias every staging
@@ -428,27 +533,28 @@ bool tile_layout(const ClassTables& ct, int KB, int KK, int TQ, int IC, int e_sm
             hB = std::max(hB, nf);
         }
         const size_t staged = even((size_t)TQ * tp->sEbS) + even((size_t)TQ * tp->sEkS) +
-                              even((size_t)TQ * KB * PS_N) + even((size_t)TQ * KK * PS_N) + even(r_need) +
-                              even((size_t)TQ * ct.nhb * ct.ncd);
+                              even((size_t)TQ * KB * ps_n) + even((size_t)TQ * KK * ps_n) + even(r_need) +
+                              even((size_t)TQ * ct.nhb * ct.ncd * nx);
         const size_t need = even(hA) + even(hB);
         if (staged < need) r_need += need - staged;
     }
     {
         // the Coulomb digestion of plans stages the tile's values there too
         const size_t staged = even((size_t)TQ * tp->sEbS) + even((size_t)TQ * tp->sEkS) +
-                              even((size_t)TQ * KB * PS_N) + even((size_t)TQ * KK * PS_N) + even(r_need) +
-                              even((size_t)TQ * ct.nhb * ct.ncd);
+                              even((size_t)TQ * KB * ps_n) + even((size_t)TQ * KK * ps_n) + even(r_need) +
+                              even((size_t)TQ * ct.nhb * ct.ncd * nx);
         const size_t need = even((size_t)TQ * ct.nab * ct.ncd);
-        if (TQ * ct.nab * ct.ncd <= kNT * kNACC && staged < need) r_need += need - staged;
+        if ((fixed || TQ * ct.nab * ct.ncd <= kNT * kNACC) && staged < need) r_need += need - staged;
     }
     tp->o_Eb = take((size_t)TQ * tp->sEbS);
     tp->o_Ek = take((size_t)TQ * tp->sEkS);
-    tp->o_Pb = take((size_t)TQ * KB * PS_N);
-    tp->o_Pk = take((size_t)TQ * KK * PS_N);
+    tp->o_Pb = take((size_t)TQ * KB * ps_n);
+    tp->o_Pk = take((size_t)TQ * KK * ps_n);
     tp->o_R = take(r_need);
-    tp->o_X = take((size_t)TQ * ct.nhb * ct.ncd);
+    tp->o_X = take((size_t)TQ * ct.nhb * ct.ncd * nx);
     tp->o_hB = (int)even(hA);
-    const size_t tab_bytes = 4 * (ct.nab + ct.ncd + 2) + 2 * (ct.Tab + ct.Tcd + ct.nhb * ct.nhk);
+    const size_t tab_bytes =
+        fixed ? fix_table_bytes(ct) : 4 * (ct.nab + ct.ncd + 2) + 2 * (ct.Tab + ct.Tcd + ct.nhb * ct.nhk);
     tp->o_tab = take((tab_bytes + 7) / 8);
     tp->o_q = take((size_t)TQ * 2);
     tp->o_geo = take(ct.hrr ? (size_t)TQ * 6 : 0);
@@ -458,11 +564,13 @@ bool tile_layout(const ClassTables& ct, int KB, int KK, int TQ, int IC, int e_sm
     tp->o_Ei = -1;
     if (!e_smem && TQ == 1 && (off + even(ct.Tab)) * 8 <= (size_t)max_smem_optin()) tp->o_Ei = take(ct.Tab);
     tp->o_Er = -1;  // added for the split form by add_e_ring
+    tp->o_fx = fixed ? take((fix_scratch_ints(TQ, KB, ct.ncd) + 1) / 2) : -1;
+    tp->o_acc = fixed ? take((size_t)TQ * ct.nab * ct.ncd) : -1;
     tp->bytes = off * 8;
-    tp->nt = kNT;
-    tp->acc_regs = (TQ * ct.nab * ct.ncd <= kNT * kNACC) ? 1 : 0;
+    tp->nt = fixed ? nt : kNT;
+    tp->acc_regs = (fixed || TQ * ct.nab * ct.ncd <= kNT * kNACC) ? 1 : 0;
     if (ct.hrr && !tp->acc_regs) return false;
-    return tp->bytes <= (size_t)max_smem_optin();
+    return tp->bytes + (fixed ? 64 : 0) <= (size_t)max_smem_optin();  // (and a few words of static shared memory)
 }
 
 // Split form: when the blocked ket stage reads its ket E rows from global
@@ -478,8 +586,51 @@ static void add_e_ring(const ClassTables& ct, int KK, TilePlan* tp)
     tp->bytes = (off + nd) * 8;
 }
 
+// Tile shape of the fixed-point tile where none has been timed: the least
+// modelled time.  A stage's round (one item per thread) costs its unit, in
+// clocks of an SM whose 512 threads (registers allow no more) all run it, shared
+// by the threads that do, but at least a third of it (one warp's latency); chunks
+// and tiles add their barriers and set-up.  The units are rough figures of the
+// stages timed on (pp|ps) and (dd|dd).
+static bool plan_fixed_tile(const ClassTables& ct, int KB, int KK, int64_t nq, TilePlan* best, size_t max_bytes)
+{
+    bool found = false;
+    double best_time = 0.0;
+    const double unit_a_low[5] = {200, 350, 550, 800, 1300};
+    const double unit_a = ct.L <= 4 ? unit_a_low[ct.L] : 12.0 * ct.nhl * ct.L;
+    const double unit_b = 150 + 24.0 * KK * ct.Tcd / ct.ncd, unit_c = 150;
+    for (int nt : {kNTSlim, kNT, kNTWide}) {
+        if (max_bytes && nt != kNT) continue;  // plans launch kNT threads
+        for (int TQ = 1; TQ <= 128 && (TQ == 1 || TQ < 2 * nq); TQ *= 2)
+            for (int IC : {KB, (KB + 1) / 2, (KB + 2) / 3, 1}) {
+                TilePlan tp;
+                if (!tile_layout(ct, KB, KK, TQ, IC, 1, &tp, XF_FIXED, nt) || (max_bytes && tp.bytes > max_bytes)) continue;
+                const int64_t tiles = (nq + TQ - 1) / TQ;
+                int64_t per_sm = std::min<int64_t>(kNTWide / nt, (int64_t)smem_per_sm() / (int64_t)(tp.bytes + 1088));
+                if (per_sm < 1) continue;
+                per_sm = std::min<int64_t>(per_sm, (tiles + sm_count() - 1) / sm_count());
+                const double share = std::max(1.0 / 3, (double)(per_sm * nt) / kNTWide);
+                auto rounds = [&](double items) { return std::ceil(items / nt); };
+                const int chunks = (KB + IC - 1) / IC;
+                const double t_chunk =
+                    800 + share * (rounds((double)TQ * IC * KK) * unit_a +
+                                   rounds(0.25 * TQ * IC * (ct.nhb - ct.pb0) * ct.ncd) * unit_b +
+                                   rounds(0.5 * TQ * ct.nab * ct.ncd) * (unit_c + 10.0 * IC * ct.Tab / ct.nab));
+                const double time = std::ceil((double)tiles / (double)(per_sm * sm_count())) *
+                                    (4000 + share * rounds((double)TQ * KB * KK) * 60 + chunks * t_chunk);
+                if (!found || time < best_time) {
+                    best_time = time;
+                    *best = tp;
+                    found = true;
+                }
+            }
+    }
+    return found;
+}
+
 bool plan_tiles(const ClassTables& ct, int KB, int KK, int64_t nq, TilePlan* best, size_t max_bytes, int split)
 {
+    if (split == XF_FIXED) return plan_fixed_tile(ct, KB, KK, nq, best, max_bytes);
     bool found = false;
     double best_score = -1.0;
     for (int e_smem = 1; e_smem >= 0; --e_smem) {
@@ -532,6 +683,53 @@ static int dev_err_to_code(int e)
 }
 
 static size_t align_up(size_t n) { return (n + 255) & ~size_t(255); }
+
+// Whether a batch of class cls may run the fixed-point tile: every primitive
+// in its range, and no pair whose exponents spread further than the scales
+// allow (eri_fixed.cuh).  info: PrepassArgs::spread.
+static bool fixed_eligible(eri_class_t cls, const int32_t* info)
+{
+    if (info[2]) return false;
+    for (int side = 0; side < 2; ++side) {
+        float r;
+        std::memcpy(&r, &info[side], 4);
+        const int l = side ? cls.lc + cls.ld : cls.la + cls.lb;
+        if (!(0.5f * (float)l * std::log2(r) <= kFixSpreadBits)) return false;
+    }
+    return true;
+}
+
+// mu of the Hermite unit: 1.1 sqrt(2 rho) = mu 2^n, mu in [1, 2), for the
+// largest reduced exponent rho of the batch (kept a little below, so that
+// fix_sigma's float product does not round past the power of two).
+static double fix_unit(double rho)
+{
+    const double s = 1.1 * std::sqrt(2.0 * rho);
+    return s > 0.0 ? s / std::ldexp(1.0, std::ilogb(s)) * 1.00001 : 1.0;
+}
+
+// The fixed-point form of one side's pair tables (in place on the bra).
+static void launch_fix_pairs(const PairTables& t, const ClassTables& ct, int64_t npairs, int KS, int side, double mu,
+                             cudaStream_t st)
+{
+    FixPairArgs f{};
+    f.E = t.E;
+    f.ps = reinterpret_cast<const FixPrim*>(t.ps);
+    f.kp = t.kp;
+    f.start = side ? ct.ket_start : ct.bra_start;
+    f.herm = side ? ct.ket_q : ct.bra_p;
+    f.npairs = npairs;
+    f.KS = KS;
+    f.T = side ? ct.Tcd : ct.Tab;
+    f.ncol = side ? ct.ncd : ct.nab;
+    f.ket = side;
+    f.c = (float)(2.42 / (mu * mu));
+    f.ex = t.ex;
+    f.norm = t.norm;
+    const int64_t n = npairs * f.ncol;
+    count_launch();
+    fix_pairs_kernel<<<(int)std::max<int64_t>(1, std::min<int64_t>((n + 127) / 128, 16LL * sm_count())), 128, 0, st>>>(f);
+}
 
 // Prepass + pair tables shared by the forward and adjoint entry points.
 // On success fills the pair tables and the largest K on each centre.
@@ -588,22 +786,36 @@ int prepare_batch(eri_class_t cls, const eri_basis_t* basis, const int32_t* bra,
         fc->form = 0;
         fc->alt = -1;
         fc->cached = 0;
+        fc->fixed = 0;
     }
     int* status = device_status();
     if (!status) return ERI_ECUDA;
     int32_t* hinfo = host_pinned_i32(16);
     if (!hinfo) return ERI_ENOMEM;
     // info lives in the status block (slots 8..16), separate from the error word:
-    // [0..6] as PrepassArgs::info, [7..8] the smallest pair counts per side
+    // [0..6] as PrepassArgs::info, [7..8] the smallest pair counts per side,
+    // [9..14] PrepassArgs::spread
     int* dinfo = status + 8;
     if (cudaMemsetAsync(dinfo, 0, 7 * sizeof(int), st) != cudaSuccess ||
-        cudaMemsetAsync(dinfo + 7, 0x7f, 2 * sizeof(int), st) != cudaSuccess)
+        cudaMemsetAsync(dinfo + 7, 0x7f, 2 * sizeof(int), st) != cudaSuccess ||
+        cudaMemsetAsync(dinfo + 9, 0, 6 * sizeof(int), st) != cudaSuccess)
         return ERI_ECUDA;
+    // Where the fixed-point tile is the faster one (GB300, ms, FP64 against fixed
+    // point): contracted 4-centre classes above (ss|ss): (pp|ps) K = 3, 1e5
+    // quartets 3.48 / 2.31; (ds|ds) 6.76 / 3.70; (dp|pp), 6.5e4, 10.6 / 7.9.  Not
+    // (ss|ss), 4e5 of mixed degrees 5.12 / 5.37, whose tiles hold few primitive
+    // quartets; not uncontracted batches, where set-up and barriers outweigh the
+    // products: (pp|ps) 3e5 0.43 / 0.49, (ff|pp) 2e4 2.39 / 3.03; not 3-centre ones,
+    // (f|dp) 1e5 4.90 / 6.20; nor small ones, (pp|pp) K = 3, 1000 quartets 0.217 / 0.236,
+    // which are not asked for their spread either.
+    const int64_t nqq = quartets ? nq : nbra * nket;
+    const bool try_fixed = fc && !split && ldelta == 0 && (kind == 0 || kind == 3) &&
+                           cls.la + cls.lb + cls.lc + cls.ld > 0 && nqq >= 2000;
     PrepassArgs pa{basis->shell_l, basis->shell_K, basis->nshell, bra, nbra, ket, nket, quartets,
                    quartets ? nq : (int64_t)0,
                    {cls.la, cls.lb, cls.lc, cls.ld}, (kind == 1 || kind == 2) ? 1 : 0, dinfo,
                    allow_swap > 1 ? 1 : 0, basis->centres, basis->shell_atom, basis->shell_off, basis->exps,
-                   dinfo + 7};
+                   dinfo + 7, try_fixed ? dinfo + 9 : nullptr, basis->coefs};
     const int64_t n = std::max(std::max(nbra, nket), quartets ? nq : (int64_t)0);
     const int grid = (int)std::min<int64_t>((n + 255) / 256, 4 * sm_count());
     {
@@ -617,11 +829,11 @@ int prepare_batch(eri_class_t cls, const eri_basis_t* basis, const int32_t* bra,
     int32_t* hmapped = nullptr;
     if (cudaHostGetDevicePointer((void**)&hmapped, hinfo, 0) == cudaSuccess && hmapped) {
         count_launch();
-        info_to_host_kernel<<<1, 32, 0, st>>>(dinfo, 9, hmapped);
+        info_to_host_kernel<<<1, 32, 0, st>>>(dinfo, 15, hmapped);
         if (cudaGetLastError() != cudaSuccess) return ERI_ECUDA;
     } else {
         cudaGetLastError();
-        if (cudaMemcpyAsync(hinfo, dinfo, 9 * sizeof(int), cudaMemcpyDeviceToHost, st) != cudaSuccess)
+        if (cudaMemcpyAsync(hinfo, dinfo, 15 * sizeof(int), cudaMemcpyDeviceToHost, st) != cudaSuccess)
             return ERI_ECUDA;
     }
     if (cudaStreamSynchronize(st) != cudaSuccess) return ERI_ECUDA;
@@ -630,6 +842,7 @@ int prepare_batch(eri_class_t cls, const eri_basis_t* basis, const int32_t* bra,
     *KB = kmax[0] * kmax[1];
     *KK = kmax[2] * kmax[3];
     if (mixed) *mixed = (hinfo[7] < *KB || hinfo[8] < *KK) ? 1 : 0;
+    const bool fix_ok = try_fixed && (int64_t)*KB * *KK >= 4 && nqq * *KB * *KK >= 150000 && fixed_eligible(cls, hinfo + 9);
     if (allow_swap) {
         // Four forms: which side is transformed first (Section 3.2.2
         // transforms the ket first, assuming it has the lower l) and whether
@@ -651,7 +864,6 @@ int prepare_batch(eri_class_t cls, const eri_basis_t* basis, const int32_t* bra,
             opt[3] = tables(cls.lc, cls.ld, cls.la, cls.lb, 0, 1);
             if (!opt[2] || !opt[3]) return err;
         }
-        const int64_t nqq = quartets ? nq : nbra * nket;
         double cost[4];
         for (int o = 0; o < 4; ++o) {
             cost[o] = -1.0;  // infeasible
@@ -664,8 +876,11 @@ int prepare_batch(eri_class_t cls, const eri_basis_t* basis, const int32_t* bra,
                 TilePlan tp;
                 if (c->nab * c->ncd > kNT * kNACC || !plan_tiles(*c, (int)kb, (int)kk, nqq, &tp)) continue;
             }
+            // a recursion step is an FP64 operation, which costs several
+            // products of the fixed-point transforms
+            const double step = fix_ok ? 6.0 : 1.0;
             cost[o] = kb * kk * ((c->nhb - c->pb0) * c->Tcd + 0.5 * c->nhl) + kb * c->ncd * c->Tab +
-                      (c->hrr ? c->nab * c->nks + c->ncd_f * c->nbs : 0);
+                      (c->hrr ? step * (c->nab * c->nks + c->ncd_f * c->nbs) : 0);
         }
         {
             // the caller's form mask (eri_set_forms), unless it leaves no feasible form
@@ -687,7 +902,7 @@ int prepare_batch(eri_class_t cls, const eri_basis_t* basis, const int32_t* bra,
             if (forced > 3 || cost[forced] < 0) return ERI_EINVAL;
             best = forced;
         } else {
-            best = lookup_form(cls, *KB, *KK, split, kind);
+            best = lookup_form(cls, *KB, *KK, fix_ok ? XF_FIXED : split, kind);
             if (best >= 0 && cost[best] >= 0) {
                 if (fc) fc->cached = 1;
             } else {
@@ -709,9 +924,29 @@ int prepare_batch(eri_class_t cls, const eri_basis_t* basis, const int32_t* bra,
             std::swap(kmax[1], kmax[3]);
         }
     }
+    // the fixed-point tile where its precision and its shared memory allow
+    TilePlan fix_tile;
+    const bool fixed = fix_ok && plan_tiles(*ct, *KB, *KK, nqq, &fix_tile, 0, XF_FIXED);
+    int fx_f = 0;
+    double mu = 1.0;
+    if (fixed) {  // |coordinate| 2^fx_f < 2^60
+        float far;
+        std::memcpy(&far, &hinfo[12], 4);
+        fx_f = 60 - std::max(-10, far > 0.f ? std::ilogb(far) + 1 : -10);
+        float zb, zk;
+        std::memcpy(&zb, &hinfo[13], 4);
+        std::memcpy(&zk, &hinfo[14], 4);
+        mu = fix_unit((double)zb * zk / ((double)zb + zk));
+    }
+    if (fc) {
+        fc->fixed = fixed;
+        fc->fx_f = fx_f;
+        fc->mu = mu;
+    }
     // workspace: pair tables of both sides
-    const size_t nb_ps = align_up(sizeof(double) * nbra * *KB * PS_N), nb_E = align_up(sizeof(double) * nbra * *KB * ct->Tab);
-    const size_t nk_ps = align_up(sizeof(double) * nket * *KK * PS_N), nk_E = align_up(sizeof(double) * nket * *KK * ct->Tcd);
+    const size_t ps_n = fixed ? sizeof(FixPrim) / 8 : PS_N;
+    const size_t nb_ps = align_up(sizeof(double) * nbra * *KB * ps_n), nb_E = align_up(sizeof(double) * nbra * *KB * ct->Tab);
+    const size_t nk_ps = align_up(sizeof(double) * nket * *KK * ps_n), nk_E = align_up(sizeof(double) * nket * *KK * ct->Tcd);
     const size_t nb_k = align_up(sizeof(int32_t) * nbra), nk_k = align_up(sizeof(int32_t) * nket);
     // ldelta 1: the raised tables of the kernel bra only (the adjoint launch
     // for one side's channels); 2: of both sides, with the E products of
@@ -723,7 +958,11 @@ int prepare_batch(eri_class_t cls, const eri_basis_t* basis, const int32_t* bra,
     const size_t nk_ax = grad_both ? align_up(sizeof(double) * nket * *KK * 3 * eaxk) : 0;
     const size_t nb_z = grad ? align_up(sizeof(double) * nbra * *KB * 2) : 0;
     const size_t nk_z = grad_both ? align_up(sizeof(double) * nket * *KK * 2) : 0;
-    uint8_t* ws = (uint8_t*)workspace(nb_ps + nb_E + nk_ps + nk_E + nb_k + nk_k + nb_ax + nk_ax + nb_z + nk_z, &err);
+    const size_t nb_x = fixed ? align_up(sizeof(int32_t) * nbra * ct->nab) : 0;
+    const size_t nk_x = fixed ? align_up(sizeof(int32_t) * nket * ct->ncd) : 0;
+    const size_t nk_n = fixed ? align_up(sizeof(float) * 8 * nket * ct->ncd) : 0;
+    const size_t n_grad = nb_ax + nk_ax + nb_z + nk_z;
+    uint8_t* ws = (uint8_t*)workspace(nb_ps + nb_E + nk_ps + nk_E + nb_k + nk_k + n_grad + nb_x + nk_x + nk_n, &err);
     if (!ws) return err;
     {
         uint8_t* g0 = ws + nb_ps + nb_E + nk_ps + nk_E + nb_k + nk_k;
@@ -733,6 +972,10 @@ int prepare_batch(eri_class_t cls, const eri_basis_t* basis, const int32_t* bra,
         pk->zz = grad_both ? (double*)(g0 + nb_ax + nk_ax + nb_z) : nullptr;
         pb->eax = eaxb;
         pk->eax = eaxk;
+        pb->ex = fixed ? (int32_t*)(g0 + n_grad) : nullptr;
+        pk->ex = fixed ? (int32_t*)(g0 + n_grad + nb_x) : nullptr;
+        pk->norm = fixed ? (float*)(g0 + n_grad + nb_x + nk_x) : nullptr;
+        pb->norm = nullptr;
     }
     pb->ps = (double*)ws;
     pb->E = (double*)(ws + nb_ps);
@@ -764,6 +1007,9 @@ int prepare_batch(eri_class_t cls, const eri_basis_t* basis, const int32_t* bra,
         p.eax = t.eax;
         p.zz = t.zz;
         p.split = split;
+        p.fixed = fixed;
+        p.fx_f = fx_f;
+        p.mu = mu;
         p.hrr = ct->hrr;
         p.scale = side ? ct->ket_scale : ct->bra_scale;
         const int64_t tot = p.npairs * p.KS;
@@ -776,6 +1022,7 @@ int prepare_batch(eri_class_t cls, const eri_basis_t* basis, const int32_t* bra,
             launch_pair(pe, std::max(g, 1), st);
         }
         launch_pair(p, std::max(g, 1), st);
+        if (fixed) launch_fix_pairs(t, *ct, p.npairs, p.KS, side, mu, st);
         if (cudaGetLastError() != cudaSuccess) return ERI_ECUDA;
     }
     return ERI_OK;
@@ -839,6 +1086,21 @@ static bool tuned_tile(const FwdArgs& base, int split, cudaStream_t st, TilePlan
     }
     std::vector<TilePlan> cands;
     for (int TQ = 1; TQ <= 128; TQ *= 2) {
+        if (split == XF_FIXED) {
+            for (int IC : {base.KB, (base.KB + 1) / 2, (base.KB + 2) / 3, 1})
+                for (int nt : {kNTSlim, kNT, kNTWide}) {
+                    TilePlan tp;
+                    if (!tile_layout(ct, base.KB, base.KK, TQ, IC, 1, &tp, split, nt)) continue;
+                    // at least half as many CTAs per SM as the registers hold
+                    if ((kNTWide / nt) * (tp.bytes + 1088) > 2 * (size_t)smem_per_sm()) continue;
+                    bool dup = false;
+                    for (auto& c : cands) dup |= c.TQ == TQ && c.IC == IC && c.nt == nt;
+                    // a chunk with too few or far too many items for the CTA is not worth timing
+                    const int items = TQ * IC * base.KK;
+                    if (!dup && (items * 8 >= nt || TQ == 1) && items <= 16 * nt) cands.push_back(tp);
+                }
+            continue;
+        }
         if (TQ * ct.nab * ct.ncd > kNT * kNACC) break;
         for (int IC : {base.KB, (base.KB + 1) / 2, 1}) {
             for (int es = 1; es >= 0; --es) {
@@ -852,7 +1114,7 @@ static bool tuned_tile(const FwdArgs& base, int split, cudaStream_t st, TilePlan
                     const bool wide = one_cta_per_sm(tp.bytes);
                     TilePlan tw = tp;
                     tw.nt = kNTWide;
-                    if (split) {
+                    if (split == XF_SPLIT) {
                         add_e_ring(ct, base.KK, &tp);
                         add_e_ring(ct, base.KK, &tw);
                     }
@@ -873,8 +1135,10 @@ static bool tuned_tile(const FwdArgs& base, int split, cudaStream_t st, TilePlan
         FwdArgs a = base;
         set_tile(a, tp);
         void (*kern)(FwdArgs) = fwd_kern(split, tp.nt);
-        if (cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)tp.bytes) != cudaSuccess)
+        if (cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)tp.bytes) != cudaSuccess) {
+            cudaGetLastError();
             continue;
+        }
         int per_sm = 0;
         cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per_sm, kern, tp.nt, tp.bytes);
         const int64_t slots = (int64_t)std::max(per_sm, 1) * sm_count();
@@ -1024,7 +1288,7 @@ extern "C" int eri_boys(int mmax, const double* T, int64_t n, double* F, void* s
 static int forward_args(const eri_basis_t* basis, const int32_t* bra_pairs, int64_t nbra,
                         const int32_t* ket_pairs, int64_t nket, const int64_t* quartets, int64_t nqq, double* out,
                         const ClassTables* ct, const PairTables& pb, const PairTables& pk, int KB, int KK, int swapped,
-                        int split, cudaStream_t st, FwdArgs* a, TilePlan* tp)
+                        int split, const FormChoice& fc, cudaStream_t st, FwdArgs* a, TilePlan* tp)
 {
     int err = ERI_OK;
     const double* boys = get_boys_table(ct->L, st, &err);
@@ -1033,6 +1297,16 @@ static int forward_args(const eri_basis_t* basis, const int32_t* bra_pairs, int6
     if (!rs) return err;
     if (!plan_tiles(*ct, KB, KK, nqq, tp, 0, split)) return ERI_EINVAL;
     *a = FwdArgs{};
+    if (split == XF_FIXED) {
+        const int64_t* fx = get_fix_boys_table(ct->L, st, &err);
+        if (!fx) return err;
+        a->fx_tab = reinterpret_cast<const long long*>(fx);
+        a->fx_far = a->fx_tab + (size_t)kFixBoysRows * fix_boys_words(ct->L);
+        a->fx_f = fc.fx_f;
+        a->fx_c = (float)(2.42 / (fc.mu * fc.mu));
+        a->fx_imu = (float)(1.0 / fc.mu);
+        a->fx_rmu = (long long)(0x1p62L / (long double)fc.mu);
+    }
     a->ct = *ct;
     a->boys = boys;
     a->rsteps = rs;
@@ -1042,6 +1316,9 @@ static int forward_args(const eri_basis_t* basis, const int32_t* bra_pairs, int6
     a->ket_ps = pk.ps;
     a->ket_E = pk.E;
     a->ket_kp = pk.kp;
+    a->bra_ex = pb.ex;
+    a->ket_ex = pk.ex;
+    a->ket_norm = pk.norm;
     a->quartets = quartets;
     a->nq = nqq;
     a->nbra = nbra;  // original roles: output layout and product-form decoding
@@ -1057,6 +1334,7 @@ static int forward_args(const eri_basis_t* basis, const int32_t* bra_pairs, int6
     a->shell_atom = basis->shell_atom;
     a->KB = KB;
     a->KK = KK;
+    a->nsm = sm_count();
     set_tile(*a, *tp);
     a->ntiles = (nqq + tp->TQ - 1) / tp->TQ;
     return ERI_OK;
@@ -1093,7 +1371,7 @@ static int run_forward(eri_class_t cls, const eri_basis_t* basis, const int32_t*
                               &KK, kmax, allow, f, split, kind, &mixed);
         if (e != ERI_OK) return e;
         e = forward_args(basis, bra_pairs, nbra, ket_pairs, nket, quartets, nqq, out, ct, pb, pk, KB, KK,
-                         f->form & 1, split, st, a, tp);
+                         f->form & 1, f->fixed ? XF_FIXED : split, *f, st, a, tp);
         if (e != ERI_OK) return e;
         if (mixed && !order && nqq > 1) {
             unsigned long long* queue = nullptr;
@@ -1115,7 +1393,7 @@ static int run_forward(eri_class_t cls, const eri_basis_t* basis, const int32_t*
     if (nqq >= kTuneMinQuartets) {
         TilePlan best;
         float ms = 0.f;
-        bool tuned = tuned_tile(a, split, st, &best, &ms);
+        bool tuned = tuned_tile(a, fc.fixed ? XF_FIXED : split, st, &best, &ms);
         if (!fc.cached && fc.alt >= 0) {
             const eri_class_t sig = cls;
             const int KB0 = (fc.form & 1) ? KK : KB, KK0 = (fc.form & 1) ? KB : KK;  // caller's orientation
@@ -1125,9 +1403,9 @@ static int run_forward(eri_class_t cls, const eri_basis_t* basis, const int32_t*
             TilePlan tp1, best1;
             float ms1 = 0.f;
             bool tuned1 = false;
-            if (prepare(&f1, &a1, &tp1) == ERI_OK) tuned1 = tuned_tile(a1, split, st, &best1, &ms1);
+            if (prepare(&f1, &a1, &tp1) == ERI_OK) tuned1 = tuned_tile(a1, f1.fixed ? XF_FIXED : split, st, &best1, &ms1);
             const bool take_alt = tuned1 && (!tuned || ms1 < ms);
-            remember_form(sig, KB0, KK0, split, kind, take_alt ? f1.form : fc.form);
+            remember_form(sig, KB0, KK0, fc.fixed || f1.fixed ? XF_FIXED : split, kind, take_alt ? f1.form : fc.form);
             if (take_alt) {
                 fc = f1;
                 a = a1;
@@ -1155,11 +1433,11 @@ static int run_forward(eri_class_t cls, const eri_basis_t* basis, const int32_t*
         // only (measured on (ff|ff): FP64 1.07 and 1.14 times faster at K = 5
         // and 1, split 1.27 and 1.34), then, split, the ring of ket E rows;
         // the tuner's candidates come with both settled
-        if (one_cta_per_sm(tp.bytes)) tp.nt = kNTWide;
+        if (!fc.fixed && one_cta_per_sm(tp.bytes)) tp.nt = kNTWide;
         if (split) add_e_ring(a.ct, a.KK, &tp);
         set_tile(a, tp);
     }
-    void (*kern)(FwdArgs) = fwd_kern(split, tp.nt);
+    void (*kern)(FwdArgs) = fwd_kern(fc.fixed ? XF_FIXED : split, tp.nt);
     if (cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)tp.bytes) != cudaSuccess)
         return ERI_ECUDA;
     int per_sm = 0;

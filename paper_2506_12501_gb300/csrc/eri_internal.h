@@ -62,6 +62,11 @@ struct ClassTables {
     const int16_t* ket_q;         // [Tcd] Hermite index of q (order <= Lk)
     const uint8_t* ket_fac;       // [Tcd][6]
     const int16_t* pq;            // [nhb][nhk] Hermite index of p+q (order <= L)
+    // ket columns in pairs (c1, c2), c2 = -1 or a column whose Hermite
+    // functions are the first ones of c1, in the same order
+    int nkpair, nbpair;
+    const int16_t* kpairs;        // [nkpair][2]
+    const int16_t* bpairs;        // [nbpair][2], the bra's columns likewise
     // adjoint: Hermite ranges widened by 2 on one side (shifted functions)
     int nhb2, nhk2, nhl2;         // Nh(Lb+2), Nh(Lk+2), Nh(L+2)
     const int16_t* pq2b;          // [nhb2][nhk] Hermite index of p'+q
@@ -122,6 +127,8 @@ const ClassTables* get_class_tables_sph(int la, int lb, int lc, int ld, int hrr,
 void solid_harmonic_table(int l, double* out);
 const double* get_boys_table(int L, cudaStream_t s, int* err);    // rows of F_{L+k}(T_j)/k!, plus exp
 const RStep* get_rsteps(cudaStream_t s, int* err);                 // recursion step table (device)
+// Fixed-point Boys rows of order L (fix_boys_words(L) each), then the constants of large T
+const int64_t* get_fix_boys_table(int L, cudaStream_t s, int* err);
 void release_all();
 
 // Host table builders that allocate nothing (they fill the caller's
@@ -149,6 +156,8 @@ struct PairTables {
     double* ax;   // adjoint only: per-axis E tables with raised indices
     int eax;      // doubles per axis table
     double* zz;   // adjoint only: [npairs][KS][2] exponents
+    int32_t* ex;  // fixed-point tile: exponents of the E columns [npairs][ncol] (see eri_fixed.cuh)
+    float* norm;  // fixed-point tile, ket: their 1-norms per Hermite order [npairs][ncol][8]
 };
 
 // Form of a forward batch: bit 0 = sides swapped (the caller's ket is the
@@ -157,6 +166,9 @@ struct FormChoice {
     int form = -1;    // in: a form to force, or -1 (remembered, else modelled); out: the form used
     int alt = -1;     // out: the modelled-cheapest feasible form of the other kind (plain vs HRR), or -1
     int cached = 0;   // out: 1 when the form was remembered from an earlier timing
+    int fixed = 0;    // out: 1 when the pair tables are those of the fixed-point tile
+    int fx_f = 0;     // out: their coordinates are in units of 2^-fx_f
+    double mu = 1.0;  // out: and their Hermite unit (eri_fixed.cuh)
 };
 // Remember the measured-faster form of a (class, K_bra, K_ket, precision) signature.
 void remember_form(eri_class_t cls, int KB, int KK, int split, int kind, int form);
@@ -205,14 +217,19 @@ struct TilePlan {
     int o_Ei;         // one-quartet tile, E not staged: the bra E products of the current bra primitive ([Tab]), or -1
     int o_Er;         // split form, blocked ket stage, E not staged: three ket E rows per warp ([nt/32][3][KK] float pairs), or -1
     size_t bytes;
-    int nt;           // threads per CTA: 256 (two CTAs per SM fit the registers) or 512 (one CTA per SM)
+    int nt;           // threads per CTA: 256 (two CTAs per SM fit the registers) or 512 (one CTA per SM); fixed point: also 128
     int r_pairs;      // split form, blocked ket stage: auxiliary integrals in the paired layout (see r_row_stride)
+    int o_fx, o_acc;  // fixed-point tile: exponents and flags; accumulators
 };
+// The arithmetic of a tile's transforms: FP64, split precision, or (the
+// caller asked for FP64) 64-bit fixed point.
+enum { XF_FP64 = 0, XF_SPLIT = 1, XF_FIXED = 2 };
 // max_bytes > 0: only shapes whose shared memory stays within it; split: the
-// tile runs the split-precision transforms
+// transforms' arithmetic (XF_*)
 bool plan_tiles(const ClassTables& ct, int KB, int KK, int64_t nq, TilePlan* best, size_t max_bytes = 0,
                 int split = 0);
-bool tile_layout(const ClassTables& ct, int KB, int KK, int TQ, int IC, int e_smem, TilePlan* tp, int split = 0);
+bool tile_layout(const ClassTables& ct, int KB, int KK, int TQ, int IC, int e_smem, TilePlan* tp, int split = 0,
+                 int nt = 256);
 
 // The tile's auxiliary integrals [r]^(0) are a table of nhl rows (Hermite
 // functions) by NI columns (quartet, bra primitive, ket primitive), ket

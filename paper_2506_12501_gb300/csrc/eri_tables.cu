@@ -1,15 +1,19 @@
 // eri_tables.cu -- host-built tables of the ERI library: Hermite numbering,
 // sparse Hermite<->Cartesian term lists per class, the auxiliary-recursion
 // step table, the Boys-function tables, and the cached device workspace.
+#include <algorithm>
 #include <cmath>
 #include <cstdio>
 #include <cstring>
 #include <array>
 #include <map>
 #include <mutex>
+#include <system_error>
+#include <thread>
 #include <tuple>
 #include <vector>
 
+#include "eri_fixaux.cuh"
 #include "eri_internal.h"
 
 namespace eri {
@@ -238,6 +242,56 @@ void solid_harmonic_table(int l, double* out)
 static const ClassTables* class_tables_impl(int la, int lb, int lc, int ld, int hrr, int pure, cudaStream_t s,
                                             int* err, int sph = 0);
 
+// Pairs of columns for the fixed-point tile's ket transform, which walks two
+// columns over one read of the auxiliary integrals: each column c1 (longest
+// first) takes the longest free column c2 whose Hermite functions all occur
+// in c1 (-1: none).  The terms of c1 are reordered so that its first ones
+// are those of c2, in c2's order.
+static std::vector<int16_t> pair_columns(const std::vector<int>& start, std::vector<int16_t>& herm,
+                                         std::vector<uint8_t>& fac, std::vector<double>& scale)
+{
+    const int n = (int)start.size() - 1;
+    std::vector<int> order(n), free_col(n, 1);
+    for (int c = 0; c < n; ++c) order[c] = c;
+    auto size = [&](int c) { return start[c + 1] - start[c]; };
+    std::stable_sort(order.begin(), order.end(), [&](int x, int y) { return size(x) > size(y); });
+    std::vector<int16_t> pairs;
+    for (int c1 : order) {
+        if (!free_col[c1]) continue;
+        free_col[c1] = 0;
+        auto first = [&](int c, int16_t h) {  // position of h in column c, or -1
+            for (int t = start[c]; t < start[c + 1]; ++t)
+                if (herm[t] == h) return t;
+            return -1;
+        };
+        int c2 = -1;
+        for (int c : order) {
+            if (!free_col[c]) continue;
+            bool inside = true;
+            for (int t = start[c]; t < start[c + 1] && inside; ++t) inside = first(c1, herm[t]) >= 0;
+            if (inside) {
+                c2 = c;
+                break;
+            }
+        }
+        if (c2 >= 0) {
+            free_col[c2] = 0;
+            for (int u = 0; u < size(c2); ++u) {
+                const int to = start[c1] + u;
+                int from = first(c1, herm[start[c2] + u]);
+                for (; from > to; --from) {  // rotate the term into place
+                    std::swap(herm[from], herm[from - 1]);
+                    for (int x = 0; x < 3; ++x) std::swap(fac[3 * from + x], fac[3 * (from - 1) + x]);
+                    if (!scale.empty()) std::swap(scale[from], scale[from - 1]);
+                }
+            }
+        }
+        pairs.push_back((int16_t)c1);
+        pairs.push_back((int16_t)c2);
+    }
+    return pairs;
+}
+
 const ClassTables* get_class_tables(int la, int lb, int lc, int ld, cudaStream_t s, int* err)
 {
     return class_tables_impl(la, lb, lc, ld, 0, 0, s, err);
@@ -361,6 +415,12 @@ static const ClassTables* class_tables_impl(int la, int lb, int lc, int ld, int 
         t.nab_f = t.nab;
         t.ncd_f = t.ncd;
     }
+    // the same rule on both sides: a side's term order depends on its shells
+    // and form alone, so plans share one table between the roles
+    const std::vector<int16_t> bpairs = pair_columns(bs, bp, bf, bsc);
+    t.nbpair = (int)bpairs.size() / 2;
+    const std::vector<int16_t> kpairs = pair_columns(ks, kq, kf, ksc);
+    t.nkpair = (int)kpairs.size() / 2;
     HrrSide hb = hrr_side(la, lb), hk = hrr_side(lc, ld);
     t.nbs = (int)hb.steps.size() / 3;
     t.nks = (int)hk.steps.size() / 3;
@@ -420,6 +480,7 @@ static const ClassTables* class_tables_impl(int la, int lb, int lc, int ld, int 
         solid_harmonic_table(ls[i], c2s[i].data());
         o_c2s[i] = take(c2s[i].size() * 8);
     }
+    size_t o_kpr = take(kpairs.size() * 2), o_bpr = take(bpairs.size() * 2);
     size_t o_bsc = take(bsc.size() * 8), o_ksc = take(ksc.size() * 8);
     size_t o_bf = take(bf.size()), o_kf = take(kf.size());
     std::vector<uint8_t> host(off);
@@ -427,6 +488,8 @@ static const ClassTables* class_tables_impl(int la, int lb, int lc, int ld, int 
         if (!c2s[i].empty()) std::memcpy(host.data() + o_c2s[i], c2s[i].data(), c2s[i].size() * 8);
     if (!bsc.empty()) std::memcpy(host.data() + o_bsc, bsc.data(), bsc.size() * 8);
     if (!ksc.empty()) std::memcpy(host.data() + o_ksc, ksc.data(), ksc.size() * 8);
+    std::memcpy(host.data() + o_kpr, kpairs.data(), kpairs.size() * 2);
+    std::memcpy(host.data() + o_bpr, bpairs.data(), bpairs.size() * 2);
     std::memcpy(host.data() + o_bs, bs.data(), bs.size() * 4);
     std::memcpy(host.data() + o_ks, ks.data(), ks.size() * 4);
     std::memcpy(host.data() + o_bp, bp.data(), bp.size() * 2);
@@ -455,6 +518,8 @@ static const ClassTables* class_tables_impl(int la, int lb, int lc, int ld, int 
     t.ket_start = (const int*)(b + o_ks);
     t.bra_p = (const int16_t*)(b + o_bp);
     t.ket_q = (const int16_t*)(b + o_kq);
+    t.kpairs = (const int16_t*)(b + o_kpr);
+    t.bpairs = (const int16_t*)(b + o_bpr);
     t.pq = (const int16_t*)(b + o_pq);
     t.pq2b = (const int16_t*)(b + o_pq2b);
     t.pq2k = (const int16_t*)(b + o_pq2k);
@@ -551,6 +616,54 @@ const double* get_boys_table(int L, cudaStream_t s, int* err)
     }
     g_boys_tabs[key] = d;
     return d;
+}
+
+const int64_t* get_fix_boys_table(int L, cudaStream_t s, int* err)
+{
+    if (L < 0 || L > kFixAuxLmax) {
+        *err = ERI_EINVAL;
+        return nullptr;
+    }
+    std::call_once(g_master_once, build_master);
+    int dev = 0;
+    cudaGetDevice(&dev);
+    std::lock_guard<std::mutex> lk(g_boys_mu);
+    auto key = std::make_pair(dev, 1000 + L);  // beside the FP64 rows of the same order
+    auto it = g_boys_tabs.find(key);
+    if (it != g_boys_tabs.end()) return reinterpret_cast<const int64_t*>(it->second);
+    const int words = fix_boys_words(L);
+    const size_t n = (size_t)kFixBoysRows * words + kFixFarWords;
+    std::vector<int64_t> tab(n, 0);
+    // (long double is software on some hosts: the rows are shared out)
+    const int nt = std::max(1, std::min(16, (int)std::thread::hardware_concurrency()));
+    std::vector<std::thread> pool;
+    auto rows = [&](int t) {
+        for (int j = t; j < kFixBoysRows; j += nt)
+            fix_boys_row(g_master_host.data(), L, j, tab.data() + (size_t)j * words);
+    };
+    for (int t = 1; t < nt; ++t) {
+        try {
+            pool.emplace_back(rows, t);
+        } catch (const std::system_error&) {
+            rows(t);  // no further thread to be had
+        }
+    }
+    rows(0);
+    for (auto& t : pool) t.join();
+    fix_far_constants(L, tab.data() + (size_t)kFixBoysRows * words);
+    double* d = nullptr;
+    if (cudaMalloc(&d, n * 8) != cudaSuccess) {
+        *err = ERI_ENOMEM;
+        return nullptr;
+    }
+    if (cudaMemcpyAsync(d, tab.data(), n * 8, cudaMemcpyHostToDevice, s) != cudaSuccess ||
+        cudaStreamSynchronize(s) != cudaSuccess) {
+        cudaFree(d);
+        *err = ERI_ECUDA;
+        return nullptr;
+    }
+    g_boys_tabs[key] = d;
+    return reinterpret_cast<const int64_t*>(d);
 }
 
 // ---------------------------------------------------------------------------

@@ -17,6 +17,7 @@
 namespace eri {
 
 constexpr int kNT = 256;   // threads per CTA of the tile kernels (plans; most eri_batch tiles)
+constexpr int kNTSlim = 128;  // fixed-point tiles that share an SM with several others
 constexpr int kNTWide = 512;  // eri_batch tiles that fill an SM's shared memory alone
 constexpr int kNACC = 16;  // outputs per thread held in registers
 
@@ -182,6 +183,17 @@ struct FwdArgs {
     int o_Ei;                 // one-quartet tile with E not staged: the bra E products of the current bra primitive, [Tab] (-1: none)
     int o_Er;                 // split blocked ket stage with E not staged: a ring of three ket E rows per warp (-1: none)
     int r_pairs;              // auxiliary integrals in the paired layout (split form, blocked ket stage)
+    int o_fx;                 // fixed-point tile: exponents and flags (fix_scratch_ints)
+    int o_acc;                // fixed-point tile: accumulators [nab][ncd][TQ]
+    int nsm;                  // fixed-point tile: SMs of the device
+    int fx_f;                 // fixed-point tile: coordinates are in units of 2^-fx_f
+    const long long* fx_tab;  // fixed-point tile: Boys rows of order L (eri_fixaux.cuh)
+    const long long* fx_far;  // and constants of T >= 320
+    float fx_c, fx_imu;       // fixed-point tile: 2.42 / mu^2 and 1 / mu of the Hermite unit mu 2^sigma
+    long long fx_rmu;         // and 2^62 / mu
+    const int32_t* bra_ex;    // fixed-point tile: exponents of the bra's E columns [nbra][nab]
+    const int32_t* ket_ex;    // fixed-point tile: exponents of the ket's column norms [nket][ncd]
+    const float* ket_norm;    // fixed-point tile: their 1-norms per Hermite order [nket][ncd][8]
     int64_t ntiles;
     // work-queue mode (plans): one bra pair, consecutive ket pairs
     int mode;                 // 0: list/product batch, 1: ranged (bra rbra, kets rk0..)
@@ -223,7 +235,16 @@ inline void set_tile(FwdArgs& a, const TilePlan& tp)
     a.o_Ei = tp.o_Ei;
     a.o_Er = tp.o_Er;
     a.r_pairs = tp.r_pairs;
+    a.o_fx = tp.o_fx;
+    a.o_acc = tp.o_acc;
 }
+
+// n / d for 0 <= n with n d < 2^32, as one high multiply (d fixed for a while)
+struct FastDiv {
+    unsigned m, one;
+    __device__ __forceinline__ explicit FastDiv(int d) : m(d > 1 ? 0xffffffffu / (unsigned)d + 1u : 0u), one(d > 1 ? 0u : ~0u) {}
+    __device__ __forceinline__ int div(int n) const { return (int)(__umulhi((unsigned)n, m) + ((unsigned)n & one)); }
+};
 
 struct Strided {
     double* p;
@@ -454,8 +475,9 @@ template <int NT>
 static __device__ void contract_index(const double* in, double* out, const double* __restrict__ M, int outer,
                                       int nin, int nout, int inner)
 {
+    const FastDiv d_inner(inner), d_nout(nout);
     for (int item = threadIdx.x; item < outer * nout * inner; item += NT) {
-        const int i = item % inner, r = item / inner, m = r % nout, o = r / nout;
+        const int r = d_inner.div(item), i = item - r * inner, o = d_nout.div(r), m = r - o * nout;
         const double* row = M + m * nin;
         const double* src = in + (size_t)o * nin * inner + i;
         double v = 0.0;
@@ -715,6 +737,180 @@ __device__ __forceinline__ void split_ket_paired(const FwdArgs& a, int TQ, int I
     }
 }
 
+// [0]^(n), n = 0..L, and P - Q of one primitive quartet from the pair scalars.
+__device__ __forceinline__ void aux_base(int L, const double* pb, const double* pk, const double* __restrict__ boys,
+                                         double* base, double& X, double& Y, double& Z)
+{
+    const double zp = pb[PS_P], zq = pk[PS_P];
+    const double rs = rsqrt_fp64(zp + zq);
+    const double rho = zp * zq * (rs * rs);
+    X = pb[PS_PX] - pk[PS_PX];
+    Y = pb[PS_PY] - pk[PS_PY];
+    Z = pb[PS_PZ] - pk[PS_PZ];
+    const double T = rho * fma(X, X, fma(Y, Y, Z * Z));
+    boys_eval(L, T, boys, base);
+    double f = rs;  // 2 pi^(5/2) / (zp zq sqrt(zp+zq)) less the pair factors in E
+    const double m2rho = -2.0 * rho;
+    for (int n = 0; n <= L; ++n) {
+        base[n] *= f;
+        f *= m2rho;
+    }
+}
+
+// Stage A of one primitive quartet: its auxiliary integrals into R, from the
+// pair scalars pb and pk.  The compile-time path for low orders; the general
+// one above them and for the warp-shared recursion of small tiles (coop:
+// every lane of a warp calls with the same arguments).
+__device__ __forceinline__ void aux_item(const ClassTables& ct, const double* pb, const double* pk,
+                                         const double* __restrict__ boys, const RStep* __restrict__ rsteps, Strided R,
+                                         bool coop, int lane)
+{
+    if (!coop && aux_integrals_fixed(ct.L, pb, pk, boys, R)) return;
+    double base[kLtotMax + 1], X, Y, Z;
+    aux_base(ct.L, pb, pk, boys, base, X, Y, Z);
+    if (coop)
+        r_recursion_warp(ct.L, base, X, Y, Z, rsteps, R, lane);
+    else
+        r_recursion(ct.L, base, X, Y, Z, rsteps, R);
+}
+
+// The calling thread's items tid + s NT < n; NS > 0: s < NS, unrolled (the
+// values live in registers indexed by s).
+template <int NT, int NS, typename F>
+__device__ __forceinline__ void for_items(int n, F f)
+{
+    if (NS > 0) {
+#pragma unroll
+        for (int s = 0; s < NS; ++s) {
+            const int item = threadIdx.x + s * NT;
+            if (item < n) f(s, item);
+        }
+    } else {
+        for (int item = threadIdx.x, s = 0; item < n; item += NT, ++s) f(s, item);
+    }
+}
+
+// The end of a tile: the horizontal recursions and the solid-harmonic map
+// where the class has them, then stores or digestion.  acc(s, item): the
+// contracted integral of the thread's s-th item (for_items), items ordered
+// quartet, cd, ab (quartet fastest); the staging regions are dead.
+template <int NT, int NS, typename Acc>
+__device__ __forceinline__ void tile_epilogue(const FwdArgs& a, Acc acc, int64_t q0, int nqt, double* sm,
+                                              const int* s_q, const int64_t* s_qq, double* s_red)
+{
+    const ClassTables& ct = a.ct;
+    const int tid = threadIdx.x, TQ = a.TQ, ncd = ct.ncd, nab = ct.nab;
+    const int nC = TQ * nab * ncd;
+    const int lgTQ = 31 - __clz(TQ);  // TQ is a power of two
+    double esum = 0.0;
+    if (!ct.hrr && ct.sph) {
+        double* buf[2] = {sm, sm + a.o_hB};
+        for_items<NT, NS>(nC, [&](int s, int item) { buf[0][item] = acc(s, item); });
+        __syncthreads();
+        const double* fin = to_solid_harmonics<NT>(a, buf, 0);
+        const FastDiv d_out(ct.ncd_s);
+        for (int item = tid; item < TQ * ct.nab_s * ct.ncd_s; item += NT) {
+            const int q = item & (TQ - 1), r = item >> lgTQ, ab = d_out.div(r), cd = r - ab * ct.ncd_s;
+            if (q < nqt) a.out[out_index(a, a.order ? s_qq[q] : q0 + q, ab, cd)] = fin[item];
+        }
+    } else if (!ct.hrr && (a.Jmat || a.Kmat)) {
+        // the values go to shared memory (the staging regions are dead)
+        for_items<NT, NS>(nC, [&](int s, int item) { sm[item] = acc(s, item); });
+        __syncthreads();
+        if (a.Jmat) digest_coulomb<NT>(a, sm, nqt, s_q, sm + a.o_dj);
+        if (a.Kmat) digest_exchange<NT>(a, sm, nqt, s_q, sm + a.o_dj);
+    } else if (!ct.hrr) {
+        const FastDiv d_ncd(ncd);
+        for_items<NT, NS>(nC, [&](int s, int item) {
+            const int q = item & (TQ - 1), r = item >> lgTQ, ab = d_ncd.div(r), cd = r - ab * ncd;
+            if (q >= nqt) return;
+            if (a.energy)
+                esum = fma(acc(s, item), digest_weight(a, s_q[4 * q], s_q[4 * q + 1], ab, cd), esum);
+            else
+                a.out[out_index(a, a.order ? s_qq[q] : q0 + q, ab, cd)] = acc(s, item);
+        });
+    } else {
+        // horizontal recursions on the contracted (f0|e0), one level at a
+        // time over the whole tile, ping-ponging between two buffers that
+        // alias the dead staging regions: ket levels on every f row
+        // ([f][e][q]), then bra levels on every (cd) column ([f][cd][q])
+        double* hbuf[2] = {sm, sm + a.o_hB};
+        double* s_geo = sm + a.o_geo;  // [q][6]: A-B, C-D
+        for_items<NT, NS>(nC, [&](int s, int item) { hbuf[0][item] = acc(s, item); });
+        for (int q = tid; q < TQ; q += NT) {
+            const int b = s_q[4 * q], k = s_q[4 * q + 1];
+            const double* A = a.centres + 3 * a.shell_atom[a.bra_sh[2 * b]];
+            const double* B = a.centres + 3 * a.shell_atom[a.bra_sh[2 * b + 1]];
+            const double* C = a.centres + 3 * a.shell_atom[a.ket_sh[2 * k]];
+            const double* D = a.centres + 3 * a.shell_atom[a.ket_sh[2 * k + 1]];
+            for (int i = 0; i < 3; ++i) {
+                s_geo[6 * q + i] = A[i] - B[i];
+                s_geo[6 * q + 3 + i] = C[i] - D[i];
+            }
+        }
+        __syncthreads();
+        int g = 0;
+        for (int j = 1; j <= ct.ld; ++j, ++g) {
+            const double* src = hbuf[g & 1];
+            double* dst = hbuf[(g + 1) & 1];
+            const int np = ct.kn[j - 1], nn = ct.kn[j];
+            const int16_t* st = ct.ksteps + 3 * ct.koff[j];
+            const FastDiv d_nn(nn);
+            for (int item = tid; item < TQ * nab * nn; item += NT) {
+                const int q = item & (TQ - 1), r = item >> lgTQ, f = d_nn.div(r), o = r - f * nn;
+                const int16_t* s3 = st + 3 * o;
+                const double* row = src + (size_t)f * np * TQ + q;
+                dst[item] = fma(s_geo[6 * q + 3 + s3[2]], row[s3[1] * TQ], row[s3[0] * TQ]);
+            }
+            __syncthreads();
+        }
+        const int ncf = ct.ncd_f;
+        const FastDiv d_ncf(ncf);
+        for (int j = 1; j <= ct.lb; ++j, ++g) {
+            const double* src = hbuf[g & 1];
+            double* dst = hbuf[(g + 1) & 1];
+            const int16_t* st = ct.bsteps + 3 * ct.boff[j];
+            for (int item = tid; item < TQ * ncf * ct.bn[j]; item += NT) {
+                const int q = item & (TQ - 1), r = item >> lgTQ, o = d_ncf.div(r), cd = r - o * ncf;
+                const int16_t* s3 = st + 3 * o;
+                const double* col = src + (size_t)cd * TQ + q;
+                dst[item] = fma(s_geo[6 * q + s3[2]], col[(size_t)s3[1] * ncf * TQ], col[(size_t)s3[0] * ncf * TQ]);
+            }
+            __syncthreads();
+        }
+        const double* fin = hbuf[g & 1];  // [ab][cd][q]
+        if (ct.sph) {
+            const double* fs = to_solid_harmonics<NT>(a, hbuf, g & 1);
+            const FastDiv d_out(ct.ncd_s);
+            for (int item = tid; item < TQ * ct.nab_s * ct.ncd_s; item += NT) {
+                const int q = item & (TQ - 1), r = item >> lgTQ, ab = d_out.div(r), cd = r - ab * ct.ncd_s;
+                if (q < nqt) a.out[out_index(a, a.order ? s_qq[q] : q0 + q, ab, cd)] = fs[item];
+            }
+        } else if (a.Jmat || a.Kmat) {
+            if (a.Jmat) digest_coulomb<NT>(a, fin, nqt, s_q, sm + a.o_dj);
+            if (a.Kmat) digest_exchange<NT>(a, fin, nqt, s_q, sm + a.o_dj);
+        } else {
+            for (int item = tid; item < TQ * ct.nab_f * ncf; item += NT) {
+                const int q = item & (TQ - 1), r = item >> lgTQ, ab = d_ncf.div(r), cd = r - ab * ncf;
+                if (q >= nqt) continue;
+                if (a.energy)
+                    esum = fma(fin[item], digest_weight(a, s_q[4 * q], s_q[4 * q + 1], ab, cd), esum);
+                else
+                    a.out[out_index(a, a.order ? s_qq[q] : q0 + q, ab, cd)] = fin[item];
+            }
+        }
+    }
+    if (a.energy) {
+        for (int o = 16; o > 0; o >>= 1) esum += __shfl_down_sync(0xffffffffu, esum, o);
+        if ((tid & 31) == 0) atomicAdd(s_red, esum);
+        __syncthreads();
+        if (tid == 0) {
+            atomicAdd(a.energy, *s_red);
+            *s_red = 0.0;
+        }
+    }
+}
+
 // One tile: quartets q0 .. q0+nqt-1 (the class tables are already staged).
 // s_red: one shared double for the digestion sum.
 template <bool SPLIT, int NT = kNT>
@@ -813,30 +1009,7 @@ __device__ void tile_body(const FwdArgs& a, int64_t q0, int nqt, double* sm, dou
             Strided R{sR + (q * IC + ii) * KKr + k, NIs};
             const int e0 = coop ? lane : 0, de = coop ? 32 : 1;
             if (i < s_q[4 * q + 2] && k < s_q[4 * q + 3]) {
-                const double* pb = sPb + (q * KB + i) * PS_N;
-                const double* pk = sPk + (q * KK + k) * PS_N;
-                // the compile-time path for low orders; the general one above them
-                // and for the warp-shared recursion of small tiles
-                if (coop || !aux_integrals_fixed(ct.L, pb, pk, a.boys, R)) {
-                    const double zp = pb[PS_P], zq = pk[PS_P];
-                    const double rs = rsqrt_fp64(zp + zq);
-                    const double rho = zp * zq * (rs * rs);
-                    const double X = pb[PS_PX] - pk[PS_PX], Y = pb[PS_PY] - pk[PS_PY], Z = pb[PS_PZ] - pk[PS_PZ];
-                    const double PQ2 = fma(X, X, fma(Y, Y, Z * Z));
-                    const double T = rho * PQ2;
-                    double base[kLtotMax + 1];
-                    boys_eval(ct.L, T, a.boys, base);
-                    double f = rs;  // 2 pi^(5/2) / (zp zq sqrt(zp+zq)) less the pair factors in E
-                    const double m2rho = -2.0 * rho;
-                    for (int n = 0; n <= ct.L; ++n) {
-                        base[n] *= f;
-                        f *= m2rho;
-                    }
-                    if (coop)
-                        r_recursion_warp(ct.L, base, X, Y, Z, a.rsteps, R, lane);
-                    else
-                        r_recursion(ct.L, base, X, Y, Z, a.rsteps, R);
-                }
+                aux_item(ct, sPb + (q * KB + i) * PS_N, sPk + (q * KK + k) * PS_N, a.boys, a.rsteps, R, coop, lane);
                 if (SPLIT && !a.r_pairs)  // each entry becomes its (hi, lo) float pair, in place
                     for (int e = e0; e < nhl; e += de) {
                         double& slot = R[e];
@@ -1006,128 +1179,8 @@ __device__ void tile_body(const FwdArgs& a, int64_t q0, int nqt, double* sm, dou
             __syncthreads();
         }
     }
-    if (a.acc_regs) {
-        const int nC = TQ * nab * ncd;
-        double esum = 0.0;
-        if (!ct.hrr && ct.sph) {
-            double* buf[2] = {sm, sm + a.o_hB};
-#pragma unroll
-            for (int s = 0; s < kNACC; ++s) {
-                const int item = tid + s * NT;
-                if (item < nC) buf[0][item] = acc[s];
-            }
-            __syncthreads();
-            const double* fin = to_solid_harmonics<NT>(a, buf, 0);
-            for (int item = tid; item < TQ * ct.nab_s * ct.ncd_s; item += NT) {
-                const int q = item % TQ, r = item / TQ, cd = r % ct.ncd_s, ab = r / ct.ncd_s;
-                if (q < nqt) a.out[out_index(a, a.order ? s_qq[q] : q0 + q, ab, cd)] = fin[item];
-            }
-        } else if (!ct.hrr && (a.Jmat || a.Kmat)) {
-            // the values go to shared memory (the staging regions are dead)
-#pragma unroll
-            for (int s = 0; s < kNACC; ++s) {
-                const int item = tid + s * NT;
-                if (item < nC) sm[item] = acc[s];
-            }
-            __syncthreads();
-            if (a.Jmat) digest_coulomb<NT>(a, sm, nqt, s_q, sm + a.o_dj);
-            if (a.Kmat) digest_exchange<NT>(a, sm, nqt, s_q, sm + a.o_dj);
-        } else if (!ct.hrr) {
-#pragma unroll
-            for (int s = 0; s < kNACC; ++s) {
-                const int item = tid + s * NT;
-                if (item < nC) {
-                    const int q = item % TQ, r = item / TQ, cd = r % ncd, ab = r / ncd;
-                    if (q < nqt) {
-                        if (a.energy)
-                            esum = fma(acc[s], digest_weight(a, s_q[4 * q], s_q[4 * q + 1], ab, cd), esum);
-                        else
-                            a.out[out_index(a, a.order ? s_qq[q] : q0 + q, ab, cd)] = acc[s];
-                    }
-                }
-            }
-        } else {
-            // horizontal recursions on the contracted (f0|e0), one level at a
-            // time over the whole tile, ping-ponging between two buffers that
-            // alias the dead staging regions: ket levels on every f row
-            // ([f][e][q]), then bra levels on every (cd) column ([f][cd][q])
-            double* hbuf[2] = {sm, sm + a.o_hB};
-            double* s_geo = sm + a.o_geo;  // [q][6]: A-B, C-D
-#pragma unroll
-            for (int s = 0; s < kNACC; ++s) {
-                const int item = tid + s * NT;
-                if (item < nC) hbuf[0][item] = acc[s];
-            }
-            for (int q = tid; q < TQ; q += NT) {
-                const int b = s_q[4 * q], k = s_q[4 * q + 1];
-                const double* A = a.centres + 3 * a.shell_atom[a.bra_sh[2 * b]];
-                const double* B = a.centres + 3 * a.shell_atom[a.bra_sh[2 * b + 1]];
-                const double* C = a.centres + 3 * a.shell_atom[a.ket_sh[2 * k]];
-                const double* D = a.centres + 3 * a.shell_atom[a.ket_sh[2 * k + 1]];
-                for (int i = 0; i < 3; ++i) {
-                    s_geo[6 * q + i] = A[i] - B[i];
-                    s_geo[6 * q + 3 + i] = C[i] - D[i];
-                }
-            }
-            __syncthreads();
-            int g = 0;
-            for (int j = 1; j <= ct.ld; ++j, ++g) {
-                const double* src = hbuf[g & 1];
-                double* dst = hbuf[(g + 1) & 1];
-                const int np = ct.kn[j - 1], nn = ct.kn[j];
-                const int16_t* st = ct.ksteps + 3 * ct.koff[j];
-                for (int item = tid; item < TQ * nab * nn; item += NT) {
-                    const int q = item % TQ, r = item / TQ, o = r % nn, f = r / nn;
-                    const int16_t* s3 = st + 3 * o;
-                    const double* row = src + (size_t)f * np * TQ + q;
-                    dst[item] = fma(s_geo[6 * q + 3 + s3[2]], row[s3[1] * TQ], row[s3[0] * TQ]);
-                }
-                __syncthreads();
-            }
-            const int ncf = ct.ncd_f;
-            for (int j = 1; j <= ct.lb; ++j, ++g) {
-                const double* src = hbuf[g & 1];
-                double* dst = hbuf[(g + 1) & 1];
-                const int16_t* st = ct.bsteps + 3 * ct.boff[j];
-                for (int item = tid; item < TQ * ncf * ct.bn[j]; item += NT) {
-                    const int q = item % TQ, r = item / TQ, cd = r % ncf, o = r / ncf;
-                    const int16_t* s3 = st + 3 * o;
-                    const double* col = src + (size_t)cd * TQ + q;
-                    dst[item] = fma(s_geo[6 * q + s3[2]], col[(size_t)s3[1] * ncf * TQ], col[(size_t)s3[0] * ncf * TQ]);
-                }
-                __syncthreads();
-            }
-            const double* fin = hbuf[g & 1];  // [ab][cd][q]
-            if (ct.sph) {
-                const double* fs = to_solid_harmonics<NT>(a, hbuf, g & 1);
-                for (int item = tid; item < TQ * ct.nab_s * ct.ncd_s; item += NT) {
-                    const int q = item % TQ, r = item / TQ, cd = r % ct.ncd_s, ab = r / ct.ncd_s;
-                    if (q < nqt) a.out[out_index(a, a.order ? s_qq[q] : q0 + q, ab, cd)] = fs[item];
-                }
-            } else if (a.Jmat || a.Kmat) {
-                if (a.Jmat) digest_coulomb<NT>(a, fin, nqt, s_q, sm + a.o_dj);
-                if (a.Kmat) digest_exchange<NT>(a, fin, nqt, s_q, sm + a.o_dj);
-            } else {
-                for (int item = tid; item < TQ * ct.nab_f * ncf; item += NT) {
-                    const int q = item % TQ, r = item / TQ, cd = r % ncf, ab = r / ncf;
-                    if (q >= nqt) continue;
-                    if (a.energy)
-                        esum = fma(fin[item], digest_weight(a, s_q[4 * q], s_q[4 * q + 1], ab, cd), esum);
-                    else
-                        a.out[out_index(a, a.order ? s_qq[q] : q0 + q, ab, cd)] = fin[item];
-                }
-            }
-        }
-        if (a.energy) {
-            for (int o = 16; o > 0; o >>= 1) esum += __shfl_down_sync(0xffffffffu, esum, o);
-            if ((tid & 31) == 0) atomicAdd(s_red, esum);
-            __syncthreads();
-            if (tid == 0) {
-                atomicAdd(a.energy, *s_red);
-                *s_red = 0.0;
-            }
-        }
-    }
+    if (a.acc_regs)
+        tile_epilogue<NT, kNACC>(a, [&](int s, int) { return acc[s]; }, q0, nqt, sm, s_q, s_qq, s_red);
 }
 
 // NT = kNT: two CTAs per SM (128 registers a thread); kNTWide: one.

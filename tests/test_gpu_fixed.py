@@ -1,0 +1,106 @@
+"""The fixed-point tile of eri_batch (contracted 4-centre classes in large
+batches) against the oracle: ket primitive counts on both sides of the folds
+and pairs of its sums, mixed contraction degrees, every order of the auxiliary
+integrals it takes, both list forms and the solid-harmonic output."""
+import numpy as np
+import pytest
+import torch
+
+import paper_2506_12501_gb300 as eri
+import synth
+from gpu_helpers import assert_close, nc, oracle_blocks, to_device
+
+pytestmark = pytest.mark.gpu
+
+# class, primitives per shell: K_ket = 4 (even), 9 (odd), 16 (past one fold), 25 and 36 for s shells (several
+# folds); L = 1..8; a component-pair list of one column, pairs and single columns
+CASES = [((1, 0, 0, 0), 2), ((0, 1, 1, 0), 3), ((1, 1, 1, 0), 4), ((1, 1, 1, 1), 3), ((2, 1, 1, 1), 3),
+         ((2, 1, 2, 1), 2), ((2, 2, 2, 1), 2), ((2, 2, 2, 2), 2), ((1, 0, 1, 0), 5), ((0, 0, 1, 0), 6), ((3, 1, 2, 0), 2)]
+
+
+def _sample_error(got, ref):
+    """Relative 2-norm error; the oracle's double build and the FP64 tile agree to a few 1e-15, times the
+    recursion forms' magnification (below 10 on these pairs)."""
+    return np.linalg.norm(got - ref) / np.linalg.norm(ref)
+
+
+@pytest.mark.parametrize("cls,K", CASES)
+def test_fixed_tile_against_oracle(cls, K):
+    nq = max(2003, 150000 // K ** 4 + 7)  # odd: the last tile is ragged
+    basis, pools = synth.class_sweep_pools(seed=3, lmax=max(cls), pool=64, K=K, cube=4.0)
+    bra, ket, q = synth.class_sweep_batch(pools, cls, seed=4, npairs=50, nq=nq)
+    b, k, qq = to_device(bra, ket, q)
+    db = eri.DeviceBasis(basis)
+    for form in (0, 1, 2, 3):
+        eri.eri_set_forms(1 << form)
+        try:
+            out = eri.eri_batch(cls, db, b, k, qq).cpu().numpy().reshape(-1, nq).T
+        finally:
+            eri.eri_set_forms(0)
+        pick = np.r_[0:12, nq - 12:nq]
+        ref = oracle_blocks(cls, basis, bra, ket, q[pick])
+        assert_close(out[pick], ref, what=f"{cls} K={K} form {form}")
+        assert _sample_error(out[pick], ref) < 2e-14
+
+
+def test_fixed_tile_mixed_degrees_product_form_and_sph():
+    cls = (1, 0, 1, 1)
+    rng = np.random.default_rng(5)
+    shells, centres = [], rng.uniform(0, 3.0, (90, 3))
+    for i in range(90):
+        l, K = (1, 0)[i % 2], (1, 2, 3, 5)[i % 4]
+        z = 0.3 * 2.0 ** np.arange(K)
+        shells.append((i, l, list(z), list(rng.uniform(0.5, 1, K) * synth.norm_coef(z, l))))
+    basis = synth.basis_from_shells(centres, shells)
+    p, s = np.arange(0, 90, 2), np.arange(1, 90, 2)
+    bra = np.stack([rng.choice(p, 61), rng.choice(s, 61)], 1).astype(np.int32)
+    ket = np.stack([rng.choice(p, 53), rng.choice(p, 53)], 1).astype(np.int32)
+    b, k, _ = to_device(bra, ket)
+    db = eri.DeviceBasis(basis)
+    nab, ncd = 3, 9
+    out = eri.eri_batch(cls, db, b, k).cpu().numpy().reshape(53, ncd, nab, 61)
+    q = np.array([(i, j) for i in range(0, 61, 7) for j in range(0, 53, 6)])
+    ref = oracle_blocks(cls, basis, bra, ket, q).reshape(len(q), nab, ncd)
+    got = np.stack([out[j, :, :, i].T for i, j in q])
+    assert_close(got, ref, what="product form, mixed degrees")
+    sph = eri.eri_batch_sph(cls, db, b, k).cpu().numpy().reshape(53, ncd, nab, 61)
+    # p functions in solid harmonics: m = -1, 0, 1 are y, z, x
+    order = np.array([1, 2, 0])
+    cd = (order[:, None] * 3 + order[None, :]).reshape(-1)
+    assert_close(np.stack([sph[j, :, :, i].T for i, j in q]), ref[:, order][:, :, cd], what="solid harmonics")
+
+
+def test_fixed_tile_far_and_coincident_centres():
+    """Boys arguments of every range: coincident centres (T = 0) to far apart (T of thousands)."""
+    cls, K, nq = (1, 1, 1, 0), 3, 4000
+    rng = np.random.default_rng(6)
+    centres = np.concatenate([np.zeros((20, 3)), rng.uniform(-1, 1, (20, 3)), rng.uniform(-60, 60, (20, 3))])
+    shells = []
+    for l in (0, 1):
+        for i in range(60):
+            z = 0.2 * 3.0 ** np.arange(K)
+            shells.append((i, l, list(z), list(rng.uniform(0.5, 1, K) * synth.norm_coef(z, l))))
+    basis = synth.basis_from_shells(centres, shells)
+    near = np.array([(60 + i, 60 + j) for i in range(60) for j in (i, (i + 1) % 20)], np.int32)
+    ket = np.array([(60 + i, j) for i in range(60) for j in (i, (i + 3) % 20)], np.int32)
+    q = np.stack([rng.integers(0, len(near), nq), rng.integers(0, len(ket), nq)], 1)
+    b, k, qq = to_device(near, ket, q)
+    out = eri.eri_batch(cls, eri.DeviceBasis(basis), b, k, qq).cpu().numpy().reshape(-1, nq).T
+    ref = oracle_blocks(cls, basis, near, ket, q[:400])
+    assert_close(out[:400], ref, what="centres of every distance")
+
+
+def test_wide_exponents_and_non_finite_primitives_keep_the_fp64_tile():
+    """Pairs whose exponents spread too far, and primitives out of the fixed-point range, give what they gave."""
+    cls, nq = (1, 1, 1, 1), 4000
+    basis, pools = synth.class_sweep_pools(seed=8, lmax=1, pool=32, K=2, cube=3.0,
+                                           exps_fn=lambda rng, K: np.array([0.05, 900.0]))
+    bra, ket, q = synth.class_sweep_batch(pools, cls, seed=9, npairs=40, nq=nq)
+    b, k, qq = to_device(bra, ket, q)
+    out = eri.eri_batch(cls, eri.DeviceBasis(basis), b, k, qq).cpu().numpy().reshape(-1, nq).T
+    assert_close(out[:60], oracle_blocks(cls, basis, bra, ket, q[:60]), what="wide exponents")
+    basis, pools = synth.class_sweep_pools(seed=8, lmax=1, pool=32, K=3, cube=3.0)
+    basis.coefs[basis.shell_off[bra[0, 0]]] = np.nan
+    out = eri.eri_batch(cls, eri.DeviceBasis(basis), b, k, qq).cpu().numpy().reshape(-1, nq).T
+    bad = np.any(bra[q[:, 0]] == bra[0, 0], axis=1) | np.any(ket[q[:, 1]] == bra[0, 0], axis=1)
+    assert bad.any() and np.isnan(out[bad]).all() and np.isfinite(out[~bad]).all()
