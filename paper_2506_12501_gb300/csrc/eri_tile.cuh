@@ -737,43 +737,6 @@ __device__ __forceinline__ void split_ket_paired(const FwdArgs& a, int TQ, int I
     }
 }
 
-// [0]^(n), n = 0..L, and P - Q of one primitive quartet from the pair scalars.
-__device__ __forceinline__ void aux_base(int L, const double* pb, const double* pk, const double* __restrict__ boys,
-                                         double* base, double& X, double& Y, double& Z)
-{
-    const double zp = pb[PS_P], zq = pk[PS_P];
-    const double rs = rsqrt_fp64(zp + zq);
-    const double rho = zp * zq * (rs * rs);
-    X = pb[PS_PX] - pk[PS_PX];
-    Y = pb[PS_PY] - pk[PS_PY];
-    Z = pb[PS_PZ] - pk[PS_PZ];
-    const double T = rho * fma(X, X, fma(Y, Y, Z * Z));
-    boys_eval(L, T, boys, base);
-    double f = rs;  // 2 pi^(5/2) / (zp zq sqrt(zp+zq)) less the pair factors in E
-    const double m2rho = -2.0 * rho;
-    for (int n = 0; n <= L; ++n) {
-        base[n] *= f;
-        f *= m2rho;
-    }
-}
-
-// Stage A of one primitive quartet: its auxiliary integrals into R, from the
-// pair scalars pb and pk.  The compile-time path for low orders; the general
-// one above them and for the warp-shared recursion of small tiles (coop:
-// every lane of a warp calls with the same arguments).
-__device__ __forceinline__ void aux_item(const ClassTables& ct, const double* pb, const double* pk,
-                                         const double* __restrict__ boys, const RStep* __restrict__ rsteps, Strided R,
-                                         bool coop, int lane)
-{
-    if (!coop && aux_integrals_fixed(ct.L, pb, pk, boys, R)) return;
-    double base[kLtotMax + 1], X, Y, Z;
-    aux_base(ct.L, pb, pk, boys, base, X, Y, Z);
-    if (coop)
-        r_recursion_warp(ct.L, base, X, Y, Z, rsteps, R, lane);
-    else
-        r_recursion(ct.L, base, X, Y, Z, rsteps, R);
-}
-
 // The calling thread's items tid + s NT < n; NS > 0: s < NS, unrolled (the
 // values live in registers indexed by s).
 template <int NT, int NS, typename F>
@@ -1009,7 +972,30 @@ __device__ void tile_body(const FwdArgs& a, int64_t q0, int nqt, double* sm, dou
             Strided R{sR + (q * IC + ii) * KKr + k, NIs};
             const int e0 = coop ? lane : 0, de = coop ? 32 : 1;
             if (i < s_q[4 * q + 2] && k < s_q[4 * q + 3]) {
-                aux_item(ct, sPb + (q * KB + i) * PS_N, sPk + (q * KK + k) * PS_N, a.boys, a.rsteps, R, coop, lane);
+                const double* pb = sPb + (q * KB + i) * PS_N;
+                const double* pk = sPk + (q * KK + k) * PS_N;
+                // the compile-time path for low orders; the general one above them
+                // and for the warp-shared recursion of small tiles
+                if (coop || !aux_integrals_fixed(ct.L, pb, pk, a.boys, R)) {
+                    const double zp = pb[PS_P], zq = pk[PS_P];
+                    const double rs = rsqrt_fp64(zp + zq);
+                    const double rho = zp * zq * (rs * rs);
+                    const double X = pb[PS_PX] - pk[PS_PX], Y = pb[PS_PY] - pk[PS_PY], Z = pb[PS_PZ] - pk[PS_PZ];
+                    const double PQ2 = fma(X, X, fma(Y, Y, Z * Z));
+                    const double T = rho * PQ2;
+                    double base[kLtotMax + 1];
+                    boys_eval(ct.L, T, a.boys, base);
+                    double f = rs;  // 2 pi^(5/2) / (zp zq sqrt(zp+zq)) less the pair factors in E
+                    const double m2rho = -2.0 * rho;
+                    for (int n = 0; n <= ct.L; ++n) {
+                        base[n] *= f;
+                        f *= m2rho;
+                    }
+                    if (coop)
+                        r_recursion_warp(ct.L, base, X, Y, Z, a.rsteps, R, lane);
+                    else
+                        r_recursion(ct.L, base, X, Y, Z, a.rsteps, R);
+                }
                 if (SPLIT && !a.r_pairs)  // each entry becomes its (hi, lo) float pair, in place
                     for (int e = e0; e < nhl; e += de) {
                         double& slot = R[e];
