@@ -236,38 +236,50 @@ struct PairArgs {
     double mu;              // and mu^(Hermite order) (eri_fixed.cuh)
 };
 
+constexpr int kPairThreads = 128;
+constexpr int64_t kPairWarpSlots = 8192;  // at most this many slots take a warp each (twice as many for 1000 terms)
 constexpr int kEax = (kLmax + 3) * (kLmax + 3) * (2 * kLmax + 5);  // per-axis E table bound (adjoint shifts)
 constexpr int kEfw = (kLmax + 1) * (kLmax + 1) * (2 * kLmax + 1);  // without the shifts (also the HRR form's)
 
 // RAISED: the adjoint's tables (a.ax != NULL): the per-axis E tables with
 // both indices raised by 2, one thread per (slot, axis).  The adjoint reads
 // no E products of that side, so none are formed.  Otherwise one thread per
-// slot forms the three tables and the E products of the class's terms.
-template <bool RAISED>
-__global__ void pair_kernel_t(PairArgs a)
+// slot forms the three tables and the E products of the class's terms; WARP: a
+// warp does, lanes 0..2 a table each (in shared memory), then every lane its
+// share of the products.  A batch of few slots with long term lists leaves one
+// thread per slot latency bound on 16 of the 152 SMs: 2048 uncontracted (ff|
+// pairs 917 us, of a batch of 7.2 ms.
+template <bool RAISED, bool WARP>
+__global__ void __launch_bounds__(kPairThreads) pair_kernel_t(PairArgs a)
 {
-    constexpr int NX = RAISED ? 1 : 3;  // axes per thread
-    const int64_t total = a.npairs * a.KS * (RAISED ? 3 : 1);
+    static_assert(!(RAISED && WARP), "the raised tables take a thread per axis");
+    constexpr int NX = RAISED || WARP ? 1 : 3;  // axes per thread
+    constexpr int PER = RAISED ? 3 : (WARP ? 32 : 1);  // threads per slot
+    __shared__ double s_E[WARP ? kPairThreads / 32 : 1][3][WARP ? kEfw : 1];
+    const int lane = WARP ? threadIdx.x & 31 : 0;
+    const int64_t total = a.npairs * a.KS * PER;
     for (int64_t gg = blockIdx.x * (int64_t)blockDim.x + threadIdx.x; gg < total;
          gg += (int64_t)gridDim.x * blockDim.x) {
-        const int64_t g = RAISED ? gg / 3 : gg;       // the slot
+        const int64_t g = gg / PER;                     // the slot
         const int x0 = RAISED ? (int)(gg - g * 3) : 0;  // its first axis
+        if (WARP) __syncwarp();                         // the last slot's tables are read
         const int64_t j = g / a.KS;
         const int s = (int)(g - j * a.KS);
         // s2 = -1: the unit function (exponent 0, coefficient 1) of a 3-centre
         // bra; its centre is immaterial and taken as the first shell's
         const int s1 = a.pairs[2 * j], s2 = a.pairs[2 * j + 1];
         const int K1 = a.shell_K[s1], K2 = s2 < 0 ? 1 : a.shell_K[s2];
-        if (s == 0 && x0 == 0) a.kprim[j] = K1 * K2;
+        if (s == 0 && x0 == 0 && lane == 0) a.kprim[j] = K1 * K2;
         if (s >= K1 * K2) {  // padding slot: finite zeros, never contributes
             if (RAISED) {
                 for (int q = 0; q < a.eax; ++q) a.ax[((size_t)g * 3 + x0) * a.eax + q] = 0.0;
                 if (x0 != 0) continue;
                 a.zz[2 * g] = a.zz[2 * g + 1] = 1.0;
             } else {
-                for (int t = 0; t < a.T; ++t)
+                for (int t = lane; t < a.T; t += WARP ? 32 : 1)
                     a.E[a.fixed && !a.ket ? (size_t)g * a.T + t : ((size_t)j * a.T + t) * a.KS + s] = 0.0;
             }
+            if (lane != 0) continue;
             if (!RAISED && a.fixed) {
                 reinterpret_cast<FixPrim*>(a.ps)[g] = FixPrim{{0, 0, 0}, 1LL << 61, 1, 1.0f};
                 continue;
@@ -295,14 +307,14 @@ __global__ void pair_kernel_t(PairArgs a)
                 }
         }
         const double inv2p = 0.5 * invp;
-        double PA[3], PB[3], P[3], AB2 = 0.0;
+        double P[3], AB2 = 0.0;
         for (int x = 0; x < 3; ++x) {
             P[x] = (z1 * A[x] + z2 * B[x]) * invp;
-            PA[x] = P[x] - A[x];
-            PB[x] = P[x] - B[x];
             const double d = A[x] - B[x];
             AB2 = fma(d, d, AB2);
         }
+        auto PA = [&](int x) { return (x == 0 ? P[0] : (x == 1 ? P[1] : P[2])) - A[x]; };
+        auto PB = [&](int x) { return (x == 0 ? P[0] : (x == 1 ? P[1] : P[2])) - B[x]; };
         // K_AB c_1 c_2 carried by the x-axis bootstrap E_00^0 (Eq. E2-000),
         // 1 on y and z: the products E^x E^y E^z are unchanged.  So is the
         // pair's factor of the Eq. 0m prefactor, 2 pi^(5/2) / zeta_p on the
@@ -316,18 +328,20 @@ __global__ void pair_kernel_t(PairArgs a)
         // horizontal-recursion form needs E_{i,0} for i <= l1 + l2
         const int m1 = a.hrr ? a.l1 + a.l2 : a.l1 + ext, m2 = a.hrr ? 0 : a.l2 + ext;
         const int L12 = a.l1 + a.l2, n2 = m2 + 1, nt = m1 + m2 + 1;
-        double E[NX][RAISED ? kEax : kEfw];
+        double El[WARP ? 1 : NX][WARP ? 1 : (RAISED ? kEax : kEfw)];
         for (int xi = 0; xi < NX; ++xi) {
-            const int x = x0 + xi;
-            double* Ex = E[xi];
+            const int x = WARP ? lane : x0 + xi;
+            if (WARP && x >= 3) break;
+            double* Ex = WARP ? s_E[threadIdx.x >> 5][x] : El[xi];
             for (int q = 0; q < (m1 + 1) * n2 * nt; ++q) Ex[q] = 0.0;
             Ex[0] = x == 0 ? e00x : 1.0;
+            const double pa = PA(x), pb = PB(x);
             // raise the first index at j = 0 (Eq. E2rr1)
             for (int i = 0; i < m1; ++i)
                 for (int t = 0; t <= i + 1; ++t) {
                     double v = 0.0;
                     if (t >= 1) v = inv2p * Ex[(i * n2) * nt + t - 1];
-                    if (t <= i) v = fma(PA[x], Ex[(i * n2) * nt + t], v);
+                    if (t <= i) v = fma(pa, Ex[(i * n2) * nt + t], v);
                     if (t + 1 <= i) v = fma((double)(float)(t + 1), Ex[(i * n2) * nt + t + 1], v);
                     Ex[((i + 1) * n2) * nt + t] = v;
                 }
@@ -338,14 +352,14 @@ __global__ void pair_kernel_t(PairArgs a)
                         const int b0 = (i * n2 + jj) * nt;
                         double v = 0.0;
                         if (t >= 1) v = inv2p * Ex[b0 + t - 1];
-                        if (t <= i + jj) v = fma(PB[x], Ex[b0 + t], v);
+                        if (t <= i + jj) v = fma(pb, Ex[b0 + t], v);
                         if (t + 1 <= i + jj) v = fma((double)(float)(t + 1), Ex[b0 + t + 1], v);
                         Ex[(i * n2 + jj + 1) * nt + t] = v;
                     }
         }
         if (RAISED) {
             double* o = a.ax + ((size_t)g * 3 + x0) * a.eax;
-            for (int q = 0; q < (m1 + 1) * n2 * nt; ++q) o[q] = E[0][q];
+            for (int q = 0; q < (m1 + 1) * n2 * nt; ++q) o[q] = El[0][q];
             if (x0 != 0) continue;
             a.zz[2 * g] = z1;
             a.zz[2 * g + 1] = z2;
@@ -354,7 +368,11 @@ __global__ void pair_kernel_t(PairArgs a)
             const size_t es = a.fixed && !a.ket ? 1 : a.KS;
             double* Eout = a.E + (a.fixed && !a.ket ? ((size_t)j * a.KS + so) * a.T : (size_t)j * a.T * a.KS + so);
             const int ntc = L12 + 1, n2c = a.hrr ? 1 : a.l2 + 1;  // dims the class-table indices use
-            for (int t = 0; t < a.T; ++t) {
+            const double* T0 = WARP ? s_E[threadIdx.x >> 5][0] : El[0];
+            const double* T1 = WARP ? s_E[threadIdx.x >> 5][1] : El[NX > 1 ? 1 : 0];
+            const double* T2 = WARP ? s_E[threadIdx.x >> 5][2] : El[NX > 2 ? 2 : 0];
+            if (WARP) __syncwarp();
+            for (int t = lane; t < a.T; t += WARP ? 32 : 1) {
                 int idx[3], lq = 0;
                 for (int x = 0; x < 3; ++x) {
                     const int f = a.fac[3 * t + x];
@@ -362,7 +380,7 @@ __global__ void pair_kernel_t(PairArgs a)
                     idx[x] = (aa * n2 + bb) * nt + tt;
                     lq += tt;
                 }
-                double v = E[0][idx[0]] * E[NX > 1 ? 1 : 0][idx[1]] * E[NX > 2 ? 2 : 0][idx[2]];
+                double v = T0[idx[0]] * T1[idx[1]] * T2[idx[2]];
                 if (a.scale) v *= a.scale[t];
                 if (a.ket && (lq & 1)) v = -v;
                 if (a.fixed)
@@ -373,6 +391,7 @@ __global__ void pair_kernel_t(PairArgs a)
                     Eout[t * es] = v;
             }
         }
+        if (lane != 0) continue;
         if (!RAISED && a.fixed) {
             FixPrim f;
             for (int x = 0; x < 3; ++x) f.x[x] = fix_coordinate(P[x], a.fx_f);
@@ -395,10 +414,19 @@ __global__ void pair_kernel_t(PairArgs a)
 // takes three per slot
 static void launch_pair(const PairArgs& p, int grid, cudaStream_t st)
 {
+    // A warp per slot where the slots are few for one thread each (time in us of
+    // one thread | one warp per slot): 1000 slots of (pp| 26 | 12, 2048 of (dd|
+    // 93 | 36, 9216 of (dd| 94 | 87, 18432 of (dp| 57 | 149, of (dd| 94 | 164;
+    // longest lists: 2048 of (ff| 917 | 92, 9216 of (ff| 1036 | 460.  Lists of fewer
+    // than 16 terms leave most lanes idle.
+    const int64_t slots = p.npairs * p.KS;
     if (p.ax)
-        pair_kernel_t<true><<<(int)std::min<int64_t>(3LL * grid, 24LL * sm_count()), 128, 0, st>>>(p);
+        pair_kernel_t<true, false><<<(int)std::min<int64_t>(3LL * grid, 24LL * sm_count()), kPairThreads, 0, st>>>(p);
+    else if (p.T >= 16 && slots <= (p.T >= 1000 ? 2 : 1) * kPairWarpSlots)
+        pair_kernel_t<false, true><<<(int)std::max<int64_t>(1, std::min<int64_t>((32 * slots + kPairThreads - 1) / kPairThreads, 16LL * sm_count())),
+                                     kPairThreads, 0, st>>>(p);
     else
-        pair_kernel_t<false><<<grid, 128, 0, st>>>(p);
+        pair_kernel_t<false, false><<<grid, kPairThreads, 0, st>>>(p);
 }
 
 static const auto fwd_kernel = fwd_kernel_t<false, kNT>;
