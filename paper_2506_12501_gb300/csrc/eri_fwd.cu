@@ -700,6 +700,48 @@ bool plan_tiles(const ClassTables& ct, int KB, int KK, int64_t nq, TilePlan* bes
     return found;
 }
 
+// FP64 tile of a batch too small to be timed: plan_tiles fills one CTA's stages,
+// which leaves a small batch's quartets on a few SMs (1000 (pp|pp), K = 1: 32 CTAs).
+// Here the least modelled time of the whole batch, in clocks: every stage's
+// warps on the busiest SM over its four FP64 pipes, 68 clocks an instruction, so
+// a tile of few quartets costs nothing until four warps queue; and the latency of
+// staging and barriers, once per wave of resident tiles.  *best (the shape of
+// plan_tiles) stays unless another is modelled 10 % faster.  Measured per call, us:
+// (pp|pp) K = 1, 50 / 1000 / 12000 quartets 140 / 145 / 211 -> 63 / 66 / 152; (ps|ps)
+// K = 3, 50 / 1000 quartets 208 / 233 -> 77 / 89; (dd|dd) K = 3, 50 / 1000 quartets
+// 1305 / 2377 -> 379 / 2140 (with the faster pair tables and checking pass).
+static void plan_small_tile(const ClassTables& ct, int KB, int KK, int64_t nq, TilePlan* best)
+{
+    auto warps = [](double items) { return std::ceil(items / 32); };
+    const int L = ct.L;
+    const double base = 45.0 + 3.0 * L, steps = (L + 1.0) * (L + 2) * (L + 3) * (L + 4) / 24;
+    auto model = [&](const TilePlan& tp) {
+        const int64_t tiles = (nq + tp.TQ - 1) / tp.TQ, per_sm = (tiles + sm_count() - 1) / sm_count();
+        const int64_t res = std::min<int64_t>(per_sm, one_cta_per_sm(tp.bytes) ? 1 : 2);
+        const double nA = (double)tp.TQ * tp.IC * KK;  // below 64 items a warp takes each (stage A)
+        auto pipe = [&](double w, double instr) { return std::ceil(res * w / 4) * instr * 68; };
+        const double a = nA < 64 ? pipe(nA, base + steps / 16 + 2 * L) : pipe(warps(nA), base + steps);
+        const double b = pipe(warps((double)tp.TQ * (ct.nhb - ct.pb0) * ct.ncd), (double)KK * ct.Tcd / ct.ncd);
+        const double c = pipe(warps((double)tp.TQ * ct.nab * ct.ncd), (double)ct.Tab / ct.nab);
+        const int chunks = (KB + tp.IC - 1) / tp.IC;
+        return (double)((per_sm + res - 1) / res) * (5000 + chunks * (800 + a) + KB * (1000 + b + c));
+    };
+    double best_time = 0.9 * model(*best);
+    for (int TQ = 1; TQ <= 128 && (TQ == 1 || TQ < 2 * nq); TQ *= 2) {
+        if (TQ > 1 && TQ * ct.nab * ct.ncd > kNT * kNACC) break;
+        for (int IC = KB, next; IC >= 1; IC = next) {  // KB, half of it, 1
+            next = IC == 1 ? 0 : (IC == KB && KB > 2 ? (KB + 1) / 2 : 1);
+            TilePlan tp;
+            if (!tile_layout(ct, KB, KK, TQ, IC, best->e_smem, &tp, XF_FP64)) continue;
+            const double t = model(tp);
+            if (t < best_time) {
+                best_time = t;
+                *best = tp;
+            }
+        }
+    }
+}
+
 static int dev_err_to_code(int e)
 {
     switch (e) {
@@ -1356,6 +1398,7 @@ static int forward_args(const eri_basis_t* basis, const int32_t* bra_pairs, int6
     const RStep* rs = get_rsteps(st, &err);
     if (!rs) return err;
     if (!plan_tiles(*ct, KB, KK, nqq, tp, 0, split)) return ERI_EINVAL;
+    if (split == XF_FP64 && nqq < kTuneMinQuartets) plan_small_tile(*ct, KB, KK, nqq, tp);
     *a = FwdArgs{};
     if (split == XF_FIXED) {
         const int64_t* fx = get_fix_boys_table(ct->L, st, &err);
