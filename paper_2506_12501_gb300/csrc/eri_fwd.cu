@@ -59,7 +59,7 @@ struct PrepassArgs {
     const int32_t* shell_atom;
     const int32_t* shell_off;
     const double* exps;
-    int* kmin;   // optional [2]: the smallest primitive-pair count K1 K2 over bra (ket) pairs
+    int* kmin;   // optional [2]: INT_MAX less the smallest primitive-pair count K1 K2 over bra (ket) pairs
     // optional [6]: the largest zeta_max / zeta_min of a bra (ket) pair (float
     // bits), 1 if a primitive lies outside the fixed-point tile's range, the
     // largest |coordinate| and the largest zeta of a bra (ket) pair (float bits)
@@ -128,20 +128,31 @@ __device__ float pair_recursion_risk(const PrepassArgs& a, int s1, int s2, int l
 
 __device__ __forceinline__ void set_err(int* p, int code) { atomicCAS(p, 0, code); }
 
+// The largest of a warp's v into *p (0 or more; floats by their bits): the pairs
+// of a batch all meet in a few words, whose atomics took most of this kernel.
+__device__ __forceinline__ void warp_max_into(int* p, int v)
+{
+    v = __reduce_max_sync(0xffffffffu, v);
+    if ((threadIdx.x & 31) == 0 && v > 0) atomicMax(p, v);
+}
+
 __global__ void prepass_kernel(PrepassArgs a)
 {
     const int64_t n = max(max(a.nbra, a.nket), a.nq);
-    int kmin[2] = {0x7fffffff, 0x7fffffff};  // this thread's smallest pair counts, reduced per warp at the end
+    // this thread's largest values, reduced per warp at the end
+    int kmax[4] = {0, 0, 0, 0}, kmin[2] = {0, 0}, risk[2] = {0, 0}, ratio[2] = {0, 0}, zeta[2] = {0, 0}, coord = 0;
     for (int64_t i = blockIdx.x * (int64_t)blockDim.x + threadIdx.x; i < n; i += (int64_t)gridDim.x * blockDim.x) {
+#pragma unroll
         for (int side = 0; side < 2; ++side) {
             const int32_t* pr = side == 0 ? a.bra : a.ket;
             const int64_t np = side == 0 ? a.nbra : a.nket;
             if (i >= np) continue;
+#pragma unroll
             for (int c = 0; c < 2; ++c) {
                 const int32_t s = pr[2 * i + c];
                 if (a.unit_b && side == 0 && c == 1) {
                     if (s != -1) set_err(&a.info[4], DEV_EINDEX);
-                    atomicMax(&a.info[1], 1);
+                    kmax[1] = 1;
                     continue;
                 }
                 if (s < 0 || s >= a.nshell) {
@@ -154,13 +165,13 @@ __global__ void prepass_kernel(PrepassArgs a)
                     set_err(&a.info[4], DEV_EK);
                     continue;
                 }
-                atomicMax(&a.info[2 * side + c], K);
+                kmax[2 * side + c] = max(kmax[2 * side + c], K);
             }
             if (a.kmin) {
                 const int s1 = pr[2 * i], s2 = pr[2 * i + 1];
                 const bool unit = a.unit_b && side == 0;
                 if (s1 >= 0 && s1 < a.nshell && (unit || (s2 >= 0 && s2 < a.nshell)))
-                    kmin[side] = min(kmin[side], a.shell_K[s1] * (unit ? 1 : a.shell_K[s2]));
+                    kmin[side] = max(kmin[side], INT_MAX - max(0, a.shell_K[s1] * (unit ? 1 : a.shell_K[s2])));
             }
             if (a.spread) {
                 const int s1 = pr[2 * i], s2 = pr[2 * i + 1];
@@ -171,10 +182,10 @@ __global__ void prepass_kernel(PrepassArgs a)
                         bool bad = false;
                         float far = 0.f, zmax;
                         const float r = pair_spread(a, s1, unit ? -1 : s2, &bad, &far, &zmax);
-                        atomicMax(&a.spread[4 + side], __float_as_int(zmax));
-                        atomicMax(&a.spread[side], __float_as_int(r));  // r >= 1: int order = float order
+                        zeta[side] = max(zeta[side], __float_as_int(zmax));
+                        ratio[side] = max(ratio[side], __float_as_int(r));  // r >= 1: int order = float order
                         if (bad) a.spread[2] = 1;
-                        atomicMax(&a.spread[3], __float_as_int(far));
+                        coord = max(coord, __float_as_int(far));
                     }
                 }
             }
@@ -184,7 +195,7 @@ __global__ void prepass_kernel(PrepassArgs a)
                     const int K1 = a.shell_K[s1], K2 = a.shell_K[s2];
                     if (K1 >= 1 && K1 <= kKmax && K2 >= 1 && K2 <= kKmax) {
                         const float r = pair_recursion_risk(a, s1, s2, a.l[2 * side + 1]);
-                        atomicMax(&a.info[5 + side], __float_as_int(r));  // r >= 0: int order = float order
+                        risk[side] = max(risk[side], __float_as_int(r));  // r >= 0: int order = float order
                     }
                 }
             }
@@ -194,13 +205,16 @@ __global__ void prepass_kernel(PrepassArgs a)
             if (b < 0 || b >= a.nbra || k < 0 || k >= a.nket) set_err(&a.info[4], DEV_EINDEX);
         }
     }
-    if (a.kmin) {  // every thread of the block reaches this point
-        const int m0 = __reduce_min_sync(0xffffffffu, kmin[0]), m1 = __reduce_min_sync(0xffffffffu, kmin[1]);
-        if ((threadIdx.x & 31) == 0) {
-            if (m0 != 0x7fffffff) atomicMin(&a.kmin[0], m0);
-            if (m1 != 0x7fffffff) atomicMin(&a.kmin[1], m1);
-        }
+    // every thread of the block reaches this point
+    for (int c = 0; c < 4; ++c) warp_max_into(&a.info[c], kmax[c]);
+    for (int side = 0; side < 2; ++side) {
+        if (a.kmin) warp_max_into(&a.kmin[side], kmin[side]);
+        if (a.risk) warp_max_into(&a.info[5 + side], risk[side]);
+        if (!a.spread) continue;
+        warp_max_into(&a.spread[side], ratio[side]);
+        warp_max_into(&a.spread[4 + side], zeta[side]);
     }
+    if (a.spread) warp_max_into(&a.spread[3], coord);
 }
 
 // ---------------------------------------------------------------------------
@@ -868,10 +882,8 @@ int prepare_batch(eri_class_t cls, const eri_basis_t* basis, const int32_t* bra,
     // [0..6] as PrepassArgs::info, [7..8] the smallest pair counts per side,
     // [9..14] PrepassArgs::spread
     int* dinfo = status + 8;
-    if (cudaMemsetAsync(dinfo, 0, 7 * sizeof(int), st) != cudaSuccess ||
-        cudaMemsetAsync(dinfo + 7, 0x7f, 2 * sizeof(int), st) != cudaSuccess ||
-        cudaMemsetAsync(dinfo + 9, 0, 6 * sizeof(int), st) != cudaSuccess)
-        return ERI_ECUDA;
+    // (one call: a small batch is bound by its launches, about 2 us each)
+    if (cudaMemsetAsync(dinfo, 0, 15 * sizeof(int), st) != cudaSuccess) return ERI_ECUDA;
     // Where the fixed-point tile is the faster one (GB300, ms, FP64 against fixed
     // point): contracted 4-centre classes above (ss|ss): (pp|ps) K = 3, 1e5
     // quartets 3.48 / 2.31; (ds|ds) 6.76 / 3.70; (dp|pp), 6.5e4, 10.6 / 7.9.  Not
@@ -879,10 +891,12 @@ int prepare_batch(eri_class_t cls, const eri_basis_t* basis, const int32_t* bra,
     // quartets; not uncontracted batches, where set-up and barriers outweigh the
     // products: (pp|ps) 3e5 0.43 / 0.49, (ff|pp) 2e4 2.39 / 3.03; not 3-centre ones,
     // (f|dp) 1e5 4.90 / 6.20; nor small ones, (pp|pp) K = 3, 1000 quartets 0.217 / 0.236,
-    // which are not asked for their spread either.
+    // which are not asked for their spread either, nor is a basis without contracted
+    // shells (it adds 7 us to the checking pass: (ps|ss) K = 1, 4000 quartets 62 / 69 us a call).
     const int64_t nqq = quartets ? nq : nbra * nket;
     const bool try_fixed = fc && !split && ldelta == 0 && (kind == 0 || kind == 3) &&
-                           cls.la + cls.lb + cls.lc + cls.ld > 0 && nqq >= 2000;
+                           cls.la + cls.lb + cls.lc + cls.ld > 0 && nqq >= 2000 &&
+                           basis->nprim > basis->nshell;
     PrepassArgs pa{basis->shell_l, basis->shell_K, basis->nshell, bra, nbra, ket, nket, quartets,
                    quartets ? nq : (int64_t)0,
                    {cls.la, cls.lb, cls.lc, cls.ld}, (kind == 1 || kind == 2) ? 1 : 0, dinfo,
@@ -913,7 +927,7 @@ int prepare_batch(eri_class_t cls, const eri_basis_t* basis, const int32_t* bra,
     for (int c = 0; c < 4; ++c) kmax[c] = hinfo[c];
     *KB = kmax[0] * kmax[1];
     *KK = kmax[2] * kmax[3];
-    if (mixed) *mixed = (hinfo[7] < *KB || hinfo[8] < *KK) ? 1 : 0;
+    if (mixed) *mixed = (INT_MAX - hinfo[7] < *KB || INT_MAX - hinfo[8] < *KK) ? 1 : 0;
     const bool fix_ok = try_fixed && (int64_t)*KB * *KK >= 4 && nqq * *KB * *KK >= 150000 && fixed_eligible(cls, hinfo + 9);
     if (allow_swap) {
         // Four forms: which side is transformed first (Section 3.2.2
