@@ -56,7 +56,8 @@ enum {
 
 /* Precision of the Hermite-to-Cartesian transforms. */
 enum {
-    ERI_PREC_FP64 = 0,  /* everything in FP64 */
+    ERI_PREC_FP64 = 0,  /* FP64, or 64-bit fixed point of no larger error in
+                           contracted 4-centre batches */
     ERI_PREC_SPLIT = 1  /* transforms in FP32 hi+lo split products with FP64
                            accumulation; Boys, R and prefactors stay FP64;
                            plain (side-swapped or not) forms only, since the
@@ -399,7 +400,8 @@ int eri_last_form(int32_t* swapped, int32_t* hrr);
  * eri_last_tile -- the tile shape of the calling thread's last successful
  * eri_batch launch (measurement support): *tq quartets per tile, *ic bra
  * primitives per chunk of the auxiliary integrals, *threads per CTA (256, or
- * 512 for a tile that fills an SM's shared memory alone), *smem_bytes of
+ * 512 for a tile that fills an SM's shared memory alone; a fixed-point tile
+ * takes 128, 256 or 512), *smem_bytes of
  * dynamic shared memory per CTA.  HOST pointers, each may be NULL.  Returns
  * ERI_EINVAL before the thread's first eri_batch launch.  No counterpart in
  * the paper, whose kernels run on CPU cores (Section 3).
