@@ -111,7 +111,7 @@ __global__ void info_to_host_kernel(const int* __restrict__ src, int n, int* dst
 // maximum being that of the smallest exponents.  In floats from the FP64
 // distance (to about 1e-5: the guard compares it with a round power of ten);
 // FP64 pow and exp and a division per primitive pair took 26 of the 30 us that
-// this kernel was of a batch of 1000 (pp|pp) (143 us); now it takes 13.
+// this kernel was of a batch of 1000 (pp|pp) (143 us); in floats it took 13.
 __device__ float pair_recursion_risk(const PrepassArgs& a, int s1, int s2, int l2)
 {
     if (l2 == 0) return 1.0f;
@@ -886,7 +886,7 @@ int prepare_batch(eri_class_t cls, const eri_basis_t* basis, const int32_t* bra,
     if (cudaMemsetAsync(dinfo, 0, 15 * sizeof(int), st) != cudaSuccess) return ERI_ECUDA;
     // Where the fixed-point tile is the faster one (GB300, ms, FP64 against fixed
     // point): contracted 4-centre classes above (ss|ss): (pp|ps) K = 3, 1e5
-    // quartets 3.48 / 2.31; (ds|ds) 6.76 / 3.70; (dp|pp), 6.5e4, 10.6 / 7.9.  Not
+    // quartets 3.50 / 2.19; (ds|ds) 6.76 / 3.70; (dp|pp), 6.5e4, 10.6 / 8.1.  Not
     // (ss|ss), 4e5 of mixed degrees 5.12 / 5.37, whose tiles hold few primitive
     // quartets; not uncontracted batches, where set-up and barriers outweigh the
     // products: (pp|ps) 3e5 0.43 / 0.49, (ff|pp) 2e4 2.39 / 3.03; not 3-centre ones,
