@@ -309,9 +309,29 @@ FIX_HD long long fix_finish(long long R, long long phi, int sh)
     return sh < 0 ? (long long)((unsigned long long)v << (-sh & 63)) : v >> (sh > 63 ? 63 : sh);
 }
 
+// |P - Q|^2 in floats, from the whole coordinates (units of 2^-f): cut to their
+// high words, centres at the far end of the range would be off by 2^-7 bohr
+FIX_HD float fix_distance2(const FixPrim& p, const FixPrim& q, int f)
+{
+    const float unit = fix_pow2(-f);
+    float r2 = 0.f;
+#pragma unroll
+    for (int i = 0; i < 3; ++i) {
+        const float d = (float)(p.x[i] - q.x[i]) * unit;
+        r2 += d * d;
+    }
+    return r2;
+}
+
 // Exponent g with |order N of the integrals| s^-N < 2^g for n_min <= N <= L, from the
 // exponents and |X|^2: at any distance sqrt(rho) (2 rho)^(N/2) (N-1)!!/(N+1) (the
 // value at X = 0), and sqrt(pi)/2 N! / |X|^(N+1) up to a factor below 3.
+// At X = 0 that is no estimate but the value itself, so top is raised by
+// kFixBoundMargin: rho (a product, a sum and an approximate division of floats) is
+// within 2^-21, the root's seed and imu within 2^-22 of theirs, to powers of up to
+// 5.5 and 10, with a rounding for each product: less than 2^-17 together.  Next to a
+// power of two a bound that fell short would take the limbs (2^62 - 2^30) past their end.
+constexpr float kFixBoundMargin = 1.0f + 0x1p-15f;
 FIX_HD int fix_bound(int L, int n_min, float rho, float r2, int sigma, float imu)
 {
     const float is = fix_pow2(-sigma) * imu, ir = r2 > 1e-30f ? fix_rsqrt_seed(r2) : 1e15f;
@@ -327,6 +347,7 @@ FIX_HD int fix_bound(int L, int n_min, float rho, float r2, int sigma, float imu
             top = fmaxf(top, fminf(nr, 3.0f * far));
         }
     }
+    top *= kFixBoundMargin;
     return top > 1e-37f ? (int)(fix_float_bits(top) >> 23) - 126 : -126;
 }
 

@@ -591,19 +591,12 @@ __device__ void tile_fixed(const FwdArgs& a, int64_t q0, int nqt, double* sm, do
     // side of order l reads none of order below l)
     const int n_min = ct.pure == 1 ? ct.la : (ct.pure == 2 ? ct.lc : 0);
     {
-        const float unit = fix_pow2(32 - a.fx_f);
         const FastDiv d_bk(KBt * KKt);
         for (int idx = tid; idx < TQ * KBt * KKt; idx += NT) {
             const int q = d_bk.div(idx), r = idx - q * KBt * KKt, i = d_kkt.div(r), k = r - i * KKt;
             if (i >= s_q[4 * q + 2] || k >= s_q[4 * q + 3]) continue;
             const FixPrim &p = sPb[q * KB + i], &c = sPk[q * KK + k];
-            float r2 = 0.f;
-#pragma unroll
-            for (int x = 0; x < 3; ++x) {
-                const float d = (float)((int)(p.x[x] >> 32) - (int)(c.x[x] >> 32)) * unit;
-                r2 = fmaf(d, d, r2);
-            }
-            const float rho = __fdividef(p.zeta * c.zeta, p.zeta + c.zeta);
+            const float r2 = fix_distance2(p, c, a.fx_f), rho = __fdividef(p.zeta * c.zeta, p.zeta + c.zeta);
             atomicMax(&s_g[q * KB + i], fix_bound(ct.L, n_min, rho, r2, s_sig[q * KB + i], a.fx_imu));
         }
     }

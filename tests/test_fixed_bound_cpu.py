@@ -1,0 +1,144 @@
+"""The bound by which the fixed-point tile scales its auxiliary integrals
+(fix_bound in csrc/eri_fixaux.cuh, host code too): every integral stays inside
+its two limbs, |R| < 2^62 - 2^30, with exponents chosen so that the bound lies
+within a few units in the last place of a power of two, and at every distance."""
+import os
+import subprocess
+
+import pytest
+
+ROOT = os.path.dirname(os.path.dirname(os.path.abspath(__file__)))
+CSRC = os.path.join(ROOT, "paper_2506_12501_gb300", "csrc")
+
+SOURCE = r"""
+#include <algorithm>
+#include <cstdio>
+#include <random>
+#include <vector>
+#include "eri_fixaux.cuh"
+using namespace eri;
+typedef long double Q;
+int main() {
+    std::mt19937_64 g(11);
+    auto uni = [&](double a, double b) { return a + (b - a) * ((g() >> 11) * 0x1p-53); };
+    auto prim = [&](double z) {
+        FixPrim p{};
+        const double u = 1 / z;
+        fix_split_exponent(u, &p.um, &p.ue);
+        p.um += (long long)(fma(-u, z, 1.0) * (double)p.um);
+        p.zeta = (float)z;
+        return p;
+    };
+    // coincident centres: order N of the recursion is (N-1)!! / 4^(N/2) R^(N/2)_0
+    for (int L = 0; L <= 10; ++L) {
+        std::vector<Q> row(kBoysMtab + 2, 1);
+        for (int m = 0; m <= kBoysMtab; ++m) row[m] = 1.0L / (2 * m + 1);
+        std::vector<int64_t> tab(fix_boys_words(L) + 2), far(kFixFarWords);
+        fix_boys_row(row.data(), L, 0, tab.data());
+        fix_far_constants(L, far.data());
+        long past = 0;
+        double top = 0;
+        for (int it = 0; it < 60000; ++it) {
+            // the bound of order N at 2^e, to about 1e-7 or 1e-4 to either side; s from the batch's largest rho, here this one
+            const int N = 2 * (int)(g() % (L / 2 + 1)), e = (int)(g() % 9) - 4;
+            double c = 1.0 / (N + 1);
+            for (int k = 1; k < N; k += 2) c *= k / (1.1 * 1.1);
+            const double rho0 = pow(ldexp(1.0, e) / c, 2) * (1 + (it & 1 ? 4e-7 : 1e-4) * uni(-1, 1)) * pow(1.00001, 2 * N);
+            const double zp = rho0 * (1 + pow(10, uni(-2, 2))), zq = 1 / (1 / rho0 - 1 / zp);
+            const FixPrim p = prim(zp), q = prim(zq);
+            const double rho = zp * zq / (zp + zq), s = 1.1 * sqrt(2 * rho), mu = s / ldexp(1.0, ilogb(s)) * 1.00001;
+            const int sigma = (ilogb(2.42 / (mu * mu) * rho) + 2) >> 1;
+            // the device's approximate division may leave rho below its value
+            const float fr = (float)rho * (1 - (float)uni(0, 0x1p-21));
+            const int gg = fix_bound(L, 0, fr, fix_distance2(p, q, 50), sigma, (float)(1 / mu));
+            long long F[11], phi[11];
+            int sh[11];
+            FixBase B;
+            fix_base<10>(L, p, q, 50, (const long long*)tab.data(), (const long long*)far.data(), F, B);
+            if (L == 0) B.U = 1LL << 61, B.ue = 0;
+            fix_factors<10>(L, B, sigma, (long long)(0x1p62L / (Q)mu), gg, phi, sh);
+            bool hit = false;
+            for (int M = 0; M <= L; M += 2) {
+                long long R = F[M / 2];
+                for (int k = 1; k < M; k += 2) R = (R * k) >> 2;
+                const long long v = std::abs(fix_finish(R, phi[M], sh[M]));
+                hit |= v >= (1LL << 62) - (1LL << 30);
+                top = std::max(top, (double)v * 0x1p-62);
+            }
+            past += hit;
+        }
+        printf("%d %ld %.9f\n", L, past, top);
+    }
+    // every distance, along an axis (the largest entries): |[N,0,0]| against the bound itself
+    // (units 2^g, before it is rounded up to a power of two, the exponent carries that)
+    double worst = 0;
+    for (int it = 0; it < 40000; ++it) {
+        const double T = pow(10, uni(-3, 2.3)), rho = pow(10, uni(-1, 2)), r = sqrt(T / rho);
+        Q F[12], term, sum;
+        const int M = 11;
+        term = sum = 1.0L / (2 * M + 1);
+        for (int k = 1; k < 3000 && term > sum * 1e-22L; ++k) { term *= 2 * (Q)T / (2 * M + 2 * k + 1); sum += term; }
+        F[M] = expl(-(Q)T) * sum;
+        for (int m = M - 1; m >= 0; --m) F[m] = (2 * (Q)T * F[m + 1] + expl(-(Q)T)) / (2 * m + 1);
+        const int L = (int)(g() % 11);
+        std::vector<Q> R(L + 1, 0);
+        R[0] = F[L] * powl(-2 * rho, L);
+        for (int n = L - 1; n >= 0; --n) {
+            for (int t = L - n; t >= 1; --t) R[t] = r * R[t - 1] + (t > 1 ? (t - 1) * R[t - 2] : 0);
+            R[0] = F[n] * powl(-2 * rho, n);
+        }
+        const double mu = uni(1, 2);
+        const int sigma = (ilogb(2.42 / (mu * mu) * rho) + 2) / 2 - (int)(g() % 6);
+        const int gg = fix_bound(L, 0, (float)rho, (float)(r * r), sigma, (float)(1 / mu));
+        for (int N = 0; N <= L; ++N)
+            worst = std::max(worst, fabs((double)(sqrtl(rho) * R[N] * powl(mu * powl(2, sigma), -N) * powl(2, -gg))));
+    }
+    printf("distance 0 %.9f\n", worst);
+    // the squared distance of centres at the far end of the admitted coordinates
+    double off = 0;
+    for (int it = 0; it < 2000; ++it) {
+        FixPrim p = prim(1), q = prim(1);
+        double r2 = 0;
+        for (int i = 0; i < 3; ++i) {
+            const double a = 1e6 * uni(-1, 1), b = a + pow(10, uni(-4, 1));
+            p.x[i] = fix_coordinate(a, 40);
+            q.x[i] = fix_coordinate(b, 40);
+            r2 += (b - a) * (b - a);
+        }
+        off = std::max(off, fabs(fix_distance2(p, q, 40) / r2 - 1));
+    }
+    printf("coordinates 0 %.3e\n", off);
+}
+"""
+
+
+@pytest.fixture(scope="module")
+def figures(tmp_path_factory):
+    d = tmp_path_factory.mktemp("bound")
+    src = d / "bound.cpp"
+    src.write_text(SOURCE)
+    from paper_2506_12501_gb300.build import nvcc
+    inc = os.path.join(os.path.dirname(os.path.dirname(os.path.realpath(nvcc()))), "include")
+    subprocess.run(["g++", "-O2", "-std=gnu++17", "-I", CSRC, "-I", inc, str(src), "-o", str(d / "bound")], check=True,
+                   capture_output=True)
+    out = subprocess.run([str(d / "bound")], check=True, capture_output=True, text=True, timeout=300).stdout
+    return {w[0]: (int(w[1]), float(w[2])) for w in (line.split() for line in out.splitlines())}
+
+
+@pytest.mark.parametrize("L", range(11))
+def test_coincident_centres_stay_inside_the_limbs(figures, L):
+    past, top = figures[str(L)]
+    assert past == 0
+    assert top < 1 - 2.0 ** -32
+    if L % 2 == 0:  # the largest bound is an even order's, which the samples do reach
+        assert top > 0.999
+
+
+def test_every_distance_stays_inside_the_bound(figures):
+    # rounding the bound up to a power of two leaves the margin where the bound is attained
+    assert 0.9 < figures["distance"][1] < 1 - 2.0 ** -32
+
+
+def test_distance_of_centres_at_the_end_of_the_range(figures):
+    # coordinates to 2^-40 bohr and 1e6 to 53 bits: 2^-33 over 1e-4 bohr, and a few roundings of a float
+    assert figures["coordinates"][1] < 2.0 ** -18
