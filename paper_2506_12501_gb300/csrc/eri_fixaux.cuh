@@ -100,6 +100,26 @@ FIX_HD unsigned fix_float_bits(float x)
 #endif
 }
 
+FIX_HD float fix_inverse(float x)  // correctly rounded
+{
+#ifdef __CUDA_ARCH__
+    return __frcp_rn(x);
+#else
+    return 1.0f / x;
+#endif
+}
+
+// sigma with mu 2^sigma >= 1.1 sqrt(2 rho), at most a factor 2 above; c = 2.42 / mu^2
+FIX_HD int fix_sigma(float rho, float c)
+{
+    const int e = (int)(fix_float_bits(c * rho) >> 23) - 127;  // 2^e <= y < 2^(e+1)
+    return (e + 2) >> 1;
+}
+// Reduced exponent of two sums of exponents.  Every operation is rounded to
+// nearest, so it never falls as zb grows: the tile's scales rely on that, and
+// zb (zk / (zb + zk)) does fall, by its last place, in one of twelve steps.
+FIX_HD float fix_reduced(float zb, float zk) { return fix_inverse(fix_inverse(zb) + fix_inverse(zk)); }
+
 // two consecutive 8-byte words, 16-byte aligned
 FIX_HD void fix_load2(const long long* p, long long& a, long long& b)
 {

@@ -62,13 +62,6 @@ __host__ __device__ __forceinline__ int herm_order(int e)
     return n;
 }
 
-// sigma with mu 2^sigma >= 1.1 sqrt(2 rho), at most a factor 2 above; c = 2.42 / mu^2
-__device__ __forceinline__ int fix_sigma(float rho, float c)
-{
-    const int e = (__float_as_int(c * rho) >> 23) - 127;  // 2^e <= y < 2^(e+1)
-    return (e + 2) >> 1;
-}
-
 // x 2^sh rounded to the nearest integer; |x 2^sh| < 2^62, zero and denormals give 0
 __device__ __forceinline__ long long fix_from(double x, int sh)
 {
@@ -565,10 +558,11 @@ __device__ void tile_fixed(const FwdArgs& a, int64_t q0, int nqt, double* sm, do
     for (int idx = tid; idx < nC; idx += NT) sA[idx] = 0;
     __syncthreads();
     // sigma of (quartet, bra primitive i): the pairs' slots are sorted by
-    // exponent, descending, so ket slot 0 gives the largest reduced exponent
+    // exponent, descending, so ket slot 0 gives the largest reduced exponent, and
+    // sigma never grows with i
     auto sigma_of = [&](int q, int i) {
         const float zb = sPb[q * KB + i].zeta, zk = sPk[q * KK].zeta;
-        return min(fix_sigma(zb, a.fx_c), fix_sigma(zb * (zk / (zb + zk)), a.fx_c));
+        return min(fix_sigma(zb, a.fx_c), fix_sigma(fix_reduced(zb, zk), a.fx_c));
     };
     auto norm_exp = [&](int q, int cd, int sigma) {
         const int64_t g = (int64_t)s_q[4 * q + 1] * ncd + cd;

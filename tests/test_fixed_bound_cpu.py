@@ -12,6 +12,7 @@ CSRC = os.path.join(ROOT, "paper_2506_12501_gb300", "csrc")
 
 SOURCE = r"""
 #include <algorithm>
+#include <climits>
 #include <cstdio>
 #include <random>
 #include <vector>
@@ -108,6 +109,19 @@ int main() {
         off = std::max(off, fabs(fix_distance2(p, q, 40) / r2 - 1));
     }
     printf("coordinates 0 %.3e\n", off);
+    // sigma along neighbouring exponents, its step placed among them
+    long falls = 0;
+    for (int it = 0; it < 20000; ++it) {
+        const float zk = (float)pow(10, uni(-1, 2));
+        float z = (float)pow(10, uni(-1, 2));
+        const float step = fix_reduced(nextafterf(z, 1e30f), zk), c = 4.0f / step;
+        for (int j = 0, last = INT_MIN; j < 64; ++j, z = nextafterf(z, 1e30f)) {
+            const int s = std::min(fix_sigma(z, c), fix_sigma(fix_reduced(z, zk), c));
+            falls += s < last;
+            last = s;
+        }
+    }
+    printf("sigma %ld 0\n", falls);
 }
 """
 
@@ -142,3 +156,8 @@ def test_every_distance_stays_inside_the_bound(figures):
 def test_distance_of_centres_at_the_end_of_the_range(figures):
     # coordinates to 2^-40 bohr and 1e6 to 53 bits: 2^-33 over 1e-4 bohr, and a few roundings of a float
     assert figures["coordinates"][1] < 2.0 ** -18
+
+
+def test_hermite_unit_never_grows_as_the_exponent_falls(figures):
+    # the tile takes the first bra primitive's unit (the largest exponent's) for the largest
+    assert figures["sigma"][0] == 0
