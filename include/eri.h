@@ -409,6 +409,26 @@ int eri_last_form(int32_t* swapped, int32_t* hrr);
 int eri_last_tile(int32_t* tq, int32_t* ic, int32_t* threads, int32_t* smem_bytes);
 
 /*
+ * eri_last_arithmetic -- the arithmetic of the transforms in the calling
+ * thread's last successful eri_batch, eri_batch_sph or eri_batch3 launch:
+ * *arithmetic is one of the values below.  HOST pointer.  Returns ERI_EINVAL
+ * before the thread's first launch.
+ */
+enum {
+    ERI_ARITH_FP64 = 0,  /* FP64 tile */
+    ERI_ARITH_SPLIT = 1, /* ERI_PREC_SPLIT */
+    ERI_ARITH_FIXED = 2  /* ERI_PREC_FP64 by the fixed-point tile */
+};
+int eri_last_arithmetic(int32_t* arithmetic);
+
+/*
+ * eri_set_fixed -- whether later ERI_PREC_FP64 batches of the CALLING THREAD
+ * may take the fixed-point tile (1, a thread's start) or keep to the FP64
+ * tile (0).  Returns the previous value, or ERI_EINVAL for another argument.
+ */
+int eri_set_fixed(int32_t allowed);
+
+/*
  * eri_set_forms -- restrict the forms later eri_batch calls (all threads)
  * may choose from: bit 0 plain, bit 1 plain with the sides swapped, bit 2
  * recursion form, bit 3 recursion form swapped; 0 restores all four.  A

@@ -45,10 +45,12 @@ EXPORTS = ["eri_boys", "eri_batch", "eri_batch_grad", "eri_last_status", "eri_er
            "eri_plan_execute", "eri_plan_set_budget", "eri_plan_status", "eri_plan_info", "eri_plan_job",
            "eri_plan_destroy", "eri_last_form", "eri_set_forms", "eri_plan_coulomb", "eri_plan_jk", "eri_plan_job_degrees", "eri_batch3", "eri_solid_harmonics", "eri_batch_sph",
            "eri_last_grad_forms", "eri_set_grad_forms", "eri_peak_probe",
-           "eri_partition", "eri_plan_set_slice", "eri_plan_slice_info", "eri_last_tile"]
+           "eri_partition", "eri_plan_set_slice", "eri_plan_slice_info", "eri_last_tile",
+           "eri_last_arithmetic", "eri_set_fixed"]
 ERI_NOALLOC_SCRATCH_BYTES = 64 * 1024 * 1024
 ERI_PLAN_STORE, ERI_PLAN_SPLIT, ERI_PLAN_NO_TUNE = 1, 2, 4
 ERI_FORM_PLAIN, ERI_FORM_HRR = 0x3, 0xC
+ERI_ARITH_FP64, ERI_ARITH_SPLIT, ERI_ARITH_FIXED = 0, 1, 2
 ERI_GRAD_X, ERI_GRAD_V, ERI_GRAD_ONE, ERI_GRAD_TWO, ERI_GRAD_ONE_SWAPPED = 0, 1, 2, 3, 4
 PROF_FWD, PROF_GRAD, PROF_PAIR, PROF_PREPASS = 0, 1, 2, 3
 
@@ -73,6 +75,8 @@ def lib() -> ctypes.CDLL:
             L.eri_last_form.argtypes = [P, P]
             L.eri_last_tile.argtypes = [P, P, P, P]
             L.eri_set_forms.argtypes = [ctypes.c_int32]
+            L.eri_last_arithmetic.argtypes = [P]
+            L.eri_set_fixed.argtypes = [ctypes.c_int32]
             L.eri_last_grad_forms.argtypes = [P, P]
             L.eri_set_grad_forms.argtypes = [ctypes.c_int32]
             L.eri_error_string.argtypes = [I]
@@ -332,6 +336,21 @@ def eri_last_tile() -> dict:
     v = [ctypes.c_int32() for _ in range(4)]
     _check(lib().eri_last_tile(*(ctypes.byref(x) for x in v)), "eri_last_tile")
     return {"tq": v[0].value, "ic": v[1].value, "threads": v[2].value, "smem_bytes": v[3].value}
+
+
+def eri_last_arithmetic() -> int:
+    """Arithmetic of this thread's last forward launch: ERI_ARITH_FP64, ERI_ARITH_SPLIT or ERI_ARITH_FIXED."""
+    v = ctypes.c_int32()
+    _check(lib().eri_last_arithmetic(ctypes.byref(v)), "eri_last_arithmetic")
+    return v.value
+
+
+def eri_set_fixed(allowed: bool) -> bool:
+    """Whether this thread's FP64-precision batches may take the fixed-point tile; returns the previous setting."""
+    code = lib().eri_set_fixed(int(allowed))
+    if code < 0:
+        _check(code, "eri_set_fixed")
+    return bool(code)
 
 
 def eri_set_grad_forms(mask: int) -> int:

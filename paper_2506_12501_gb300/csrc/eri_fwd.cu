@@ -826,6 +826,9 @@ constexpr double kRecursionRisk = 900.0;
 // Forms eri_batch may use (eri_set_forms): bit o allows form o.
 static std::atomic<int> g_form_mask{0xF};
 
+// Whether the calling thread's batches may take the fixed-point tile (eri_set_fixed).
+static thread_local int g_allow_fixed = 1;
+
 // Forms chosen by timing, per (device, class, K_bra, K_ket, precision).
 static std::map<std::tuple<int, int, int, int, int, int, int, int, int>, int> g_forms;
 static std::mutex g_forms_mu;
@@ -894,7 +897,7 @@ int prepare_batch(eri_class_t cls, const eri_basis_t* basis, const int32_t* bra,
     // which are not asked for their spread either, nor is a basis without contracted
     // shells (it adds 7 us to the checking pass: (ps|ss) K = 1, 4000 quartets 62 / 69 us a call).
     const int64_t nqq = quartets ? nq : nbra * nket;
-    const bool try_fixed = fc && !split && ldelta == 0 && (kind == 0 || kind == 3) &&
+    const bool try_fixed = fc && g_allow_fixed && !split && ldelta == 0 && (kind == 0 || kind == 3) &&
                            cls.la + cls.lb + cls.lc + cls.ld > 0 && nqq >= 2000 &&
                            basis->nprim > basis->nshell;
     PrepassArgs pa{basis->shell_l, basis->shell_K, basis->nshell, bra, nbra, ket, nket, quartets,
@@ -1459,6 +1462,7 @@ static int forward_args(const eri_basis_t* basis, const int32_t* bra_pairs, int6
 
 static thread_local int g_last_form = -1;
 static thread_local TilePlan g_last_tile{};
+static thread_local int g_last_arithmetic = XF_FP64;
 
 // One forward batch of any kind (0: 4-centre; 1, 2: 3-centre with the unit
 // function as the second bra shell, Cartesian or solid-harmonic x): form
@@ -1573,6 +1577,7 @@ static int run_forward(eri_class_t cls, const eri_basis_t* basis, const int32_t*
     if (cudaGetLastError() != cudaSuccess) return ERI_ECUDA;
     g_last_form = fc.form;
     g_last_tile = tp;
+    g_last_arithmetic = fc.fixed ? XF_FIXED : split;
     return ERI_OK;
 }
 
@@ -1661,6 +1666,23 @@ extern "C" int eri_last_tile(int32_t* tq, int32_t* ic, int32_t* threads, int32_t
     if (threads) *threads = g_last_tile.nt;
     if (smem_bytes) *smem_bytes = (int32_t)g_last_tile.bytes;
     return ERI_OK;
+}
+
+static_assert(XF_FP64 == ERI_ARITH_FP64 && XF_SPLIT == ERI_ARITH_SPLIT && XF_FIXED == ERI_ARITH_FIXED, "one numbering");
+
+extern "C" int eri_last_arithmetic(int32_t* arithmetic)
+{
+    if (!arithmetic || g_last_form < 0) return ERI_EINVAL;
+    *arithmetic = g_last_arithmetic;
+    return ERI_OK;
+}
+
+extern "C" int eri_set_fixed(int32_t allowed)
+{
+    if (allowed != 0 && allowed != 1) return ERI_EINVAL;
+    const int prev = g_allow_fixed;
+    g_allow_fixed = allowed;
+    return prev;
 }
 
 extern "C" int eri_last_form(int32_t* swapped, int32_t* hrr)

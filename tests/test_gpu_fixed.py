@@ -35,6 +35,7 @@ def test_fixed_tile_against_oracle(cls, K):
         eri.eri_set_forms(1 << form)
         try:
             out = eri.eri_batch(cls, db, b, k, qq).cpu().numpy().reshape(-1, nq).T
+            assert eri.eri_last_arithmetic() == eri.ERI_ARITH_FIXED
         finally:
             eri.eri_set_forms(0)
         pick = np.r_[0:12, nq - 12:nq]
@@ -59,11 +60,13 @@ def test_fixed_tile_mixed_degrees_product_form_and_sph():
     db = eri.DeviceBasis(basis)
     nab, ncd = 3, 9
     out = eri.eri_batch(cls, db, b, k).cpu().numpy().reshape(53, ncd, nab, 61)
+    assert eri.eri_last_arithmetic() == eri.ERI_ARITH_FIXED
     q = np.array([(i, j) for i in range(0, 61, 7) for j in range(0, 53, 6)])
     ref = oracle_blocks(cls, basis, bra, ket, q).reshape(len(q), nab, ncd)
     got = np.stack([out[j, :, :, i].T for i, j in q])
     assert_close(got, ref, what="product form, mixed degrees")
     sph = eri.eri_batch_sph(cls, db, b, k).cpu().numpy().reshape(53, ncd, nab, 61)
+    assert eri.eri_last_arithmetic() == eri.ERI_ARITH_FIXED
     # p functions in solid harmonics: m = -1, 0, 1 are y, z, x
     order = np.array([1, 2, 0])
     cd = (order[:, None] * 3 + order[None, :]).reshape(-1)
@@ -86,6 +89,7 @@ def test_fixed_tile_far_and_coincident_centres():
     q = np.stack([rng.integers(0, len(near), nq), rng.integers(0, len(ket), nq)], 1)
     b, k, qq = to_device(near, ket, q)
     out = eri.eri_batch(cls, eri.DeviceBasis(basis), b, k, qq).cpu().numpy().reshape(-1, nq).T
+    assert eri.eri_last_arithmetic() == eri.ERI_ARITH_FIXED
     ref = oracle_blocks(cls, basis, near, ket, q[:400])
     assert_close(out[:400], ref, what="centres of every distance")
 
@@ -98,9 +102,47 @@ def test_wide_exponents_and_non_finite_primitives_keep_the_fp64_tile():
     bra, ket, q = synth.class_sweep_batch(pools, cls, seed=9, npairs=40, nq=nq)
     b, k, qq = to_device(bra, ket, q)
     out = eri.eri_batch(cls, eri.DeviceBasis(basis), b, k, qq).cpu().numpy().reshape(-1, nq).T
+    assert eri.eri_last_arithmetic() == eri.ERI_ARITH_FP64
     assert_close(out[:60], oracle_blocks(cls, basis, bra, ket, q[:60]), what="wide exponents")
     basis, pools = synth.class_sweep_pools(seed=8, lmax=1, pool=32, K=3, cube=3.0)
     basis.coefs[basis.shell_off[bra[0, 0]]] = np.nan
     out = eri.eri_batch(cls, eri.DeviceBasis(basis), b, k, qq).cpu().numpy().reshape(-1, nq).T
+    assert eri.eri_last_arithmetic() == eri.ERI_ARITH_FP64
     bad = np.any(bra[q[:, 0]] == bra[0, 0], axis=1) | np.any(ket[q[:, 1]] == bra[0, 0], axis=1)
     assert bad.any() and np.isnan(out[bad]).all() and np.isfinite(out[~bad]).all()
+
+
+@pytest.mark.parametrize("cls,K,nq", [((1, 1, 1, 0), 3, 20011), ((2, 1, 2, 0), 2, 16384), ((2, 2, 1, 1), 2, 16385)])
+def test_timed_tiles_and_form_against_oracle(cls, K, nq):
+    """Batches long enough to be timed: the tile shape and the form come from the timing; the second call, which
+    uses what the first remembered, gives the same bits."""
+    basis, pools = synth.class_sweep_pools(seed=13, lmax=max(cls), pool=64, K=K, cube=4.0)
+    bra, ket, q = synth.class_sweep_batch(pools, cls, seed=14, npairs=50, nq=nq)
+    b, k, qq = to_device(bra, ket, q)
+    db = eri.DeviceBasis(basis)
+    out = []
+    for _ in range(2):
+        out.append(eri.eri_batch(cls, db, b, k, qq).cpu().numpy().reshape(-1, nq).T)
+        assert eri.eri_last_arithmetic() == eri.ERI_ARITH_FIXED
+    pick = np.r_[0:12, nq // 2:nq // 2 + 12, nq - 12:nq]
+    assert_close(out[0][pick], oracle_blocks(cls, basis, bra, ket, q[pick]), what=f"{cls} K={K}")
+    np.testing.assert_array_equal(out[0], out[1])
+
+
+def test_callers_choice_of_the_fp64_tile():
+    """eri_set_fixed(False) keeps this thread's batches on the FP64 tile; both agree to round-off."""
+    cls, nq = (1, 1, 1, 0), 4001
+    basis, pools = synth.class_sweep_pools(seed=15, lmax=1, pool=32, K=3, cube=4.0)
+    bra, ket, q = synth.class_sweep_batch(pools, cls, seed=16, npairs=40, nq=nq)
+    b, k, qq = to_device(bra, ket, q)
+    db = eri.DeviceBasis(basis)
+    fixed = eri.eri_batch(cls, db, b, k, qq).cpu().numpy()
+    assert eri.eri_last_arithmetic() == eri.ERI_ARITH_FIXED
+    assert eri.eri_set_fixed(False) is True
+    try:
+        fp64 = eri.eri_batch(cls, db, b, k, qq).cpu().numpy()
+        assert eri.eri_last_arithmetic() == eri.ERI_ARITH_FP64
+    finally:
+        assert eri.eri_set_fixed(True) is False
+    assert_close(fixed, fp64, what="fixed point against FP64")
+    assert not np.array_equal(fixed, fp64)

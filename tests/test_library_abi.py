@@ -103,3 +103,19 @@ def test_tile_query_and_probe_kinds_without_gpu():
     assert L.eri_peak_probe(4, ctypes.byref(g), None, None) == eri.ERI_EINVAL
     assert L.eri_peak_probe(-1, ctypes.byref(g), None, None) == eri.ERI_EINVAL
     assert L.eri_peak_probe(3, None, None, None) == eri.ERI_EINVAL
+
+
+def test_arithmetic_selector_without_gpu():
+    """eri_set_fixed and eri_last_arithmetic check their arguments on the host; the setting is the thread's own."""
+    import threading
+    import paper_2506_12501_gb300 as eri
+    L = eri.lib()
+    assert L.eri_last_arithmetic(None) == eri.ERI_EINVAL
+    assert L.eri_set_fixed(2) == eri.ERI_EINVAL and L.eri_set_fixed(-1) == eri.ERI_EINVAL
+    assert eri.eri_set_fixed(False) is True
+    seen = []
+    t = threading.Thread(target=lambda: seen.append(eri.eri_set_fixed(True)))
+    t.start()
+    t.join()
+    assert seen == [True]
+    assert eri.eri_set_fixed(True) is False
