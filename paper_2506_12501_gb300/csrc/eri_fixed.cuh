@@ -46,6 +46,12 @@ namespace eri {
 
 // log2 of the largest spread factor of a pair for the fixed-point tile
 constexpr float kFixSpreadBits = 6.0f;
+// Largest order the tile takes.  Above it one exponent for the integrals of all
+// orders costs more than the FP64 tile's roundings: relative 2-norm error against
+// the oracle, fixed point | FP64, K = 2, pairs of two centres in a 4-bohr cube:
+// (fd|fd), order 10, 2.8e-14 | 1.3e-15; (fd|dd), order 9, 1.2e-14 | 1.0e-15.
+constexpr int kFixLmax = 8;
+static_assert(kFixLmax <= kFixAuxLmax, "order of the fixed-point auxiliary integrals");
 // products per low-limb accumulator between folds: each below 2^28 2^31.  Even:
 // the ket transform reads its operands in aligned pairs from each multiple on.
 constexpr int kFixFold = 14;
@@ -656,7 +662,7 @@ __device__ void tile_fixed(const FwdArgs& a, int64_t q0, int nqt, double* sm, do
                 case 2: run(IntC<2>(), IntC<1>()); break;
                 case 3: run(IntC<3>(), IntC<1>()); break;
                 case 4: run(IntC<4>(), IntC<1>()); break;
-                default: run(IntC<kFixAuxLmax>(), IntC<0>());
+                default: run(IntC<kFixLmax>(), IntC<0>());
             }
         }
         {

@@ -547,7 +547,7 @@ bool tile_layout(const ClassTables& ct, int KB, int KK, int TQ, int IC, int e_sm
     const bool fixed = split == XF_FIXED;
     const int nx = fixed ? IC : 1;  // X of a chunk's bra primitives, or of one
     const int ps_n = fixed ? (int)(sizeof(FixPrim) / 8) : PS_N;
-    if (fixed && ct.L > kFixAuxLmax) return false;
+    if (fixed && ct.L > kFixLmax) return false;
     if (fixed && !e_smem) return false;
     const int KS = (KK + 1) & ~1;
     if (fixed) {
@@ -897,8 +897,9 @@ int prepare_batch(eri_class_t cls, const eri_basis_t* basis, const int32_t* bra,
     // which are not asked for their spread either, nor is a basis without contracted
     // shells (it adds 7 us to the checking pass: (ps|ss) K = 1, 4000 quartets 62 / 69 us a call).
     const int64_t nqq = quartets ? nq : nbra * nket;
+    const int L = cls.la + cls.lb + cls.lc + cls.ld;
     const bool try_fixed = fc && g_allow_fixed && !split && ldelta == 0 && (kind == 0 || kind == 3) &&
-                           cls.la + cls.lb + cls.lc + cls.ld > 0 && nqq >= 2000 &&
+                           L > 0 && L <= kFixLmax && nqq >= 2000 &&
                            basis->nprim > basis->nshell;
     PrepassArgs pa{basis->shell_l, basis->shell_K, basis->nshell, bra, nbra, ket, nket, quartets,
                    quartets ? nq : (int64_t)0,

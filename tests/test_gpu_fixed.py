@@ -112,6 +112,22 @@ def test_wide_exponents_and_non_finite_primitives_keep_the_fp64_tile():
     assert bad.any() and np.isnan(out[bad]).all() and np.isfinite(out[~bad]).all()
 
 
+@pytest.mark.parametrize("cls", [(3, 2, 2, 2), (3, 2, 3, 2)])
+def test_orders_above_eight_keep_the_fp64_tile(cls):
+    """Contracted classes of order 9 and 10: FP64 tile, whose error stays at a few 1e-15 (in fixed point it was 1e-14)."""
+    nq = 9382
+    basis, pools = synth.class_sweep_pools(seed=3, lmax=3, pool=64, K=2, cube=4.0)
+    bra, ket, q = synth.class_sweep_batch(pools, cls, seed=4, npairs=50, nq=nq)
+    b, k, qq = to_device(bra, ket, q)
+    eri.eri_set_forms(1)
+    try:
+        out = eri.eri_batch(cls, eri.DeviceBasis(basis), b, k, qq).cpu().numpy().reshape(-1, nq).T
+    finally:
+        eri.eri_set_forms(0)
+    assert eri.eri_last_arithmetic() == eri.ERI_ARITH_FP64
+    assert _sample_error(out[:24], oracle_blocks(cls, basis, bra, ket, q[:24], prec="ld")) < 5e-15
+
+
 @pytest.mark.parametrize("cls,K,nq", [((1, 1, 1, 0), 3, 20011), ((2, 1, 2, 0), 2, 16384), ((2, 2, 1, 1), 2, 16385)])
 def test_timed_tiles_and_form_against_oracle(cls, K, nq):
     """Batches long enough to be timed: the tile shape and the form come from the timing; the second call, which
