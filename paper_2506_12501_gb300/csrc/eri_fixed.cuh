@@ -19,8 +19,14 @@
 //    terms over all ket primitives (2^h), so no sum of products overflows:
 //    |sum E R| <= 2^60 2^62.  Likewise the bra's E, over all its primitives.
 //  * X (the ket-transformed integrals) is aligned to the quartet's largest g and
-//    h and to sigma_i before the bra transform, whose sums over bra
-//    primitives then add without further scaling.
+//    h before the bra transform, whose sums over bra primitives then add without
+//    further scaling.
+//  * the bra's limbs are formed once a pair, with sigma_i; X of order n is then
+//    shifted by n (sigma_i - sigma) to meet them.  A column without low orders
+//    (p_x p_y of one centre has order 2 alone) would lose those bits: a
+//    quartet in which a column may lose more than kFixWeakBits forms its limbs
+//    from the E products at its own sigmas, relative to a bound F of the 1-norm
+//    there, and leaves X as it is.
 // A number is held as two signed limbs, hi 2^31 + lo (R), hi 2^32 + lo (X) or
 // hi 2^29 + lo (E); a product keeps hi hi, hi lo and lo hi, and the dropped lo lo is below
 // 2^-64 of the bound.
@@ -56,6 +62,9 @@ static_assert(kFixLmax <= kFixAuxLmax, "order of the fixed-point auxiliary integ
 // the ket transform reads its operands in aligned pairs from each multiple on.
 constexpr int kFixFold = 14;
 static_assert(kFixFold % 2 == 0, "pairs of ket primitives stay 16-byte aligned");
+
+// bits a bra column may lose to the shift of X before its quartet forms the limbs itself
+constexpr int kFixWeakBits = 4;
 
 template <int N>
 using IntC = std::integral_constant<int, N>;
@@ -121,13 +130,16 @@ __device__ __forceinline__ long long fix_bra_sum(const FixAcc& s)
 }
 
 // ---- pair tables -----------------------------------------------------------
-// One thread per (pair, component pair) over its terms and primitives.  Bra
-// role: the column's E products become limbs in place, times 2^(sigma_i |p|)
-// and relative to the column's 1-norm, whose exponent goes to ex.  Ket role:
-// the products stay doubles (each quartet scales them by its own sigma); the
-// 1-norms per Hermite order go to norm[8] relative to 2^ex.
+// One thread per (pair, component pair) over its terms and primitives: the
+// column's 1-norms per Hermite order go to norm[8], relative to 2^ex.  Ket role:
+// of the products themselves, which each quartet scales by its own sigma.  Bra
+// role: of the products times 2^(sigma_i |p|); their limbs, relative to the whole
+// 1-norm (2^ex again); and the bits by which its order 0 lies below that, the
+// largest of a pair to weak.
 struct FixPairArgs {
-    double* E;            // ket role [npairs][T][KS], bra role [npairs][KS][T]
+    const double* E;      // ket role [npairs][T][KS], bra role [npairs][KS][T]
+    int2* limbs;          // [npairs][KS][T] (bra role)
+    int* weak;            // [npairs], zeros (bra role)
     const FixPrim* ps;    // [npairs][KS]
     const int32_t* kp;    // [npairs]
     const int* start;     // [ncol + 1] terms of a column
@@ -136,7 +148,7 @@ struct FixPairArgs {
     int KS, T, ncol, ket;
     float c;              // 2.42 / mu^2 (fix_sigma)
     int* ex;              // [npairs][ncol]
-    float* norm;          // [npairs][ncol][8] (ket role)
+    float* norm;          // [npairs][ncol][8]
 };
 
 __device__ __forceinline__ int fix_norm_exp(const float* n, int base, int sigma)
@@ -152,7 +164,7 @@ static __global__ void __launch_bounds__(128) fix_pairs_kernel(FixPairArgs a)
     for (int64_t g = blockIdx.x * (int64_t)blockDim.x + threadIdx.x; g < total; g += (int64_t)gridDim.x * blockDim.x) {
         const int64_t j = g / a.ncol;
         const int c = (int)(g - j * a.ncol), K = a.kp[j];
-        double* E = a.E + (size_t)j * a.T * a.KS;
+        const double* E = a.E + (size_t)j * a.T * a.KS;
         const FixPrim* ps = a.ps + (size_t)j * a.KS;
         const int t0 = a.start[c], t1 = a.start[c + 1], ts = a.ket ? a.KS : 1, ks = a.ket ? 1 : a.T;
         int top = 0;
@@ -167,29 +179,28 @@ static __global__ void __launch_bounds__(128) fix_pairs_kernel(FixPairArgs a)
             for (int k = 0; k < K; ++k) {
                 const int hi = __double2hiint(E[t * ts + k * ks]) & 0x7fffffff;
                 const int e = (hi >> 20) - 1023 - base;
-                const float v = e > -120 ? __int_as_float((((e + 127) << 23) | ((hi & 0xfffff) << 3)) + 8) : 0.f;
-                if (a.ket) {
-#pragma unroll
-                    for (int i = 0; i < 7; ++i)
-                        if (i == o) n[i] = __fadd_ru(n[i], v);
-                } else {
-                    const int sg = fix_sigma(ps[k].zeta, a.c) * o;
-                    sum = __fadd_ru(sum, v * __int_as_float((127 + sg) << 23));
+                float v = e > -120 ? __int_as_float((((e + 127) << 23) | ((hi & 0xfffff) << 3)) + 8) : 0.f;
+                if (!a.ket) {
+                    v *= __int_as_float((127 + fix_sigma(ps[k].zeta, a.c) * o) << 23);
+                    sum = __fadd_ru(sum, v);
                 }
+#pragma unroll
+                for (int i = 0; i < 7; ++i)
+                    if (i == o) n[i] = __fadd_ru(n[i], v);
             }
         }
-        if (a.ket) {
-            for (int i = 0; i < 8; ++i) a.norm[8 * g + i] = n[i];
-            a.ex[g] = top ? base : -1000;
-        } else {
-            const int f = top ? base + (__float_as_int(sum) >> 23) - 126 : -1000;
-            a.ex[g] = f;
+        // (bra: in units of the 1-norm, a power of two)
+        const int up = a.ket ? 0 : (__float_as_int(sum) >> 23) - 126;
+        for (int i = 0; i < 8; ++i) a.norm[8 * g + i] = a.ket ? n[i] : ldexpf(n[i], -up);
+        a.ex[g] = top ? base + up : -1000;
+        if (!a.ket) {
+            const int f = top ? base + up : -1000;
+            if (top) atomicMax(&a.weak[j], n[0] > 0.f ? (__float_as_int(sum) >> 23) - (__float_as_int(n[0]) >> 23) : 1000);
             for (int t = t0; t < t1; ++t) {
                 const int o = herm_order(a.herm[t]);
                 for (int k = 0; k < K; ++k) {
-                    double* e = E + t * ts + k * ks;
                     const int sg = fix_sigma(ps[k].zeta, a.c) * o;
-                    *reinterpret_cast<int2*>(e) = fix_limbs<kLimbE>(fix_from(*e, 60 + sg - f));
+                    a.limbs[((size_t)j * a.KS + k) * a.T + t] = fix_limbs<kLimbE>(fix_from(E[t + k * ks], 60 + sg - f));
                 }
             }
         }
@@ -449,6 +460,7 @@ struct FixTables {
     const int16_t* kq;    // [Tcd]
     const uint16_t* pq;   // [nhb][nhk] offset into R of p+q
     const int16_t* tc;    // [Tcd] 8 column + order of a ket term
+    const int16_t* bc;    // [Tab] and of a bra term
     const int16_t* ord;   // [nhl] order of a Hermite function
     const int16_t *kpair, *bpair; // [nkpair][2], [nbpair][2]
     const FixStep* st;    // [nhl]
@@ -461,7 +473,8 @@ struct FixTables {
         kq = reinterpret_cast<const int16_t*>(bp + ct.Tab);
         pq = reinterpret_cast<const uint16_t*>(kq + ct.Tcd);
         tc = reinterpret_cast<const int16_t*>(pq + ct.nhb * ct.nhk);
-        ord = tc + ct.Tcd;
+        bc = tc + ct.Tcd;
+        ord = bc + ct.Tab;
         kpair = ord + ct.nhl;
         bpair = kpair + 2 * ct.nkpair;
     }
@@ -469,17 +482,18 @@ struct FixTables {
 inline size_t fix_table_bytes(const ClassTables& ct)
 {
     return sizeof(FixStep) * (size_t)ct.nhl + 4 * (ct.nab + ct.ncd + 2) +
-           2 * (ct.Tab + 2 * ct.Tcd + ct.nhb * ct.nhk + ct.nhl + 2 * ct.nkpair + 2 * ct.nbpair);
+           2 * (2 * ct.Tab + 2 * ct.Tcd + ct.nhb * ct.nhk + ct.nhl + 2 * ct.nkpair + 2 * ct.nbpair);
 }
 
 // The tile's integer scratch: per (quartet, bra primitive) sigma, the bound g
-// (then its distance to the quartet's largest G), sigma_i - sigma and whether
-// the ket's E change there; per bra primitive whether any quartet's do; per
-// quartet G; per (quartet, column) the exponent H (largest sigma) and its
-// distance to the current sigma's.
-__host__ __device__ __forceinline__ int fix_scratch_ints(int TQ, int KB, int ncd)
+// (then its distance to the quartet's largest G), sigma_i - sigma, and flags: bit 0
+// the ket's E change there, bit 1 the quartet forms its bra limbs itself; per bra
+// primitive whether any quartet's E change; per quartet G; per (quartet, ket column)
+// the exponent H (largest sigma) and its distance to the current sigma's; per
+// (quartet, bra column) the exponent F.
+__host__ __device__ __forceinline__ int fix_scratch_ints(int TQ, int KB, int nab, int ncd)
 {
-    return 4 * TQ * KB + KB + TQ + 2 * TQ * ncd;
+    return 4 * TQ * KB + KB + TQ + 2 * TQ * ncd + TQ * nab;
 }
 
 constexpr int kFixRegL = 4;  // auxiliary integrals in registers up to this order
@@ -506,6 +520,7 @@ __device__ void tile_fixed(const FwdArgs& a, int64_t q0, int nqt, double* sm, do
     int* s_G = s_any + KB;
     int* s_dh = s_G + TQ;
     int* s_H = s_dh + TQ * ncd;
+    int* s_F = s_H + TQ * ncd;
     const int lgTQ = 31 - __clz(TQ);  // TQ is a power of two
     const FastDiv d_ncd(ncd), d_kb(KB);
     __shared__ int s_kmax[2], s_next;
@@ -521,13 +536,15 @@ __device__ void tile_fixed(const FwdArgs& a, int64_t q0, int nqt, double* sm, do
     {
         int mkb = 0, mkk = 0;
         for (int q = tid; q < TQ; q += NT) {
-            int b = 0, k = 0, kb = 0, kk = 0;
+            int b = 0, k = 0, kb = 0, kk = 0, weak = 0;
             const int64_t qq = q < nqt && a.order ? a.order[q0 + q] : q0 + q;
             if (q < nqt) {
                 quartet_pairs(a, qq, &b, &k);
                 kb = a.bra_kp[b];
                 kk = a.ket_kp[k];
+                weak = a.bra_weak[b] > kFixWeakBits;
             }
+            s_ch[q * KB] = weak;
             s_q[4 * q] = b;
             s_q[4 * q + 1] = k;
             s_q[4 * q + 2] = kb;
@@ -587,6 +604,24 @@ __device__ void tile_fixed(const FwdArgs& a, int64_t q0, int nqt, double* sm, do
         s_H[idx] = q < nqt ? norm_exp(q, idx - q * ncd, sigma_of(q, 0)) : 0;
     }
     __syncthreads();
+    // whether quartet q forms its bra limbs itself; lo: the smallest sigma_i - sigma
+    auto own_limbs = [&](int q, int* lo) {
+        int hi = 0;
+        *lo = 1000;
+        if (!s_ch[q * KB]) return false;  // (so far: whether the pair has a weak column)
+        for (int i = 0; i < s_q[4 * q + 2]; ++i) {
+            hi = max(hi, s_ds[q * KB + i]);
+            *lo = min(*lo, s_ds[q * KB + i]);
+        }
+        return hi * (ct.la + ct.lb) > kFixWeakBits;
+    };
+    for (int idx = tid; idx < TQ * nab; idx += NT) {
+        const int q = idx & (TQ - 1), ab = idx >> lgTQ;
+        int lo;
+        if (!own_limbs(q, &lo)) continue;
+        const int64_t g = (int64_t)s_q[4 * q] * nab + ab;
+        s_F[idx] = fix_norm_exp(a.bra_norm + 8 * g, a.bra_ex[g], -lo);
+    }
     // bounds of the auxiliary integrals the transforms read (a solid-harmonic
     // side of order l reads none of order below l)
     const int n_min = ct.pure == 1 ? ct.la : (ct.pure == 2 ? ct.lc : 0);
@@ -604,8 +639,12 @@ __device__ void tile_fixed(const FwdArgs& a, int64_t q0, int nqt, double* sm, do
     for (int i = tid; i < KB; i += NT) s_any[i] = 0;
     __syncthreads();
     for (int q = tid; q < TQ; q += NT) {
-        int G = -1000, cur = INT_MIN;
-        for (int i = 0; i < s_q[4 * q + 2]; ++i) G = max(G, s_g[q * KB + i]);
+        int G = -1000, cur = INT_MIN, lo;
+        const bool own = own_limbs(q, &lo);
+        for (int i = 0; i < s_q[4 * q + 2]; ++i) {
+            G = max(G, s_g[q * KB + i]);
+            if (own) s_ds[q * KB + i] = 0;
+        }
         for (int i = 0; i < KB; ++i) {
             const int sg = s_sig[q * KB + i];
             int ch = 0;
@@ -614,7 +653,7 @@ __device__ void tile_fixed(const FwdArgs& a, int64_t q0, int nqt, double* sm, do
                 cur = sg;
                 if (ch) s_any[i] = 1;
             }
-            s_ch[q * KB + i] = ch;
+            s_ch[q * KB + i] = ch + 2 * own;
         }
         s_G[q] = G;
     }
@@ -670,11 +709,19 @@ __device__ void tile_fixed(const FwdArgs& a, int64_t q0, int nqt, double* sm, do
             const int nb = n * ct.Tab;
             const FastDiv d_nb(nb), d_tab(ct.Tab);
             for (int idx = tid; idx < TQ * nb; idx += NT) {
-                const int q = d_nb.div(idx), r = idx - q * nb;
-                sEb[q * a.sEbS + r] =
-                    i0 + d_tab.div(r) < s_q[4 * q + 2]
-                        ? reinterpret_cast<const int2*>(a.bra_E)[((size_t)s_q[4 * q] * KB + i0) * ct.Tab + r]
-                        : make_int2(0, 0);
+                const int q = d_nb.div(idx), r = idx - q * nb, ii = d_tab.div(r);
+                const size_t src = ((size_t)s_q[4 * q] * KB + i0) * ct.Tab + r;
+                int2 e = make_int2(0, 0);
+                if (i0 + ii < s_q[4 * q + 2]) {
+                    if (s_ch[q * KB] & 2) {
+                        const int bc = tb.bc[r - ii * ct.Tab];
+                        const int sh = 60 + s_sig[q * KB + i0 + ii] * (bc & 7) - s_F[(bc >> 3) * TQ + q];
+                        e = fix_limbs<kLimbE>(fix_from(a.bra_E[src], sh));
+                    } else {
+                        e = a.bra_limbs[src];
+                    }
+                }
+                sEb[q * a.sEbS + r] = e;
             }
         }
         if (s_any[i0]) {
@@ -682,14 +729,14 @@ __device__ void tile_fixed(const FwdArgs& a, int64_t q0, int nqt, double* sm, do
             // to their columns' 1-norms at the new sigma
             for (int idx = tid; idx < TQ * ncd; idx += NT) {
                 const int q = d_ncd.div(idx);
-                if (s_ch[q * KB + i0]) s_dh[idx] = s_H[idx] - norm_exp(q, idx - q * ncd, s_sig[q * KB + i0]);
+                if (s_ch[q * KB + i0] & 1) s_dh[idx] = s_H[idx] - norm_exp(q, idx - q * ncd, s_sig[q * KB + i0]);
             }
             __syncthreads();
             const int nk = KK * ct.Tcd;
             const FastDiv d_qk(nk), d_kk(KK);
             for (int idx = tid; idx < TQ * nk; idx += NT) {
                 const int q = d_qk.div(idx), r = idx - q * nk, t = d_kk.div(r), k = r - t * KK;
-                if (!s_ch[q * KB + i0]) continue;
+                if (!(s_ch[q * KB + i0] & 1)) continue;
                 const int tc = tb.tc[t], c = q * ncd + (tc >> 3);
                 const int sh = 60 + s_sig[q * KB + i0] * (tc & 7) - s_H[c] + s_dh[c];
                 sEk[q * a.sEkS + t * KS + k] =
@@ -717,7 +764,8 @@ __device__ void tile_fixed(const FwdArgs& a, int64_t q0, int nqt, double* sm, do
                     const int t2 = c2 < 0 ? t1 : tb.kstart[c2], n2 = c2 < 0 ? 0 : tb.kstart[c2 + 1] - t2;
                     const int2* Rc = reinterpret_cast<const int2*>(sR) + q * QS + ii * KS;
                     const int p0 = ct.pb0 + pg, p1 = ct.pb0 + pg + npg;
-                    // (for a quartet without primitive i the bra's E are zero, and X immaterial)
+                    // (for a quartet without primitive i the bra's E are zero, and X immaterial;
+                    // ds is 0 where the quartet forms its own bra limbs)
                     const int dG = s_G[q] - s_g[x], ds = s_ds[x];
                     int2* X = sX + ii * XS + q;
                     auto put = [&](int p, int cd, const FixAcc& v) {
@@ -807,7 +855,8 @@ __device__ void tile_fixed(const FwdArgs& a, int64_t q0, int nqt, double* sm, do
         [&](int, int item) {
             const int q = item & (TQ - 1), r = item >> lgTQ, ab = d_ncd.div(r), cd = r - ab * ncd;
             if (q >= nqt) return 0.0;
-            const int e = s_G[q] + s_H[q * ncd + cd] + a.bra_ex[(size_t)s_q[4 * q] * nab + ab] - 62;
+            const int F = s_ch[q * KB] & 2 ? s_F[ab * TQ + q] : a.bra_ex[(size_t)s_q[4 * q] * nab + ab];
+            const int e = s_G[q] + s_H[q * ncd + cd] + F - 62;
             // two factors: e may pass the exponent range of one
             const int eh = max(-1000, min(1000, e)), el = max(-1000, min(1000, e - eh));
             double v = (double)sA[item] * __hiloint2double((1023 + eh) << 20, 0);
@@ -818,7 +867,7 @@ __device__ void tile_fixed(const FwdArgs& a, int64_t q0, int nqt, double* sm, do
 }
 
 // Class tables into shared memory: the FP64 tile's, with the Hermite indices
-// turned into offsets of this tile shape, the ket terms' columns and orders,
+// turned into offsets of this tile shape, the terms' columns and orders,
 // the Hermite orders.
 template <int NT>
 __device__ __forceinline__ void stage_fixed_tables(const FwdArgs& a, double* sm)
@@ -836,6 +885,9 @@ __device__ __forceinline__ void stage_fixed_tables(const FwdArgs& a, double* sm)
     for (int cd = tid; cd < ct.ncd; cd += NT)
         for (int t = ct.ket_start[cd]; t < ct.ket_start[cd + 1]; ++t)
             const_cast<int16_t*>(tb.tc)[t] = (int16_t)(cd * 8 + herm_order(ct.ket_q[t]));
+    for (int ab = tid; ab < ct.nab; ab += NT)
+        for (int t = ct.bra_start[ab]; t < ct.bra_start[ab + 1]; ++t)
+            const_cast<int16_t*>(tb.bc)[t] = (int16_t)(ab * 8 + herm_order(ct.bra_p[t]));
     for (int e = tid; e < ct.nhl; e += NT) {
         const_cast<int16_t*>(tb.ord)[e] = (int16_t)herm_order(e);
         const RStep r = a.rsteps[e];

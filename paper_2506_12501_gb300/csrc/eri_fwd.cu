@@ -249,6 +249,7 @@ struct PairArgs {
     // zeta, ps holds FixPrim with coordinates in units of 2^-fx_f, and the E
     // products carry a further zeta^(-1/2),
     int fixed, fx_f;
+    int32_t* weak;          // [npairs], zeroed here (bra)
     double mu;              // and mu^(Hermite order) (eri_fixed.cuh)
 };
 
@@ -285,7 +286,10 @@ __global__ void __launch_bounds__(kPairThreads) pair_kernel_t(PairArgs a)
         // bra; its centre is immaterial and taken as the first shell's
         const int s1 = a.pairs[2 * j], s2 = a.pairs[2 * j + 1];
         const int K1 = a.shell_K[s1], K2 = s2 < 0 ? 1 : a.shell_K[s2];
-        if (s == 0 && x0 == 0 && lane == 0) a.kprim[j] = K1 * K2;
+        if (s == 0 && x0 == 0 && lane == 0) {
+            a.kprim[j] = K1 * K2;
+            if (!RAISED && a.weak) a.weak[j] = 0;
+        }
         if (s >= K1 * K2) {  // padding slot: finite zeros, never contributes
             if (RAISED) {
                 for (int q = 0; q < a.eax; ++q) a.ax[((size_t)g * 3 + x0) * a.eax + q] = 0.0;
@@ -608,7 +612,7 @@ bool tile_layout(const ClassTables& ct, int KB, int KK, int TQ, int IC, int e_sm
     tp->o_Ei = -1;
     if (!e_smem && TQ == 1 && (off + even(ct.Tab)) * 8 <= (size_t)max_smem_optin()) tp->o_Ei = take(ct.Tab);
     tp->o_Er = -1;  // added for the split form by add_e_ring
-    tp->o_fx = fixed ? take((fix_scratch_ints(TQ, KB, ct.ncd) + 1) / 2) : -1;
+    tp->o_fx = fixed ? take((fix_scratch_ints(TQ, KB, ct.nab, ct.ncd) + 1) / 2) : -1;
     tp->o_acc = fixed ? take((size_t)TQ * ct.nab * ct.ncd) : -1;
     tp->bytes = off * 8;
     tp->nt = fixed ? nt : kNT;
@@ -794,12 +798,14 @@ static double fix_unit(double rho)
     return s > 0.0 ? s / std::ldexp(1.0, std::ilogb(s)) * 1.00001 : 1.0;
 }
 
-// The fixed-point form of one side's pair tables (in place on the bra).
+// The fixed-point form of one side's pair tables.
 static void launch_fix_pairs(const PairTables& t, const ClassTables& ct, int64_t npairs, int KS, int side, double mu,
                              cudaStream_t st)
 {
     FixPairArgs f{};
     f.E = t.E;
+    f.limbs = t.limbs;
+    f.weak = t.weak;
     f.ps = reinterpret_cast<const FixPrim*>(t.ps);
     f.kp = t.kp;
     f.start = side ? ct.ket_start : ct.bra_start;
@@ -1051,8 +1057,10 @@ int prepare_batch(eri_class_t cls, const eri_basis_t* basis, const int32_t* bra,
     const size_t nb_x = fixed ? align_up(sizeof(int32_t) * nbra * ct->nab) : 0;
     const size_t nk_x = fixed ? align_up(sizeof(int32_t) * nket * ct->ncd) : 0;
     const size_t nk_n = fixed ? align_up(sizeof(float) * 8 * nket * ct->ncd) : 0;
+    const size_t nb_n = fixed ? align_up(sizeof(float) * 8 * nbra * ct->nab) : 0;
+    const size_t nb_l = fixed ? nb_E : 0, nb_w = fixed ? align_up(sizeof(int32_t) * nbra) : 0;
     const size_t n_grad = nb_ax + nk_ax + nb_z + nk_z;
-    uint8_t* ws = (uint8_t*)workspace(nb_ps + nb_E + nk_ps + nk_E + nb_k + nk_k + n_grad + nb_x + nk_x + nk_n, &err);
+    uint8_t* ws = (uint8_t*)workspace(nb_ps + nb_E + nk_ps + nk_E + nb_k + nk_k + n_grad + nb_x + nk_x + nk_n + nb_n + nb_l + nb_w, &err);
     if (!ws) return err;
     {
         uint8_t* g0 = ws + nb_ps + nb_E + nk_ps + nk_E + nb_k + nk_k;
@@ -1065,7 +1073,12 @@ int prepare_batch(eri_class_t cls, const eri_basis_t* basis, const int32_t* bra,
         pb->ex = fixed ? (int32_t*)(g0 + n_grad) : nullptr;
         pk->ex = fixed ? (int32_t*)(g0 + n_grad + nb_x) : nullptr;
         pk->norm = fixed ? (float*)(g0 + n_grad + nb_x + nk_x) : nullptr;
-        pb->norm = nullptr;
+        uint8_t* l0 = g0 + n_grad + nb_x + nk_x + nk_n;
+        pb->norm = fixed ? (float*)l0 : nullptr;
+        pb->limbs = fixed ? (int2*)(l0 + nb_n) : nullptr;
+        pb->weak = fixed ? (int32_t*)(l0 + nb_n + nb_l) : nullptr;
+        pk->limbs = nullptr;
+        pk->weak = nullptr;
     }
     pb->ps = (double*)ws;
     pb->E = (double*)(ws + nb_ps);
@@ -1100,6 +1113,7 @@ int prepare_batch(eri_class_t cls, const eri_basis_t* basis, const int32_t* bra,
         p.fixed = fixed;
         p.fx_f = fx_f;
         p.mu = mu;
+        p.weak = t.weak;
         p.hrr = ct->hrr;
         p.scale = side ? ct->ket_scale : ct->bra_scale;
         const int64_t tot = p.npairs * p.KS;
@@ -1438,6 +1452,9 @@ static int forward_args(const eri_basis_t* basis, const int32_t* bra_pairs, int6
     a->ket_E = pk.E;
     a->ket_kp = pk.kp;
     a->bra_ex = pb.ex;
+    a->bra_norm = pb.norm;
+    a->bra_limbs = pb.limbs;
+    a->bra_weak = pb.weak;
     a->ket_ex = pk.ex;
     a->ket_norm = pk.norm;
     a->quartets = quartets;

@@ -157,7 +157,9 @@ struct PairTables {
     int eax;      // doubles per axis table
     double* zz;   // adjoint only: [npairs][KS][2] exponents
     int32_t* ex;  // fixed-point tile: exponents of the E columns [npairs][ncol] (see eri_fixed.cuh)
-    float* norm;  // fixed-point tile, ket: their 1-norms per Hermite order [npairs][ncol][8]
+    float* norm;  // fixed-point tile: their 1-norms per Hermite order [npairs][ncol][8]
+    int2* limbs;  // fixed-point tile, bra: the E products as limbs [npairs][KS][T]
+    int32_t* weak;  // fixed-point tile, bra: bits of the weakest order 0 of a pair's columns [npairs]
 };
 
 // Form of a forward batch: bit 0 = sides swapped (the caller's ket is the

@@ -39,3 +39,55 @@ def test_one_centre_bounds_at_powers_of_two(N, cls):
             np.testing.assert_array_equal(out[1:], out[:-1])
     finally:
         eri.eri_set_forms(0)
+
+
+def _column_errors(got, ref):
+    """Relative 2-norm error of every component quadruple over the quartets, where it is not zero by symmetry."""
+    top = np.linalg.norm(ref, axis=0)
+    on = top > 1e-40
+    return (np.linalg.norm(got - ref, axis=0)[on] / top[on])
+
+
+def _both_tiles(cls, basis, bra, ket, q, n):
+    """The first n quartets' integrals from the fixed-point and the FP64 tile, and the oracle's."""
+    b, k, qq = to_device(bra, ket, q)
+    db = eri.DeviceBasis(basis)
+    out = []
+    for fixed in (True, False):
+        eri.eri_set_fixed(fixed)
+        try:
+            out.append(eri.eri_batch(cls, db, b, k, qq).cpu().numpy().reshape(-1, len(q)).T[:n])
+        finally:
+            eri.eri_set_fixed(True)
+        assert eri.eri_last_arithmetic() == (eri.ERI_ARITH_FIXED if fixed else eri.ERI_ARITH_FP64)
+    return out[0], out[1], oracle_blocks(cls, basis, bra, ket, q[:n], prec="ld")
+
+
+@pytest.mark.parametrize("tight", [30.0, 2e3, 1e5])
+@pytest.mark.parametrize("cls", [(1, 0, 1, 0), (2, 1, 1, 0), (1, 1, 1, 1), (2, 2, 1, 0)])
+def test_tight_one_centre_pairs_against_diffuse_ones(cls, tight):
+    """A one-centre pair's columns may start at any Hermite order: each component is as close as from the FP64 tile,
+    however far the pair's exponents lie above the other side's.  (Tight pairs at the origin: elsewhere the rounding
+    of their centre, 1e-16 of the coordinate, bounds both tiles.)"""
+    rng = np.random.default_rng(31)
+    n, m, nq = 8, 40, 10240
+    centres = np.concatenate([np.zeros((1, 3)), rng.uniform(-3, 3, (m, 3))])
+    diffuse = 0.2 * np.array([1.0, 2.0])
+    shells = sum((_shells([0] * n, l, [tight * (1 + i / n) * diffuse for i in range(n)], rng) for l in cls[:2]), [])
+    shells += sum((_shells(range(1, m + 1), l, [diffuse] * m, rng) for l in cls[2:]), [])
+    basis = synth.basis_from_shells(centres, shells)
+    i, j = np.arange(n), np.arange(m)
+    core = np.stack([i, n + i], 1).astype(np.int32)
+    val = np.stack([2 * n + j, 2 * n + m + (j + j % 3) % m], 1).astype(np.int32)  # one- and two-centre pairs
+    q = np.stack([np.arange(nq) % n, np.arange(nq) // n % m], 1).astype(np.int64)
+    for sides, forms in ((0, 1), (1, 2)):  # the tight pair on the kernel's bra, from either place in the call
+        eri.eri_set_forms(forms)
+        try:
+            if sides == 0:
+                fixed, fp64, ref = _both_tiles(cls, basis, core, val, q, n * m)
+            else:
+                fixed, fp64, ref = _both_tiles(cls[2:] + cls[:2], basis, val, core, q[:, ::-1].copy(), n * m)
+        finally:
+            eri.eri_set_forms(0)
+        # a component: one rounding of each product and sum, twice that for sums of a few hundred terms
+        assert _column_errors(fixed, ref).max() < max(2e-14, 2 * _column_errors(fp64, ref).max())
