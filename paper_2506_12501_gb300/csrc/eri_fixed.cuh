@@ -9,10 +9,14 @@
 //
 // Scales (all powers of two, so scaling rounds nothing):
 //  * Hermite orders carry a length: for bra primitive i a unit s = mu 2^sigma
-//    with s >= 1.1 sqrt(2 rho), rho the largest reduced exponent i meets, and mu
+//    with s >= 1.1 sqrt(2 rho), rho the largest reduced exponent i meets or, at a
+//    distance r of the two pairs, kFixFarT / r^2 if that is less, and mu
 //    in [1, 2) fixed for the batch (exact for its largest rho; the E products
 //    come with mu^|q|); R of order N is taken times s^(-N), E of order |q|
 //    times 2^(sigma |q|).  sigma_i (bra alone, rho -> zeta_i) bounds it from above.
+//    At a distance order N falls as N! / r^N, so that in units of sqrt(2 rho) high
+//    orders, which are the whole integral of one-centre pairs such as p_x p_y, would
+//    keep few of the bits that all orders share; in units of about 3 / r they stay level.
 //  * R of one (quartet, bra primitive) is relative to 2^g, a bound of its
 //    entries over the ket primitives (fix_bound); |R| <= 2^62 units.
 //  * each column (component pair) of E is relative to the 1-norm of its
@@ -63,6 +67,9 @@ static_assert(kFixLmax <= kFixAuxLmax, "order of the fixed-point auxiliary integ
 constexpr int kFixFold = 14;
 static_assert(kFixFold % 2 == 0, "pairs of ket primitives stay 16-byte aligned");
 
+// T = rho r^2 from which the Hermite unit follows the distance: s r >= 1.1 sqrt(8) = 3.1,
+// at most twice that, keeps N! / (s r)^N between 2^-6 and 2^6 for N <= 8
+constexpr float kFixFarT = 4.0f;
 // bits a bra column may lose to the shift of X before its quartet forms the limbs itself
 constexpr int kFixWeakBits = 4;
 
@@ -149,6 +156,8 @@ struct FixPairArgs {
     float c;              // 2.42 / mu^2 (fix_sigma)
     int* ex;              // [npairs][ncol]
     float* norm;          // [npairs][ncol][8]
+    float* box;           // [npairs][6] smallest, largest coordinates of the primitive pairs' centres
+    int f;                // their units 2^-f
 };
 
 __device__ __forceinline__ int fix_norm_exp(const float* n, int base, int sigma)
@@ -166,6 +175,16 @@ static __global__ void __launch_bounds__(128) fix_pairs_kernel(FixPairArgs a)
         const int c = (int)(g - j * a.ncol), K = a.kp[j];
         const double* E = a.E + (size_t)j * a.T * a.KS;
         const FixPrim* ps = a.ps + (size_t)j * a.KS;
+        if (c == 0)
+            for (int x = 0; x < 3; ++x) {
+                long long lo = ps[0].x[x], hi = lo;
+                for (int k = 1; k < K; ++k) {
+                    lo = min(lo, ps[k].x[x]);
+                    hi = max(hi, ps[k].x[x]);
+                }
+                a.box[6 * j + x] = (float)lo * fix_pow2(-a.f);
+                a.box[6 * j + 3 + x] = (float)hi * fix_pow2(-a.f);
+            }
         const int t0 = a.start[c], t1 = a.start[c + 1], ts = a.ket ? a.KS : 1, ks = a.ket ? 1 : a.T;
         int top = 0;
         for (int t = t0; t < t1; ++t)
@@ -488,12 +507,12 @@ inline size_t fix_table_bytes(const ClassTables& ct)
 // The tile's integer scratch: per (quartet, bra primitive) sigma, the bound g
 // (then its distance to the quartet's largest G), sigma_i - sigma, and flags: bit 0
 // the ket's E change there, bit 1 the quartet forms its bra limbs itself; per bra
-// primitive whether any quartet's E change; per quartet G; per (quartet, ket column)
+// primitive whether any quartet's E change; per quartet G and the largest rho for its distance; per (quartet, ket column)
 // the exponent H (largest sigma) and its distance to the current sigma's; per
 // (quartet, bra column) the exponent F.
 __host__ __device__ __forceinline__ int fix_scratch_ints(int TQ, int KB, int nab, int ncd)
 {
-    return 4 * TQ * KB + KB + TQ + 2 * TQ * ncd + TQ * nab;
+    return 4 * TQ * KB + KB + 2 * TQ + 2 * TQ * ncd + TQ * nab;
 }
 
 constexpr int kFixRegL = 4;  // auxiliary integrals in registers up to this order
@@ -521,6 +540,7 @@ __device__ void tile_fixed(const FwdArgs& a, int64_t q0, int nqt, double* sm, do
     int* s_dh = s_G + TQ;
     int* s_H = s_dh + TQ * ncd;
     int* s_F = s_H + TQ * ncd;
+    float* s_lim = reinterpret_cast<float*>(s_F + TQ * nab);
     const int lgTQ = 31 - __clz(TQ);  // TQ is a power of two
     const FastDiv d_ncd(ncd), d_kb(KB);
     __shared__ int s_kmax[2], s_next;
@@ -544,6 +564,15 @@ __device__ void tile_fixed(const FwdArgs& a, int64_t q0, int nqt, double* sm, do
                 kk = a.ket_kp[k];
                 weak = a.bra_weak[b] > kFixWeakBits;
             }
+            // the distance of the pairs' boxes
+            float r2 = 0.f;
+#pragma unroll
+            for (int x = 0; x < 3; ++x) {
+                const float *B = a.bra_box + 6 * (int64_t)b + x, *K = a.ket_box + 6 * (int64_t)k + x;
+                const float d = fmaxf(0.f, fmaxf(B[0] - K[3], K[0] - B[3]));
+                r2 = fmaf(d, d, r2);
+            }
+            s_lim[q] = __fdividef(kFixFarT, r2);
             s_ch[q * KB] = weak;
             s_q[4 * q] = b;
             s_q[4 * q + 1] = k;
@@ -585,7 +614,7 @@ __device__ void tile_fixed(const FwdArgs& a, int64_t q0, int nqt, double* sm, do
     // sigma never grows with i
     auto sigma_of = [&](int q, int i) {
         const float zb = sPb[q * KB + i].zeta, zk = sPk[q * KK].zeta;
-        return min(fix_sigma(zb, a.fx_c), fix_sigma(fix_reduced(zb, zk), a.fx_c));
+        return min(fix_sigma(zb, a.fx_c), fix_sigma(fminf(fix_reduced(zb, zk), s_lim[q]), a.fx_c));
     };
     auto norm_exp = [&](int q, int cd, int sigma) {
         const int64_t g = (int64_t)s_q[4 * q + 1] * ncd + cd;

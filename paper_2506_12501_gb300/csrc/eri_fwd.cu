@@ -800,7 +800,7 @@ static double fix_unit(double rho)
 
 // The fixed-point form of one side's pair tables.
 static void launch_fix_pairs(const PairTables& t, const ClassTables& ct, int64_t npairs, int KS, int side, double mu,
-                             cudaStream_t st)
+                             int fx_f, cudaStream_t st)
 {
     FixPairArgs f{};
     f.E = t.E;
@@ -818,6 +818,8 @@ static void launch_fix_pairs(const PairTables& t, const ClassTables& ct, int64_t
     f.c = (float)(2.42 / (mu * mu));
     f.ex = t.ex;
     f.norm = t.norm;
+    f.box = t.box;
+    f.f = fx_f;
     const int64_t n = npairs * f.ncol;
     count_launch();
     fix_pairs_kernel<<<(int)std::max<int64_t>(1, std::min<int64_t>((n + 127) / 128, 16LL * sm_count())), 128, 0, st>>>(f);
@@ -1058,9 +1060,10 @@ int prepare_batch(eri_class_t cls, const eri_basis_t* basis, const int32_t* bra,
     const size_t nk_x = fixed ? align_up(sizeof(int32_t) * nket * ct->ncd) : 0;
     const size_t nk_n = fixed ? align_up(sizeof(float) * 8 * nket * ct->ncd) : 0;
     const size_t nb_n = fixed ? align_up(sizeof(float) * 8 * nbra * ct->nab) : 0;
+    const size_t nb_b = fixed ? align_up(sizeof(float) * 6 * nbra) : 0, nk_b = fixed ? align_up(sizeof(float) * 6 * nket) : 0;
     const size_t nb_l = fixed ? nb_E : 0, nb_w = fixed ? align_up(sizeof(int32_t) * nbra) : 0;
     const size_t n_grad = nb_ax + nk_ax + nb_z + nk_z;
-    uint8_t* ws = (uint8_t*)workspace(nb_ps + nb_E + nk_ps + nk_E + nb_k + nk_k + n_grad + nb_x + nk_x + nk_n + nb_n + nb_l + nb_w, &err);
+    uint8_t* ws = (uint8_t*)workspace(nb_ps + nb_E + nk_ps + nk_E + nb_k + nk_k + n_grad + nb_x + nk_x + nk_n + nb_n + nb_l + nb_w + nb_b + nk_b, &err);
     if (!ws) return err;
     {
         uint8_t* g0 = ws + nb_ps + nb_E + nk_ps + nk_E + nb_k + nk_k;
@@ -1079,6 +1082,8 @@ int prepare_batch(eri_class_t cls, const eri_basis_t* basis, const int32_t* bra,
         pb->weak = fixed ? (int32_t*)(l0 + nb_n + nb_l) : nullptr;
         pk->limbs = nullptr;
         pk->weak = nullptr;
+        pb->box = fixed ? (float*)(l0 + nb_n + nb_l + nb_w) : nullptr;
+        pk->box = fixed ? (float*)(l0 + nb_n + nb_l + nb_w + nb_b) : nullptr;
     }
     pb->ps = (double*)ws;
     pb->E = (double*)(ws + nb_ps);
@@ -1126,7 +1131,7 @@ int prepare_batch(eri_class_t cls, const eri_basis_t* basis, const int32_t* bra,
             launch_pair(pe, std::max(g, 1), st);
         }
         launch_pair(p, std::max(g, 1), st);
-        if (fixed) launch_fix_pairs(t, *ct, p.npairs, p.KS, side, mu, st);
+        if (fixed) launch_fix_pairs(t, *ct, p.npairs, p.KS, side, mu, fx_f, st);
         if (cudaGetLastError() != cudaSuccess) return ERI_ECUDA;
     }
     return ERI_OK;
@@ -1453,6 +1458,8 @@ static int forward_args(const eri_basis_t* basis, const int32_t* bra_pairs, int6
     a->ket_kp = pk.kp;
     a->bra_ex = pb.ex;
     a->bra_norm = pb.norm;
+    a->bra_box = pb.box;
+    a->ket_box = pk.box;
     a->bra_limbs = pb.limbs;
     a->bra_weak = pb.weak;
     a->ket_ex = pk.ex;

@@ -158,6 +158,7 @@ struct PairTables {
     double* zz;   // adjoint only: [npairs][KS][2] exponents
     int32_t* ex;  // fixed-point tile: exponents of the E columns [npairs][ncol] (see eri_fixed.cuh)
     float* norm;  // fixed-point tile: their 1-norms per Hermite order [npairs][ncol][8]
+    float* box;   // fixed-point tile: smallest, largest coordinates of a pair's primitives [npairs][6]
     int2* limbs;  // fixed-point tile, bra: the E products as limbs [npairs][KS][T]
     int32_t* weak;  // fixed-point tile, bra: bits of the weakest order 0 of a pair's columns [npairs]
 };

@@ -192,6 +192,8 @@ struct FwdArgs {
     float fx_c, fx_imu;       // fixed-point tile: 2.42 / mu^2 and 1 / mu of the Hermite unit mu 2^sigma
     long long fx_rmu;         // and 2^62 / mu
     const int32_t* bra_ex;    // fixed-point tile: exponents of the bra's column norms [nbra][nab]
+    const float* bra_box;     // fixed-point tile: coordinates of the pairs' boxes [nbra][6]
+    const float* ket_box;     // [nket][6]
     const float* bra_norm;    // fixed-point tile: their 1-norms per Hermite order [nbra][nab][8]
     const int2* bra_limbs;    // fixed-point tile: the bra's E products as limbs [nbra][KB][Tab]
     const int32_t* bra_weak;  // fixed-point tile: bits of the weakest order 0 of a bra pair's columns [nbra]

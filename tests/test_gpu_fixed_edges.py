@@ -91,3 +91,30 @@ def test_tight_one_centre_pairs_against_diffuse_ones(cls, tight):
             eri.eri_set_forms(0)
         # a component: one rounding of each product and sum, twice that for sums of a few hundred terms
         assert _column_errors(fixed, ref).max() < max(2e-14, 2 * _column_errors(fp64, ref).max())
+
+
+@pytest.mark.parametrize("r", [4.0, 25.0, 90.0])
+@pytest.mark.parametrize("cls", [(1, 1, 1, 1), (2, 1, 1, 1), (2, 2, 2, 1)])
+def test_one_centre_pairs_at_a_distance(cls, r):
+    """Quartets of one-centre pairs, whose integrals are multipoles of any order: each component is as close as from
+    the FP64 tile at every distance.  (One side at the origin, the other at coordinates whose weighted means are exact:
+    elsewhere the rounding of a centre, 1e-16 of the coordinate, bounds both tiles.)"""
+    rng = np.random.default_rng(41)
+    n, m, nq = 6, 40, 10240
+    u = rng.normal(size=(m, 3))
+    far = np.round(8 * r * rng.uniform(1, 1.3, (m, 1)) * u / np.linalg.norm(u, axis=1, keepdims=True)) / 8
+    shells = sum((_shells([0] * n, l, [0.3 * np.array([1.0, 2.5]) * (1 + i / n) for i in range(n)], rng)
+                  for l in cls[:2]), [])
+    shells += sum((_shells(range(1, m + 1), l, [np.array([0.5, 0.5])] * m, rng) for l in cls[2:]), [])
+    basis = synth.basis_from_shells(np.concatenate([np.zeros((1, 3)), far]), shells)
+    i, j = np.arange(n), np.arange(m)
+    bra = np.stack([i, n + i], 1).astype(np.int32)
+    ket = np.stack([2 * n + j, 2 * n + m + j], 1).astype(np.int32)
+    q = np.stack([np.arange(nq) % n, np.arange(nq) // n % m], 1).astype(np.int64)
+    for forms in (1, 2):
+        eri.eri_set_forms(forms)
+        try:
+            fixed, fp64, ref = _both_tiles(cls, basis, bra, ket, q, n * m)
+        finally:
+            eri.eri_set_forms(0)
+        assert _column_errors(fixed, ref).max() < max(2e-14, 2 * _column_errors(fp64, ref).max())
