@@ -14,6 +14,7 @@ __constant__ double c_inv_odd[32] = {
 
 // 2 pi^(5/2), the constant of Eq. 0m
 constexpr double kTwoPi52 = 34.986836655249725693;
+constexpr double kTwoPi52Lo = 7.2256294425378e-16;  // 2 pi^(5/2) less its double
 // sqrt(pi)/2
 constexpr double kHalfSqrtPi = 0.88622692545275801365;
 

@@ -258,6 +258,27 @@ constexpr int64_t kPairWarpSlots = 8192;  // at most this many slots take a warp
 constexpr int kEax = (kLmax + 3) * (kLmax + 3) * (2 * kLmax + 5);  // per-axis E table bound (adjoint shifts)
 constexpr int kEfw = (kLmax + 1) * (kLmax + 1) * (2 * kLmax + 1);  // without the shifts (also the HRR form's)
 
+// c1 c2 k zeta^(-3/2) (times 2 pi^(5/2) on the bra), rounded once at the end: the
+// fixed-point tile takes its E products as they come, so the roundings of this
+// factor, two more than the FP64 tile's, would be most of its error.
+__device__ __forceinline__ double fix_e00(double c1, double c2, double k, double p, double invp, int ket)
+{
+    // products as unevaluated sums hi + lo
+    const double a = c1 * c2, al = fma(c1, c2, -a);
+    const double b = a * k, bl = fma(a, k, -b) + al * k;
+    const double s = sqrt(invp), sl = fma(-s, s, invp) * (0.5 / s);
+    double w = invp * s;
+    // (1/zeta)^(3/2) = invp^(3/2) (1 + 3/2 (1 - invp zeta))
+    double wl = fma(invp, s, -w) + invp * sl + 1.5 * w * fma(-invp, p, 1.0);
+    if (!ket) {
+        const double v = w * kTwoPi52;
+        wl = fma(w, kTwoPi52, -v) + (wl * kTwoPi52 + w * kTwoPi52Lo);
+        w = v;
+    }
+    const double r = b * w;
+    return r + (fma(b, w, -r) + (b * wl + bl * w));
+}
+
 // RAISED: the adjoint's tables (a.ax != NULL): the per-axis E tables with
 // both indices raised by 2, one thread per (slot, axis).  The adjoint reads
 // no E products of that side, so none are formed.  Otherwise one thread per
@@ -341,8 +362,10 @@ __global__ void __launch_bounds__(kPairThreads) pair_kernel_t(PairArgs a)
         // bra and 1 / zeta_q on the ket: every E of the pair (per-axis tables
         // and products alike) carries it once, and [0]^(m) needs only the
         // quartet's 1/sqrt(zeta_p + zeta_q).
-        double e00x = a.coefs[p1] * c2 * exp(-z1 * z2 * invp * AB2) * (a.ket ? invp : kTwoPi52 * invp);
-        if (!RAISED && a.fixed) e00x *= sqrt(invp);  // 1/sqrt(zeta_p + zeta_q) = sqrt(rho / (zeta_p zeta_q))
+        const double kab = exp(-z1 * z2 * invp * AB2);
+        // (fixed point: with zeta^(-1/2), 1/sqrt(zeta_p + zeta_q) = sqrt(rho / (zeta_p zeta_q)))
+        const double e00x = !RAISED && a.fixed ? fix_e00(a.coefs[p1], c2, kab, p, invp, a.ket)
+                                               : a.coefs[p1] * c2 * kab * (a.ket ? invp : kTwoPi52 * invp);
         const int ext = RAISED ? 2 : 0;
         // largest raised indices: the adjoint raises both by 2; the
         // horizontal-recursion form needs E_{i,0} for i <= l1 + l2

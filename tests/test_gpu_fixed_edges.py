@@ -1,11 +1,13 @@
 """The fixed-point tile of eri_batch where its scales are tight: one-centre
-quartets whose scale bound is attained, at powers of two."""
+quartets whose scale bound is attained at powers of two, tight pairs against
+diffuse ones, multipoles at a distance, and its error beside the FP64 tile's."""
 import numpy as np
 import pytest
 
+import oracle
 import paper_2506_12501_gb300 as eri
 import synth
-from gpu_helpers import assert_close, oracle_blocks, to_device
+from gpu_helpers import THREADS, assert_close, oracle_blocks, to_device
 
 pytestmark = pytest.mark.gpu
 
@@ -43,9 +45,15 @@ def test_one_centre_bounds_at_powers_of_two(N, cls):
 
 def _column_errors(got, ref):
     """Relative 2-norm error of every component quadruple over the quartets, where it is not zero by symmetry."""
-    top = np.linalg.norm(ref, axis=0)
+    top = np.sqrt((ref ** 2).sum(axis=0))
     on = top > 1e-40
-    return (np.linalg.norm(got - ref, axis=0)[on] / top[on])
+    return (np.sqrt(((got - ref) ** 2).sum(axis=0))[on] / top[on]).astype(float)
+
+
+def _reference(cls, basis, bra, ket, q):
+    """The long double oracle's blocks, in long double."""
+    ref = oracle.eri_quartets(basis, synth.quartet_shells(bra, ket, q), prec="ld", threads=THREADS)
+    return ref.reshape(len(q), -1)
 
 
 def _both_tiles(cls, basis, bra, ket, q, n):
@@ -60,7 +68,7 @@ def _both_tiles(cls, basis, bra, ket, q, n):
         finally:
             eri.eri_set_fixed(True)
         assert eri.eri_last_arithmetic() == (eri.ERI_ARITH_FIXED if fixed else eri.ERI_ARITH_FP64)
-    return out[0], out[1], oracle_blocks(cls, basis, bra, ket, q[:n], prec="ld")
+    return out[0], out[1], _reference(cls, basis, bra, ket, q[:n])
 
 
 @pytest.mark.parametrize("tight", [30.0, 2e3, 1e5])
@@ -118,3 +126,28 @@ def test_one_centre_pairs_at_a_distance(cls, r):
         finally:
             eri.eri_set_forms(0)
         assert _column_errors(fixed, ref).max() < max(2e-14, 2 * _column_errors(fp64, ref).max())
+
+
+@pytest.mark.parametrize("one_centre", [False, True])
+@pytest.mark.parametrize("cls,K", [((1, 0, 1, 0), 3), ((1, 1, 1, 1), 2), ((1, 1, 1, 1), 3), ((2, 1, 1, 1), 2),
+                                   ((2, 2, 1, 1), 2), ((2, 1, 2, 1), 2)])
+def test_error_no_larger_than_the_fp64_tile(cls, K, one_centre):
+    """Relative 2-norm error over a batch against the long double oracle, both tiles in the plain form.  The bound is
+    a tenth over 1 for the sample: the means of a few thousand roundings."""
+    rng = np.random.default_rng(51)
+    m, nq = 24, 10240
+    z = 0.2 * 3.0 ** np.arange(K)
+    shells = sum((_shells(range(m), l, [z] * m, rng) for l in cls), [])
+    basis = synth.basis_from_shells(rng.uniform(0, 4.0, (m, 3)), shells)
+    i, j = rng.integers(0, m, (2, 60)), rng.integers(0, m, (2, 60))
+    if one_centre:
+        i[1], j[1] = i[0], j[0]
+    bra, ket = (i.T + [0, m]).astype(np.int32), (j.T + [2 * m, 3 * m]).astype(np.int32)
+    q = rng.integers(0, 60, (nq, 2)).astype(np.int64)
+    eri.eri_set_forms(1)
+    try:
+        fixed, fp64, ref = _both_tiles(cls, basis, bra, ket, q, 400)
+    finally:
+        eri.eri_set_forms(0)
+    error = [float(np.sqrt(((x - ref) ** 2).sum())) for x in (fixed, fp64)]
+    assert error[0] <= 1.1 * error[1], error
