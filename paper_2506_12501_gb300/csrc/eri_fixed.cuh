@@ -58,9 +58,12 @@ namespace eri {
 constexpr float kFixSpreadBits = 6.0f;
 // Largest order the tile takes.  Above it one exponent for the integrals of all
 // orders costs more than the FP64 tile's roundings: relative 2-norm error against
-// the oracle, fixed point | FP64, K = 2, pairs of two centres in a 4-bohr cube:
-// (fd|fd), order 10, 2.8e-14 | 1.3e-15; (fd|dd), order 9, 1.2e-14 | 1.0e-15.
-constexpr int kFixLmax = 8;
+// the oracle, fixed point over FP64, plain form, K = 2 of ratio 3, pairs of two
+// centres in cubes of 1.5 | 4 | 8 bohr: (fd|pp), order 7, 3.4 | 2.1 | 1.2; (dd|dp), 7,
+// 2.3 | 1.6 | 1.1; (ff|pp), 8, 2.9 | 3.4 | 1.8; (dd|dd), 8, 1.6 | 1.9 | 1.2.  Order 6: (dp|dp) 0.97 |
+// 0.99 | 1.0, (dd|pp) 0.63 | 0.89 | 1.0; three primitives, the widest it takes, (dp|dp)
+// 1.5 | 1.1 | 1.0.  Order 5 and less: 0.6 to 1.02.
+constexpr int kFixLmax = 6;
 static_assert(kFixLmax <= kFixAuxLmax, "order of the fixed-point auxiliary integrals");
 // products per low-limb accumulator between folds: each below 2^28 2^31.  Even:
 // the ket transform reads its operands in aligned pairs from each multiple on.
@@ -68,7 +71,7 @@ constexpr int kFixFold = 14;
 static_assert(kFixFold % 2 == 0, "pairs of ket primitives stay 16-byte aligned");
 
 // T = rho r^2 from which the Hermite unit follows the distance: s r >= 1.1 sqrt(8) = 3.1,
-// at most twice that, keeps N! / (s r)^N between 2^-6 and 2^6 for N <= 8
+// at most twice that, keeps N! / (s r)^N between 2^-7 and 1 for N <= 6
 constexpr float kFixFarT = 4.0f;
 // bits a bra column may lose to the shift of X before its quartet forms the limbs itself
 constexpr int kFixWeakBits = 4;

@@ -17,7 +17,7 @@ def _shells(atoms, l, exps, rng):
             for a, z in zip(atoms, exps)]
 
 
-@pytest.mark.parametrize("N,cls", [(0, (1, 0, 1, 0)), (6, (2, 1, 2, 1)), (8, (2, 2, 2, 2))])
+@pytest.mark.parametrize("N,cls", [(0, (1, 0, 1, 0)), (6, (2, 1, 2, 1))])
 def test_one_centre_bounds_at_powers_of_two(N, cls):
     """One-centre quartets whose order-N integral at the largest exponents, (N-1)!!/(N+1) sqrt(rho) in units of
     s = 1.1 sqrt(2 rho), attains the scale's bound at a power of two, to the rounding of a float on either side."""
@@ -102,7 +102,7 @@ def test_tight_one_centre_pairs_against_diffuse_ones(cls, tight):
 
 
 @pytest.mark.parametrize("r", [4.0, 25.0, 90.0])
-@pytest.mark.parametrize("cls", [(1, 1, 1, 1), (2, 1, 1, 1), (2, 2, 2, 1)])
+@pytest.mark.parametrize("cls", [(1, 1, 1, 1), (2, 1, 1, 1), (2, 2, 2, 0)])
 def test_one_centre_pairs_at_a_distance(cls, r):
     """Quartets of one-centre pairs, whose integrals are multipoles of any order: each component is as close as from
     the FP64 tile at every distance.  (One side at the origin, the other at coordinates whose weighted means are exact:
