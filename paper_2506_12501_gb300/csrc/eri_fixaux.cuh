@@ -343,7 +343,7 @@ FIX_HD float fix_distance2(const FixPrim& p, const FixPrim& q, int f)
     return r2;
 }
 
-// Exponent g with |order N of the integrals| s^-N < 2^g for n_min <= N <= L, from the
+// Exponent g with |order N of the integrals| s^-N < 2^g for N <= L, from the
 // exponents and |X|^2: at any distance sqrt(rho) (2 rho)^(N/2) (N-1)!!/(N+1) (the
 // value at X = 0), and sqrt(pi)/2 N! / |X|^(N+1) up to a factor below 3.
 // At X = 0 that is no estimate but the value itself, so top is raised by
@@ -352,7 +352,7 @@ FIX_HD float fix_distance2(const FixPrim& p, const FixPrim& q, int f)
 // 5.5 and 10, with a rounding for each product: less than 2^-17 together.  Next to a
 // power of two a bound that fell short would take the limbs (2^62 - 2^30) past their end.
 constexpr float kFixBoundMargin = 1.0f + 0x1p-15f;
-FIX_HD int fix_bound(int L, int n_min, float rho, float r2, int sigma, float imu)
+FIX_HD int fix_bound(int L, float rho, float r2, int sigma, float imu)
 {
     const float is = fix_pow2(-sigma) * imu, ir = r2 > 1e-30f ? fix_rsqrt_seed(r2) : 1e15f;
     float near = rho * fix_rsqrt_seed(rho), far = 0.8863f * ir, top = 0.f;
@@ -362,10 +362,8 @@ FIX_HD int fix_bound(int L, int n_min, float rho, float r2, int sigma, float imu
         if (N > 0) far *= (float)N * rf;
         if (N > 0 && !(N & 1)) even *= (float)(N - 1) * rn;
         // an odd order stays below the larger of its neighbours
-        if (N >= n_min) {
-            const float nr = (N & 1) ? fmaxf(even / (float)N, even * (float)N * rn / (float)(N + 2)) : even / (float)(N + 1);
-            top = fmaxf(top, fminf(nr, 3.0f * far));
-        }
+        const float nr = (N & 1) ? fmaxf(even / (float)N, even * (float)N * rn / (float)(N + 2)) : even / (float)(N + 1);
+        top = fmaxf(top, fminf(nr, 3.0f * far));
     }
     top *= kFixBoundMargin;
     return top > 1e-37f ? (int)(fix_float_bits(top) >> 23) - 126 : -126;

@@ -313,7 +313,7 @@ struct alignas(16) FixStep {
 // time, all sources read before any is written (a lane alone takes four).
 // on: false for lanes without an item, which only keep the warp's barriers.
 __device__ __forceinline__ void fix_recursion(int L, const long long* F, const int (&x1)[3], const int (&x0s)[3],
-                                              const long long* phi, const int* sh, int n_min, const FixStep* st,
+                                              const long long* phi, const int* sh, const FixStep* st,
                                               const int16_t* ord, long long* R, int NIs, int G, int j, bool on)
 {
     const char* Rb = reinterpret_cast<const char*>(R);
@@ -344,7 +344,7 @@ __device__ __forceinline__ void fix_recursion(int L, const long long* F, const i
         }
         const int nhl = (L + 1) * (L + 2) * (L + 3) / 6;
         if (on)
-            for (int e = j + n_min * (n_min + 1) * (n_min + 2) / 6; e < nhl; e += G) {
+            for (int e = j; e < nhl; e += G) {
                 const int N = ord[e];
                 *reinterpret_cast<int2*>(&R[e * NIs]) = fix_limbs<kLimbR>(fix_finish(R[e * NIs], phi[N], sh[N]));
             }
@@ -369,9 +369,9 @@ __device__ __forceinline__ void fix_recursion(int L, const long long* F, const i
         for (; e >= 1; --e, Re -= NIs) *Re = step(st[e]);
         R[0] = F[n];
     }
-    int e = n_min * (n_min + 1) * (n_min + 2) / 6;
-    long long* Re = R + e * NIs;
-    for (int N = n_min; N <= L; ++N) {
+    int e = 0;
+    long long* Re = R;
+    for (int N = 0; N <= L; ++N) {
         const long long f = phi[N];
         const int s = sh[N];
         for (const int top = (N + 1) * (N + 2) * (N + 3) / 6; e < top; ++e, Re += NIs)
@@ -449,7 +449,7 @@ __device__ __forceinline__ void fix_recursion_c(const long long (&F)[L + 1], con
 template <int LMAX, int FIXED>
 __device__ __forceinline__ void fix_aux_item(int Lr, const FixPrim& p, const FixPrim& q, int f,
                                              const long long* __restrict__ tab, const long long* __restrict__ far,
-                                             int sigma, long long rmu, int g, int n_min, const FixStep* st, const int16_t* ord,
+                                             int sigma, long long rmu, int g, const FixStep* st, const int16_t* ord,
                                              long long* R, int NIs, int G, int j, bool on)
 {
     const int L = FIXED ? LMAX : Lr;
@@ -470,7 +470,7 @@ __device__ __forceinline__ void fix_aux_item(int Lr, const FixPrim& p, const Fix
         if constexpr (FIXED) {
             fix_recursion_c<LMAX>(F, x1, x0s, phi, sh, R, NIs);
         } else {
-            fix_recursion(L, F, x1, x0s, phi, sh, n_min, st, ord, R, NIs, G, j, on);
+            fix_recursion(L, F, x1, x0s, phi, sh, st, ord, R, NIs, G, j, on);
         }
     }
 }
@@ -654,9 +654,7 @@ __device__ void tile_fixed(const FwdArgs& a, int64_t q0, int nqt, double* sm, do
         const int64_t g = (int64_t)s_q[4 * q] * nab + ab;
         s_F[idx] = fix_norm_exp(a.bra_norm + 8 * g, a.bra_ex[g], -lo);
     }
-    // bounds of the auxiliary integrals the transforms read (a solid-harmonic
-    // side of order l reads none of order below l)
-    const int n_min = ct.pure == 1 ? ct.la : (ct.pure == 2 ? ct.lc : 0);
+    // bounds of the auxiliary integrals
     {
         const FastDiv d_bk(KBt * KKt);
         for (int idx = tid; idx < TQ * KBt * KKt; idx += NT) {
@@ -664,7 +662,7 @@ __device__ void tile_fixed(const FwdArgs& a, int64_t q0, int nqt, double* sm, do
             if (i >= s_q[4 * q + 2] || k >= s_q[4 * q + 3]) continue;
             const FixPrim &p = sPb[q * KB + i], &c = sPk[q * KK + k];
             const float r2 = fix_distance2(p, c, a.fx_f), rho = __fdividef(p.zeta * c.zeta, p.zeta + c.zeta);
-            atomicMax(&s_g[q * KB + i], fix_bound(ct.L, n_min, rho, r2, s_sig[q * KB + i], a.fx_imu));
+            atomicMax(&s_g[q * KB + i], fix_bound(ct.L, rho, r2, s_sig[q * KB + i], a.fx_imu));
         }
     }
     __syncthreads();
@@ -707,7 +705,7 @@ __device__ void tile_fixed(const FwdArgs& a, int64_t q0, int nqt, double* sm, do
         // ---- A: auxiliary integrals
         // (columns of primitives a quartet lacks keep whatever they hold: the E
         // products they meet are zero)
-        const bool regs = !n_min && ct.L <= kFixRegL;
+        const bool regs = ct.L <= kFixRegL;
         // lanes per item: as many as put every thread to work, up to four (each
         // lane repeats the item's base), or more where a warp would hold few items
         const int fill = max(1, NT / NIt);
@@ -724,7 +722,7 @@ __device__ void tile_fixed(const FwdArgs& a, int64_t q0, int nqt, double* sm, do
             const int sg = s_sig[q * KB + i], g = s_g[q * KB + i];
             auto run = [&](auto lmax, auto fixed) {
                 fix_aux_item<decltype(lmax)::value, decltype(fixed)::value>(
-                    ct.L, sPb[q * KB + i], sPk[q * KK + k], a.fx_f, a.fx_tab, a.fx_far, sg, a.fx_rmu, g, n_min, tb.st, tb.ord, R,
+                    ct.L, sPb[q * KB + i], sPk[q * KK + k], a.fx_f, a.fx_tab, a.fx_far, sg, a.fx_rmu, g, tb.st, tb.ord, R,
                     NIs, G, lane & (G - 1), on);
             };
             switch (regs ? ct.L : -1) {

@@ -663,7 +663,7 @@ static void add_e_ring(const ClassTables& ct, int KK, TilePlan* tp)
 // by the threads that do, but at least a third of it (one warp's latency); chunks
 // and tiles add their barriers and set-up.  The units are rough figures of the
 // stages timed on (pp|ps) and (dd|dd).
-static bool plan_fixed_tile(const ClassTables& ct, int KB, int KK, int64_t nq, TilePlan* best, size_t max_bytes)
+static bool plan_fixed_tile(const ClassTables& ct, int KB, int KK, int64_t nq, TilePlan* best)
 {
     bool found = false;
     double best_time = 0.0;
@@ -671,11 +671,10 @@ static bool plan_fixed_tile(const ClassTables& ct, int KB, int KK, int64_t nq, T
     const double unit_a = ct.L <= 4 ? unit_a_low[ct.L] : 12.0 * ct.nhl * ct.L;
     const double unit_b = 150 + 24.0 * KK * ct.Tcd / ct.ncd, unit_c = 150;
     for (int nt : {kNTSlim, kNT, kNTWide}) {
-        if (max_bytes && nt != kNT) continue;  // plans launch kNT threads
         for (int TQ = 1; TQ <= 128 && (TQ == 1 || TQ < 2 * nq); TQ *= 2)
             for (int IC : {KB, (KB + 1) / 2, (KB + 2) / 3, 1}) {
                 TilePlan tp;
-                if (!tile_layout(ct, KB, KK, TQ, IC, 1, &tp, XF_FIXED, nt) || (max_bytes && tp.bytes > max_bytes)) continue;
+                if (!tile_layout(ct, KB, KK, TQ, IC, 1, &tp, XF_FIXED, nt)) continue;
                 const int64_t tiles = (nq + TQ - 1) / TQ;
                 int64_t per_sm = std::min<int64_t>(kNTWide / nt, (int64_t)smem_per_sm() / (int64_t)(tp.bytes + 1088));
                 if (per_sm < 1) continue;
@@ -701,7 +700,7 @@ static bool plan_fixed_tile(const ClassTables& ct, int KB, int KK, int64_t nq, T
 
 bool plan_tiles(const ClassTables& ct, int KB, int KK, int64_t nq, TilePlan* best, size_t max_bytes, int split)
 {
-    if (split == XF_FIXED) return plan_fixed_tile(ct, KB, KK, nq, best, max_bytes);
+    if (split == XF_FIXED) return plan_fixed_tile(ct, KB, KK, nq, best);
     bool found = false;
     double best_score = -1.0;
     for (int e_smem = 1; e_smem >= 0; --e_smem) {

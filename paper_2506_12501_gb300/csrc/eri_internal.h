@@ -227,7 +227,7 @@ struct TilePlan {
 // The arithmetic of a tile's transforms: FP64, split precision, or (the
 // caller asked for FP64) 64-bit fixed point.
 enum { XF_FP64 = 0, XF_SPLIT = 1, XF_FIXED = 2 };
-// max_bytes > 0: only shapes whose shared memory stays within it; split: the
+// max_bytes > 0: only shapes whose shared memory stays within it (not for XF_FIXED); split: the
 // transforms' arithmetic (XF_*)
 bool plan_tiles(const ClassTables& ct, int KB, int KK, int64_t nq, TilePlan* best, size_t max_bytes = 0,
                 int split = 0);

@@ -88,7 +88,7 @@ int main() {
             if (L == 0) B.U = 1LL << 61, B.ue = 0;
             const double mu = 1.37;
             const int sigma = ((int)floor(log2(2.42 / (mu * mu) * rho)) + 2) >> 1;
-            const int gg = fix_bound(L, 0, (float)rho, (float)R2, sigma, (float)(1 / mu));
+            const int gg = fix_bound(L, (float)rho, (float)R2, sigma, (float)(1 / mu));
             fix_factors<10>(L, B, sigma, (long long)(0x1p62L / (Q)mu), gg, phi, sh);
             std::vector<long long> R(nh);
             int x1[3], x0[3];

@@ -51,7 +51,7 @@ int main() {
             const int sigma = (ilogb(2.42 / (mu * mu) * rho) + 2) >> 1;
             // the device's approximate division may leave rho below its value
             const float fr = (float)rho * (1 - (float)uni(0, 0x1p-21));
-            const int gg = fix_bound(L, 0, fr, fix_distance2(p, q, 50), sigma, (float)(1 / mu));
+            const int gg = fix_bound(L, fr, fix_distance2(p, q, 50), sigma, (float)(1 / mu));
             long long F[11], phi[11];
             int sh[11];
             FixBase B;
@@ -90,7 +90,7 @@ int main() {
         }
         const double mu = uni(1, 2);
         const int sigma = (ilogb(2.42 / (mu * mu) * rho) + 2) / 2 - (int)(g() % 6);
-        const int gg = fix_bound(L, 0, (float)rho, (float)(r * r), sigma, (float)(1 / mu));
+        const int gg = fix_bound(L, (float)rho, (float)(r * r), sigma, (float)(1 / mu));
         for (int N = 0; N <= L; ++N)
             worst = std::max(worst, fabs((double)(sqrtl(rho) * R[N] * powl(mu * powl(2, sigma), -N) * powl(2, -gg))));
     }
