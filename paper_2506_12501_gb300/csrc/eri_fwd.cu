@@ -963,6 +963,7 @@ int prepare_batch(eri_class_t cls, const eri_basis_t* basis, const int32_t* bra,
     *KK = kmax[2] * kmax[3];
     if (mixed) *mixed = (INT_MAX - hinfo[7] < *KB || INT_MAX - hinfo[8] < *KK) ? 1 : 0;
     const bool fix_ok = try_fixed && (int64_t)*KB * *KK >= 4 && nqq * *KB * *KK >= 150000 && fixed_eligible(cls, hinfo + 9);
+    const int key = fix_ok ? XF_FIXED : split;
     if (allow_swap) {
         // Four forms: which side is transformed first (Section 3.2.2
         // transforms the ket first, assuming it has the lower l) and whether
@@ -997,8 +998,10 @@ int prepare_batch(eri_class_t cls, const eri_basis_t* basis, const int32_t* bra,
                 if (c->nab * c->ncd > kNT * kNACC || !plan_tiles(*c, (int)kb, (int)kk, nqq, &tp)) continue;
             }
             // a recursion step is an FP64 operation, which costs several
-            // products of the fixed-point transforms
-            const double step = fix_ok ? 6.0 : 1.0;
+            // products of the fixed-point transforms (where the smallest tile fits)
+            TilePlan least;
+            const bool fits = fix_ok && tile_layout(*c, (int)kb, (int)kk, 1, 1, 1, &least, XF_FIXED, kNTSlim);
+            const double step = fits ? 6.0 : 1.0;
             cost[o] = kb * kk * ((c->nhb - c->pb0) * c->Tcd + 0.5 * c->nhl) + kb * c->ncd * c->Tab +
                       (c->hrr ? step * (c->nab * c->nks + c->ncd_f * c->nbs) : 0);
         }
@@ -1022,7 +1025,7 @@ int prepare_batch(eri_class_t cls, const eri_basis_t* basis, const int32_t* bra,
             if (forced > 3 || cost[forced] < 0) return ERI_EINVAL;
             best = forced;
         } else {
-            best = lookup_form(cls, *KB, *KK, fix_ok ? XF_FIXED : split, kind);
+            best = lookup_form(cls, *KB, *KK, key, kind);
             if (best >= 0 && cost[best] >= 0) {
                 if (fc) fc->cached = 1;
             } else {
@@ -1059,6 +1062,7 @@ int prepare_batch(eri_class_t cls, const eri_basis_t* basis, const int32_t* bra,
         mu = fix_unit((double)zb * zk / ((double)zb + zk));
     }
     if (fc) {
+        fc->key = key;
         fc->fixed = fixed;
         fc->fx_f = fx_f;
         fc->mu = mu;
@@ -1578,7 +1582,7 @@ static int run_forward(eri_class_t cls, const eri_basis_t* basis, const int32_t*
             // its recursion form 3.7e-15); (dp|dp) K = 2, 50000, 3.30 against 3.77 ms stays.
             auto weight = [](const FormChoice& f) { return f.fixed && f.form >= 2 ? 1.1f : 1.0f; };
             const bool take_alt = tuned1 && (!tuned || weight(f1) * ms1 < weight(fc) * ms);
-            remember_form(sig, KB0, KK0, fc.fixed || f1.fixed ? XF_FIXED : split, kind, take_alt ? f1.form : fc.form);
+            remember_form(sig, KB0, KK0, fc.key, kind, take_alt ? f1.form : fc.form);
             if (take_alt) {
                 fc = f1;
                 a = a1;

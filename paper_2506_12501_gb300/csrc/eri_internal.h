@@ -169,6 +169,8 @@ struct FormChoice {
     int form = -1;    // in: a form to force, or -1 (remembered, else modelled); out: the form used
     int alt = -1;     // out: the modelled-cheapest feasible form of the other kind (plain vs HRR), or -1
     int cached = 0;   // out: 1 when the form was remembered from an earlier timing
+    int key = 0;      // out: the arithmetic (XF_*) the form is remembered under: what the class may take,
+                      // whichever tile the form's shared memory then allows
     int fixed = 0;    // out: 1 when the pair tables are those of the fixed-point tile
     int fx_f = 0;     // out: their coordinates are in units of 2^-fx_f
     double mu = 1.0;  // out: and their Hermite unit (eri_fixed.cuh)

@@ -254,3 +254,37 @@ def test_contraction_degree_limits(cuda, cls, K):
         with pytest.raises(eri.EriError) as e:
             gpu_list(cls, basis, bra, ket, q, precision=prec)
         assert e.value.code == eri.ERI_EINVAL
+
+
+def test_form_choice_is_remembered_whatever_tile_runs():
+    """A contracted class of order 11, whose exponents lie close together: from the second long batch on, the call
+    launches what a call with that form alone launches (no further pair tables, checking passes or timings)."""
+    cls, nq = (3, 3, 3, 2), 16384
+    rng = np.random.default_rng(61)
+    shells, m = [], 12
+    for l in cls:
+        for a in range(m):
+            z = 0.5 * np.array([1.0, 2.0])
+            shells.append((a, l, list(z), list(rng.uniform(0.5, 1, 2) * synth.norm_coef(z, l))))
+    basis = synth.basis_from_shells(rng.uniform(0, 3.0, (m, 3)), shells)
+    i = np.arange(m)  # one-centre pairs: the recursion forms are candidates
+    bra, ket = np.stack([i, m + i], 1).astype(np.int32), np.stack([2 * m + i, 3 * m + i], 1).astype(np.int32)
+    q = rng.integers(0, m, (nq, 2)).astype(np.int64)
+    b, k, qq = to_device(bra, ket, q)
+    db = eri.DeviceBasis(basis)
+
+    def launches():
+        n = eri.eri_launch_count()
+        eri.eri_batch(cls, db, b, k, qq)
+        return eri.eri_launch_count() - n
+
+    launches()
+    swapped, hrr = eri.eri_last_form()
+    again = launches()
+    eri.eri_set_forms(1 << (int(swapped) + 2 * int(hrr)))
+    try:
+        launches()
+        alone = launches()
+    finally:
+        eri.eri_set_forms(0)
+    assert again == alone
