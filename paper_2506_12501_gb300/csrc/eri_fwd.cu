@@ -1049,7 +1049,12 @@ int prepare_batch(eri_class_t cls, const eri_basis_t* basis, const int32_t* bra,
     }
     // the fixed-point tile where its precision and its shared memory allow
     TilePlan fix_tile;
-    const bool fixed = fix_ok && plan_tiles(*ct, *KB, *KK, nqq, &fix_tile, 0, XF_FIXED);
+    bool fixed = fix_ok && plan_tiles(*ct, *KB, *KK, nqq, &fix_tile, 0, XF_FIXED);
+    if (fixed && !get_fix_boys_table(ct->L, st, &err)) {
+        if (err != ERI_ENOMEM) return err;
+        fixed = false;  // the FP64 tile needs less memory
+        err = ERI_OK;
+    }
     int fx_f = 0;
     double mu = 1.0;
     if (fixed) {  // |coordinate| 2^fx_f < 2^60
@@ -1061,36 +1066,49 @@ int prepare_batch(eri_class_t cls, const eri_basis_t* basis, const int32_t* bra,
         std::memcpy(&zk, &hinfo[14], 4);
         mu = fix_unit((double)zb * zk / ((double)zb + zk));
     }
-    if (fc) {
-        fc->key = key;
-        fc->fixed = fixed;
-        fc->fx_f = fx_f;
-        fc->mu = mu;
-    }
-    // workspace: pair tables of both sides
-    const size_t ps_n = fixed ? sizeof(FixPrim) / 8 : PS_N;
-    const size_t nb_ps = align_up(sizeof(double) * nbra * *KB * ps_n), nb_E = align_up(sizeof(double) * nbra * *KB * ct->Tab);
-    const size_t nk_ps = align_up(sizeof(double) * nket * *KK * ps_n), nk_E = align_up(sizeof(double) * nket * *KK * ct->Tcd);
-    const size_t nb_k = align_up(sizeof(int32_t) * nbra), nk_k = align_up(sizeof(int32_t) * nket);
+    // workspace: pair tables of both sides.
     // ldelta 1: the raised tables of the kernel bra only (the adjoint launch
     // for one side's channels); 2: of both sides, with the E products of
     // both (the adjoint launch for every channel)
     const int grad = ldelta > 0, grad_both = ldelta > 1;
     const int eaxb = (cls.la + 3) * (cls.lb + 3) * (cls.la + cls.lb + 5);
     const int eaxk = (cls.lc + 3) * (cls.ld + 3) * (cls.lc + cls.ld + 5);
+    const size_t nb_E = align_up(sizeof(double) * nbra * *KB * ct->Tab);
+    const size_t nk_E = align_up(sizeof(double) * nket * *KK * ct->Tcd);
+    const size_t nb_k = align_up(sizeof(int32_t) * nbra), nk_k = align_up(sizeof(int32_t) * nket);
     const size_t nb_ax = grad ? align_up(sizeof(double) * nbra * *KB * 3 * eaxb) : 0;
     const size_t nk_ax = grad_both ? align_up(sizeof(double) * nket * *KK * 3 * eaxk) : 0;
     const size_t nb_z = grad ? align_up(sizeof(double) * nbra * *KB * 2) : 0;
     const size_t nk_z = grad_both ? align_up(sizeof(double) * nket * *KK * 2) : 0;
-    const size_t nb_x = fixed ? align_up(sizeof(int32_t) * nbra * ct->nab) : 0;
-    const size_t nk_x = fixed ? align_up(sizeof(int32_t) * nket * ct->ncd) : 0;
-    const size_t nk_n = fixed ? align_up(sizeof(float) * 8 * nket * ct->ncd) : 0;
-    const size_t nb_n = fixed ? align_up(sizeof(float) * 8 * nbra * ct->nab) : 0;
-    const size_t nb_b = fixed ? align_up(sizeof(float) * 6 * nbra) : 0, nk_b = fixed ? align_up(sizeof(float) * 6 * nket) : 0;
-    const size_t nb_l = fixed ? nb_E : 0, nb_w = fixed ? align_up(sizeof(int32_t) * nbra) : 0;
     const size_t n_grad = nb_ax + nk_ax + nb_z + nk_z;
-    uint8_t* ws = (uint8_t*)workspace(nb_ps + nb_E + nk_ps + nk_E + nb_k + nk_k + n_grad + nb_x + nk_x + nk_n + nb_n + nb_l + nb_w + nb_b + nk_b, &err);
+    size_t nb_ps, nk_ps, nb_x, nk_x, nk_n, nb_n, nb_b, nk_b, nb_l, nb_w;
+    auto total = [&]() {
+        const size_t ps_n = fixed ? sizeof(FixPrim) / 8 : PS_N, on = fixed;
+        nb_ps = align_up(sizeof(double) * nbra * *KB * ps_n);
+        nk_ps = align_up(sizeof(double) * nket * *KK * ps_n);
+        nb_x = on * align_up(sizeof(int32_t) * nbra * ct->nab);
+        nk_x = on * align_up(sizeof(int32_t) * nket * ct->ncd);
+        nk_n = on * align_up(sizeof(float) * 8 * nket * ct->ncd);
+        nb_n = on * align_up(sizeof(float) * 8 * nbra * ct->nab);
+        nb_b = on * align_up(sizeof(float) * 6 * nbra);
+        nk_b = on * align_up(sizeof(float) * 6 * nket);
+        nb_l = on * nb_E;
+        nb_w = on * align_up(sizeof(int32_t) * nbra);
+        return nb_ps + nb_E + nk_ps + nk_E + nb_k + nk_k + n_grad + nb_x + nk_x + nk_n + nb_n + nb_l + nb_w + nb_b + nk_b;
+    };
+    uint8_t* ws = (uint8_t*)workspace(total(), &err);
+    if (!ws && fixed && err == ERI_ENOMEM) {
+        fixed = false;  // no limbs, norms and boxes: what the FP64 tile needs
+        err = ERI_OK;
+        ws = (uint8_t*)workspace(total(), &err);
+    }
     if (!ws) return err;
+    if (fc) {
+        fc->key = key;
+        fc->fixed = fixed;
+        fc->fx_f = fx_f;
+        fc->mu = mu;
+    }
     {
         uint8_t* g0 = ws + nb_ps + nb_E + nk_ps + nk_E + nb_k + nk_k;
         pb->ax = grad ? (double*)g0 : nullptr;

@@ -8,7 +8,7 @@
 #include <array>
 #include <map>
 #include <mutex>
-#include <system_error>
+#include <new>
 #include <thread>
 #include <tuple>
 #include <vector>
@@ -633,10 +633,17 @@ const int64_t* get_fix_boys_table(int L, cudaStream_t s, int* err)
     if (it != g_boys_tabs.end()) return reinterpret_cast<const int64_t*>(it->second);
     const int words = fix_boys_words(L);
     const size_t n = (size_t)kFixBoysRows * words + kFixFarWords;
-    std::vector<int64_t> tab(n, 0);
     // (long double is software on some hosts: the rows are shared out)
     const int nt = std::max(1, std::min(16, (int)std::thread::hardware_concurrency()));
+    std::vector<int64_t> tab;
     std::vector<std::thread> pool;
+    try {
+        tab.assign(n, 0);
+        pool.reserve(nt);
+    } catch (const std::bad_alloc&) {
+        *err = ERI_ENOMEM;
+        return nullptr;
+    }
     auto rows = [&](int t) {
         for (int j = t; j < kFixBoysRows; j += nt)
             fix_boys_row(g_master_host.data(), L, j, tab.data() + (size_t)j * words);
@@ -644,8 +651,8 @@ const int64_t* get_fix_boys_table(int L, cudaStream_t s, int* err)
     for (int t = 1; t < nt; ++t) {
         try {
             pool.emplace_back(rows, t);
-        } catch (const std::system_error&) {
-            rows(t);  // no further thread to be had
+        } catch (const std::exception&) {
+            rows(t);  // no further thread (or its state) to be had
         }
     }
     rows(0);
@@ -653,6 +660,7 @@ const int64_t* get_fix_boys_table(int L, cudaStream_t s, int* err)
     fix_far_constants(L, tab.data() + (size_t)kFixBoysRows * words);
     double* d = nullptr;
     if (cudaMalloc(&d, n * 8) != cudaSuccess) {
+        cudaGetLastError();
         *err = ERI_ENOMEM;
         return nullptr;
     }

@@ -2,6 +2,10 @@
 batches) against the oracle: ket primitive counts on both sides of the folds
 and pairs of its sums, mixed contraction degrees, every order of the auxiliary
 integrals it takes, both list forms and the solid-harmonic output."""
+import os
+import subprocess
+import sys
+
 import numpy as np
 import pytest
 import torch
@@ -163,3 +167,50 @@ def test_callers_choice_of_the_fp64_tile():
         assert eri.eri_set_fixed(True) is False
     assert_close(fixed, fp64, what="fixed point against FP64")
     assert not np.array_equal(fixed, fp64)
+
+
+# in a process of its own: the library keeps its tables and workspace
+_MEMORY = """
+import sys
+import numpy as np
+import torch
+import paper_2506_12501_gb300 as eri
+import synth
+from gpu_helpers import assert_close, nc, oracle_blocks, to_device
+
+npairs, leave = int(sys.argv[1]), int(sys.argv[2])
+cls, K, nq = (2, 1, 1, 0), 3, 10240
+basis, pools = synth.class_sweep_pools(seed=17, lmax=2, pool=32, K=K, cube=4.0,
+                                       exps_fn=lambda rng, K: 0.3 * 1.5 ** np.arange(K))
+bra, ket, q = synth.class_sweep_batch(pools, cls, seed=18, npairs=64, nq=nq)
+b, k, qq = to_device(np.tile(bra, (npairs // 64, 1)), ket, q)
+db = eri.DeviceBasis(basis)
+out = torch.empty(nq * nc(2) * nc(1) * nc(1), dtype=torch.float64, device="cuda")
+eri.eri_set_forms(1)
+if leave < 1 << 30:  # the FP64 tile's tables are there already
+    eri.eri_set_fixed(False)
+    eri.eri_batch(cls, db, b, k, qq, out=out)
+    eri.eri_set_fixed(True)
+torch.cuda.synchronize()
+held = torch.empty(torch.cuda.mem_get_info()[0] - leave, dtype=torch.uint8, device="cuda")
+eri.eri_batch(cls, db, b, k, qq, out=out)
+assert eri.eri_last_arithmetic() == eri.ERI_ARITH_FP64
+del held
+torch.cuda.empty_cache()
+got = out.cpu().numpy().reshape(-1, nq).T
+eri.eri_batch(cls, db, b, k, qq, out=out)
+assert eri.eri_last_arithmetic() == eri.ERI_ARITH_FIXED
+assert_close(out.cpu().numpy().reshape(-1, nq).T, got)
+assert_close(got[:16], oracle_blocks(cls, basis, bra, ket, q[:16]))
+print("memory: ok")
+"""
+
+
+@pytest.mark.parametrize("what,npairs,leave", [("Boys rows", 64, 6 << 20), ("pair tables", 260_032, 4 << 30)])
+def test_memory_for_the_fp64_tile_is_enough(what, npairs, leave):
+    """Where the fixed-point tile's tables find no memory, the batch runs on the FP64 tile, which needs less."""
+    root = os.path.dirname(os.path.dirname(os.path.abspath(__file__)))
+    env = dict(os.environ, PYTHONPATH=os.pathsep.join([root, os.path.join(root, "tests")]))
+    r = subprocess.run([sys.executable, "-c", _MEMORY, str(npairs), str(leave)], cwd=root, env=env,
+                       capture_output=True, text=True, timeout=300)
+    assert "memory: ok" in r.stdout, what + r.stderr[-2000:]
