@@ -422,11 +422,18 @@ enum {
 int eri_last_arithmetic(int32_t* arithmetic);
 
 /*
- * eri_set_fixed -- whether later ERI_PREC_FP64 batches of the CALLING THREAD
- * may take the fixed-point tile (1, a thread's start) or keep to the FP64
- * tile (0).  Returns the previous value, or ERI_EINVAL for another argument.
+ * eri_set_fixed -- when later ERI_PREC_FP64 batches of the CALLING THREAD
+ * take the fixed-point tile: never, where it is expected to be the faster one
+ * (a thread's start), or wherever its precision allows (contracted or not,
+ * of any length; for tests and measurements).  Returns the previous mode, or
+ * ERI_EINVAL for another argument.
  */
-int eri_set_fixed(int32_t allowed);
+enum {
+    ERI_FIXED_NEVER = 0,
+    ERI_FIXED_RULE = 1,
+    ERI_FIXED_ALWAYS = 2
+};
+int eri_set_fixed(int32_t mode);
 
 /*
  * eri_set_forms -- restrict the forms later eri_batch calls (all threads)

@@ -51,6 +51,7 @@ ERI_NOALLOC_SCRATCH_BYTES = 64 * 1024 * 1024
 ERI_PLAN_STORE, ERI_PLAN_SPLIT, ERI_PLAN_NO_TUNE = 1, 2, 4
 ERI_FORM_PLAIN, ERI_FORM_HRR = 0x3, 0xC
 ERI_ARITH_FP64, ERI_ARITH_SPLIT, ERI_ARITH_FIXED = 0, 1, 2
+ERI_FIXED_NEVER, ERI_FIXED_RULE, ERI_FIXED_ALWAYS = 0, 1, 2
 ERI_GRAD_X, ERI_GRAD_V, ERI_GRAD_ONE, ERI_GRAD_TWO, ERI_GRAD_ONE_SWAPPED = 0, 1, 2, 3, 4
 PROF_FWD, PROF_GRAD, PROF_PAIR, PROF_PREPASS = 0, 1, 2, 3
 
@@ -345,12 +346,13 @@ def eri_last_arithmetic() -> int:
     return v.value
 
 
-def eri_set_fixed(allowed: bool) -> bool:
-    """Whether this thread's FP64-precision batches may take the fixed-point tile; returns the previous setting."""
-    code = lib().eri_set_fixed(int(allowed))
+def eri_set_fixed(mode: int) -> int:
+    """When this thread's FP64-precision batches take the fixed-point tile: ERI_FIXED_NEVER, ERI_FIXED_RULE (where it
+    is expected to be faster) or ERI_FIXED_ALWAYS (wherever its precision allows); returns the previous mode."""
+    code = lib().eri_set_fixed(int(mode))
     if code < 0:
         _check(code, "eri_set_fixed")
-    return bool(code)
+    return code
 
 
 def eri_set_grad_forms(mask: int) -> int:

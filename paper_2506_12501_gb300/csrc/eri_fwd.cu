@@ -663,7 +663,7 @@ static void add_e_ring(const ClassTables& ct, int KK, TilePlan* tp)
 // by the threads that do, but at least a third of it (one warp's latency); chunks
 // and tiles add their barriers and set-up.  The units are rough figures of the
 // stages timed on (pp|ps) and (dd|dd).
-static bool plan_fixed_tile(const ClassTables& ct, int KB, int KK, int64_t nq, TilePlan* best)
+static bool plan_fixed_tile(const ClassTables& ct, int KB, int KK, int64_t nq, TilePlan* best, double* time_out = nullptr)
 {
     bool found = false;
     double best_time = 0.0;
@@ -695,6 +695,7 @@ static bool plan_fixed_tile(const ClassTables& ct, int KB, int KK, int64_t nq, T
                 }
             }
     }
+    if (found && time_out) *time_out = best_time;
     return found;
 }
 
@@ -750,7 +751,8 @@ bool plan_tiles(const ClassTables& ct, int KB, int KK, int64_t nq, TilePlan* bes
 // (pp|pp) K = 1, 50 / 1000 / 12000 quartets 140 / 145 / 211 -> 63 / 66 / 152; (ps|ps)
 // K = 3, 50 / 1000 quartets 208 / 233 -> 77 / 89; (dd|dd) K = 3, 50 / 1000 quartets
 // 1305 / 2377 -> 379 / 2140 (with the faster pair tables and checking pass).
-static void plan_small_tile(const ClassTables& ct, int KB, int KK, int64_t nq, TilePlan* best)
+// Returns the modelled time of *best.
+static double plan_small_tile(const ClassTables& ct, int KB, int KK, int64_t nq, TilePlan* best)
 {
     auto warps = [](double items) { return std::ceil(items / 32); };
     const int L = ct.L;
@@ -766,7 +768,9 @@ static void plan_small_tile(const ClassTables& ct, int KB, int KK, int64_t nq, T
         const int chunks = (KB + tp.IC - 1) / tp.IC;
         return (double)((per_sm + res - 1) / res) * (5000 + chunks * (800 + a) + KB * (1000 + b + c));
     };
-    double best_time = 0.9 * model(*best);
+    const double planned = model(*best);
+    double best_time = 0.9 * planned;
+    bool other = false;
     for (int TQ = 1; TQ <= 128 && (TQ == 1 || TQ < 2 * nq); TQ *= 2) {
         if (TQ > 1 && TQ * ct.nab * ct.ncd > kNT * kNACC) break;
         for (int IC = KB, next; IC >= 1; IC = next) {  // KB, half of it, 1
@@ -777,9 +781,11 @@ static void plan_small_tile(const ClassTables& ct, int KB, int KK, int64_t nq, T
             if (t < best_time) {
                 best_time = t;
                 *best = tp;
+                other = true;
             }
         }
     }
+    return other ? best_time : planned;
 }
 
 static int dev_err_to_code(int e)
@@ -847,6 +853,22 @@ static void launch_fix_pairs(const PairTables& t, const ClassTables& ct, int64_t
     fix_pairs_kernel<<<(int)std::max<int64_t>(1, std::min<int64_t>((n + 127) / 128, 16LL * sm_count())), 128, 0, st>>>(f);
 }
 
+// A batch too small to be timed takes the fixed-point tile from this many
+// primitive quartets a quartet on: K = 2 (16), 16383 quartets, us, FP64 against
+// fixed point: (ps|ss) 114 / 154, (pp|ps) 242 / 289, (dp|dp) 1570 / 2280.
+constexpr int kFixSmallPrims = 81;
+// And where its modelled time (plan_fixed_tile; rough clocks that a stage's
+// threads share) and that of its pair tables' second pass (setup: terms of a
+// column times primitives) stay below the FP64 tile's (plan_small_tile; clocks).
+// Fitted to 23 classes of K = 3, 4 and 5 with 2000 to 16383 quartets: what it lets in
+// measured 0.3 to 1.03 times the FP64 call, e.g. (pp|pp) K = 3, 8000 quartets 876 us / 530,
+// (dp|pp) K = 3, 4000, 895 / 772; what it keeps out up to 1.6: (dd|ss) K = 3, 2000, 314 / 507,
+// (ps|ss) K = 3, 2000, 106 / 145, (ff|ss) K = 4, 4000, 3840 / 5258.
+static bool fix_small_faster(int L, double fix_time, double setup, double fp64_time)
+{
+    return (L >= 5 ? 14.0 : 11.0) * fix_time + 75e3 + 1800.0 * setup < fp64_time;
+}
+
 // Prepass + pair tables shared by the forward and adjoint entry points.
 // On success fills the pair tables and the largest K on each centre.
 // Largest product of bra and ket recursion risks for which the recursion
@@ -856,8 +878,10 @@ constexpr double kRecursionRisk = 900.0;
 // Forms eri_batch may use (eri_set_forms): bit o allows form o.
 static std::atomic<int> g_form_mask{0xF};
 
-// Whether the calling thread's batches may take the fixed-point tile (eri_set_fixed).
-static thread_local int g_allow_fixed = 1;
+// When the calling thread's batches take the fixed-point tile (eri_set_fixed).
+static thread_local int g_fixed_mode = ERI_FIXED_RULE;
+// Batches of at least this many quartets time their tile shapes and forms.
+constexpr int64_t kTuneMinQuartets = 16384;
 
 // Forms chosen by timing, per (device, class, K_bra, K_ket, precision).
 static std::map<std::tuple<int, int, int, int, int, int, int, int, int>, int> g_forms;
@@ -876,6 +900,23 @@ static int lookup_form(eri_class_t cls, int KB, int KK, int split, int kind)
     std::lock_guard<std::mutex> lk(g_forms_mu);
     auto it = g_forms.find(form_key(cls, KB, KK, split, kind));
     return it == g_forms.end() ? -1 : it->second;
+}
+
+// Whether the FP64 tile was timed faster than the fixed-point one, by the same key
+// (arithmetic XF_FIXED); nothing where they were not compared.
+static std::map<std::tuple<int, int, int, int, int, int, int, int, int>, bool> g_fp64_faster;
+
+static int lookup_fp64_faster(eri_class_t cls, int KB, int KK, int kind)  // 1, 0, or -1: not compared
+{
+    std::lock_guard<std::mutex> lk(g_forms_mu);
+    auto it = g_fp64_faster.find(form_key(cls, KB, KK, XF_FIXED, kind));
+    return it == g_fp64_faster.end() ? -1 : (int)it->second;
+}
+
+static void remember_fp64_faster(eri_class_t cls, int KB, int KK, int kind, bool faster)
+{
+    std::lock_guard<std::mutex> lk(g_forms_mu);
+    g_fp64_faster[form_key(cls, KB, KK, XF_FIXED, kind)] = faster;
 }
 
 void remember_form(eri_class_t cls, int KB, int KK, int split, int kind, int form)
@@ -917,20 +958,19 @@ int prepare_batch(eri_class_t cls, const eri_basis_t* basis, const int32_t* bra,
     int* dinfo = status + 8;
     // (one call: a small batch is bound by its launches, about 2 us each)
     if (cudaMemsetAsync(dinfo, 0, 15 * sizeof(int), st) != cudaSuccess) return ERI_ECUDA;
-    // Where the fixed-point tile is the faster one (GB300, ms, FP64 against fixed
-    // point): contracted 4-centre classes above (ss|ss): (pp|ps) K = 3, 1e5
-    // quartets 3.50 / 2.19; (ds|ds) 6.76 / 3.70; (dp|pp), 6.5e4, 10.6 / 8.1.  Not
-    // (ss|ss), 4e5 of mixed degrees 5.12 / 5.37, whose tiles hold few primitive
-    // quartets; not uncontracted batches, where set-up and barriers outweigh the
-    // products: (pp|ps) 3e5 0.43 / 0.49, (ff|pp) 2e4 2.39 / 3.03; not 3-centre ones,
-    // (f|dp) 1e5 4.90 / 6.20; nor small ones, (pp|pp) K = 3, 1000 quartets 0.217 / 0.236,
-    // which are not asked for their spread either, nor is a basis without contracted
-    // shells (it adds 7 us to the checking pass: (ps|ss) K = 1, 4000 quartets 62 / 69 us a call).
+    // Where the fixed-point tile can be the faster one (GB300, ms, FP64 against fixed
+    // point): contracted 4-centre classes above (ss|ss).  Not (ss|ss), 4e5 of mixed
+    // degrees 5.12 / 5.37, whose tiles hold few primitive quartets; not uncontracted
+    // batches, where set-up and barriers outweigh the products: (pp|ps) 3e5 0.43 / 0.49;
+    // not 3-centre ones, (f|dp) 1e5 4.90 / 6.20; nor the smallest, which are not asked
+    // for their spread either, nor is a basis without contracted shells (it adds 7 us
+    // to the checking pass: (ps|ss) K = 1, 4000 quartets 62 / 69 us a call).
     const int64_t nqq = quartets ? nq : nbra * nket;
     const int L = cls.la + cls.lb + cls.lc + cls.ld;
-    const bool try_fixed = fc && g_allow_fixed && !split && ldelta == 0 && (kind == 0 || kind == 3) &&
-                           L > 0 && L <= kFixLmax && nqq >= 2000 &&
-                           basis->nprim > basis->nshell;
+    const bool by_rule = g_fixed_mode == ERI_FIXED_RULE;
+    const bool try_fixed = fc && !fc->no_fixed && g_fixed_mode != ERI_FIXED_NEVER && !split && ldelta == 0 &&
+                           (kind == 0 || kind == 3) && L > 0 && L <= kFixLmax &&
+                           (!by_rule || (nqq >= 2000 && basis->nprim > basis->nshell));
     PrepassArgs pa{basis->shell_l, basis->shell_K, basis->nshell, bra, nbra, ket, nket, quartets,
                    quartets ? nq : (int64_t)0,
                    {cls.la, cls.lb, cls.lc, cls.ld}, (kind == 1 || kind == 2) ? 1 : 0, dinfo,
@@ -962,8 +1002,10 @@ int prepare_batch(eri_class_t cls, const eri_basis_t* basis, const int32_t* bra,
     *KB = kmax[0] * kmax[1];
     *KK = kmax[2] * kmax[3];
     if (mixed) *mixed = (INT_MAX - hinfo[7] < *KB || INT_MAX - hinfo[8] < *KK) ? 1 : 0;
-    const bool fix_ok = try_fixed && (int64_t)*KB * *KK >= 4 && nqq * *KB * *KK >= 150000 && fixed_eligible(cls, hinfo + 9);
-    const int key = fix_ok ? XF_FIXED : split;
+    bool fix_ok = try_fixed && fixed_eligible(cls, hinfo + 9);
+    if (fix_ok && by_rule)
+        fix_ok = (int64_t)*KB * *KK >= (nqq < kTuneMinQuartets ? kFixSmallPrims : 4) && nqq * *KB * *KK >= 150000 &&
+                 lookup_fp64_faster(cls, *KB, *KK, kind) != 1;
     if (allow_swap) {
         // Four forms: which side is transformed first (Section 3.2.2
         // transforms the ket first, assuming it has the lower l) and whether
@@ -986,26 +1028,26 @@ int prepare_batch(eri_class_t cls, const eri_basis_t* basis, const int32_t* bra,
             if (!opt[2] || !opt[3]) return err;
         }
         double cost[4];
-        for (int o = 0; o < 4; ++o) {
-            cost[o] = -1.0;  // infeasible
-            const ClassTables* c = opt[o];
-            if (!c) continue;
-            const double kb = (o & 1) ? *KK : *KB, kk = (o & 1) ? *KB : *KK;
-            if (c->hrr) {
-                // (f0|e0) must fit the register accumulators and the
-                // recursion buffers of the epilogue the shared memory
-                TilePlan tp;
-                if (c->nab * c->ncd > kNT * kNACC || !plan_tiles(*c, (int)kb, (int)kk, nqq, &tp)) continue;
+        auto set_costs = [&]() {
+            for (int o = 0; o < 4; ++o) {
+                cost[o] = -1.0;  // infeasible
+                const ClassTables* c = opt[o];
+                if (!c) continue;
+                const double kb = (o & 1) ? *KK : *KB, kk = (o & 1) ? *KB : *KK;
+                if (c->hrr) {
+                    // (f0|e0) must fit the register accumulators and the
+                    // recursion buffers of the epilogue the shared memory
+                    TilePlan tp;
+                    if (c->nab * c->ncd > kNT * kNACC || !plan_tiles(*c, (int)kb, (int)kk, nqq, &tp)) continue;
+                }
+                // a recursion step is an FP64 operation, which costs several
+                // products of the fixed-point transforms (where the smallest tile fits)
+                TilePlan least;
+                const bool fits = fix_ok && tile_layout(*c, (int)kb, (int)kk, 1, 1, 1, &least, XF_FIXED, kNTSlim);
+                const double step = fits ? 6.0 : 1.0;
+                cost[o] = kb * kk * ((c->nhb - c->pb0) * c->Tcd + 0.5 * c->nhl) + kb * c->ncd * c->Tab +
+                          (c->hrr ? step * (c->nab * c->nks + c->ncd_f * c->nbs) : 0);
             }
-            // a recursion step is an FP64 operation, which costs several
-            // products of the fixed-point transforms (where the smallest tile fits)
-            TilePlan least;
-            const bool fits = fix_ok && tile_layout(*c, (int)kb, (int)kk, 1, 1, 1, &least, XF_FIXED, kNTSlim);
-            const double step = fits ? 6.0 : 1.0;
-            cost[o] = kb * kk * ((c->nhb - c->pb0) * c->Tcd + 0.5 * c->nhl) + kb * c->ncd * c->Tab +
-                      (c->hrr ? step * (c->nab * c->nks + c->ncd_f * c->nbs) : 0);
-        }
-        {
             // the caller's form mask (eri_set_forms), unless it leaves no feasible form
             const int mask = g_form_mask.load();
             bool any = false;
@@ -1013,25 +1055,45 @@ int prepare_batch(eri_class_t cls, const eri_basis_t* basis, const int32_t* bra,
             if (any)
                 for (int o = 0; o < 4; ++o)
                     if (!(mask >> o & 1)) cost[o] = -1.0;
-        }
+        };
         auto cheapest = [&](int lo, int hi) {
             int b = -1;
             for (int o = lo; o < hi; ++o)
                 if (cost[o] >= 0 && (b < 0 || cost[o] < cost[b])) b = o;
             return b;
         };
-        int best = -1;
-        if (forced >= 0) {
-            if (forced > 3 || cost[forced] < 0) return ERI_EINVAL;
+        int best = -1, cached = 0;
+        auto choose = [&]() {  // false: the caller's form is not feasible
+            set_costs();
             best = forced;
-        } else {
-            best = lookup_form(cls, *KB, *KK, key, kind);
-            if (best >= 0 && cost[best] >= 0) {
-                if (fc) fc->cached = 1;
-            } else {
-                best = cheapest(0, 4);
+            if (forced >= 0) return forced <= 3 && cost[forced] >= 0;
+            best = lookup_form(cls, *KB, *KK, fix_ok ? XF_FIXED : split, kind);
+            cached = best >= 0 && cost[best] >= 0;
+            if (!cached) best = cheapest(0, 4);
+            return true;
+        };
+        if (!choose()) return ERI_EINVAL;
+        if (fix_ok && by_rule && nqq < kTuneMinQuartets && forced < 0) {
+            // a batch too small to be timed: the models of both tiles
+            auto degree = [&](int o, bool ket) { return ((o & 1) != 0) == ket ? *KB : *KK; };
+            const ClassTables& cf = *opt[best];
+            const bool fix_plain = best < 2;
+            double fix_time = 0.0, fp64_time = 1e300;
+            TilePlan tp;
+            if (plan_fixed_tile(cf, degree(best, 0), degree(best, 1), nqq, &tp, &fix_time)) {
+                const double setup = (double)degree(best, 0) * cf.Tab / cf.nab + (double)degree(best, 1) * cf.Tcd / cf.ncd;
+                fix_ok = false;
+                if (!choose()) return ERI_EINVAL;
+                const ClassTables& c64 = *opt[best];
+                if (plan_tiles(c64, degree(best, 0), degree(best, 1), nqq, &tp))
+                    fp64_time = plan_small_tile(c64, degree(best, 0), degree(best, 1), nqq, &tp);
+                // (an FP64 recursion form, of the larger error, by 10 % against a plain one)
+                if (fix_plain && best >= 2) fp64_time *= 1.1;
+                fix_ok = fix_small_faster(L, fix_time, setup, fp64_time);
+                if (fix_ok && !choose()) return ERI_EINVAL;
             }
         }
+        if (fc) fc->cached = cached;
         if (fc) {
             fc->form = best;
             fc->alt = best >= 2 ? cheapest(0, 2) : cheapest(2, 4);
@@ -1104,7 +1166,7 @@ int prepare_batch(eri_class_t cls, const eri_basis_t* basis, const int32_t* bra,
     }
     if (!ws) return err;
     if (fc) {
-        fc->key = key;
+        fc->key = fix_ok ? XF_FIXED : split;
         fc->fixed = fixed;
         fc->fx_f = fx_f;
         fc->mu = mu;
@@ -1217,7 +1279,6 @@ int check_batch_args(eri_class_t cls, const eri_basis_t* basis, const int32_t* b
 // kTuneQuartets) and remember the fastest with its time per quartet
 // (eri_batch compares forms by it).  The trial launches write (part
 // of) `out`; the real launch overwrites it.
-constexpr int64_t kTuneMinQuartets = 16384;
 constexpr int64_t kTuneQuartets = 8192;
 static std::map<std::tuple<int, int, int, int, int, int, int, int, int, int>, std::pair<TilePlan, float>> g_tuned;
 static std::mutex g_tuned_mu;
@@ -1581,42 +1642,80 @@ static int run_forward(eri_class_t cls, const eri_basis_t* basis, const int32_t*
     // cheapest plain and horizontal-recursion forms are both timed on the
     // batch's own leading quartets and the faster is remembered
     if (nqq >= kTuneMinQuartets) {
-        TilePlan best;
-        float ms = 0.f;
-        bool tuned = tuned_tile(a, fc.fixed ? XF_FIXED : split, st, &best, &ms);
-        if (!fc.cached && fc.alt >= 0) {
-            const eri_class_t sig = cls;
-            const int KB0 = (fc.form & 1) ? KK : KB, KK0 = (fc.form & 1) ? KB : KK;  // caller's orientation
-            FormChoice f1;
-            f1.form = fc.alt;
+        struct Timed {
+            FormChoice fc;
+            TilePlan tile;
+            float ms = 0.f;  // per quartet
+            bool tuned = false;
+        };
+        // The form and tile of the arithmetic that fc came out with; leaves the
+        // chosen form prepared (the pair tables share one workspace).
+        auto select = [&](Timed* t) -> int {
+            t->tuned = tuned_tile(a, t->fc.fixed ? XF_FIXED : split, st, &t->tile, &t->ms);
+            if (t->fc.cached || t->fc.alt < 0) return ERI_OK;
+            const int KB0 = (t->fc.form & 1) ? KK : KB, KK0 = (t->fc.form & 1) ? KB : KK;  // caller's orientation
+            Timed other;
+            other.fc.form = t->fc.alt;
+            other.fc.no_fixed = t->fc.no_fixed;
             FwdArgs a1;
-            TilePlan tp1, best1;
-            float ms1 = 0.f;
-            bool tuned1 = false;
-            if (prepare(&f1, &a1, &tp1) == ERI_OK) tuned1 = tuned_tile(a1, f1.fixed ? XF_FIXED : split, st, &best1, &ms1);
+            TilePlan tp1;
+            if (prepare(&other.fc, &a1, &tp1) == ERI_OK)
+                other.tuned = tuned_tile(a1, other.fc.fixed ? XF_FIXED : split, st, &other.tile, &other.ms);
             // In fixed point a recursion form, whose epilogue rounds in FP64, has to
             // be 10 % faster: (dp|pp) K = 3, 65000 quartets 7.58 ms against 8.25, error
             // against 64 bits 1.8e-15 against 1.6e-15 (the FP64 tile's plain form 1.6e-15,
             // its recursion form 3.7e-15); (dp|dp) K = 2, 50000, 3.30 against 3.77 ms stays.
             auto weight = [](const FormChoice& f) { return f.fixed && f.form >= 2 ? 1.1f : 1.0f; };
-            const bool take_alt = tuned1 && (!tuned || weight(f1) * ms1 < weight(fc) * ms);
-            remember_form(sig, KB0, KK0, fc.key, kind, take_alt ? f1.form : fc.form);
+            const bool take_alt = other.tuned && (!t->tuned || weight(other.fc) * other.ms < weight(t->fc) * t->ms);
+            remember_form(cls, KB0, KK0, t->fc.key, kind, take_alt ? other.fc.form : t->fc.form);
             if (take_alt) {
-                fc = f1;
+                *t = other;
                 a = a1;
                 tp = tp1;
-                best = best1;
-                tuned = tuned1;
+                return ERI_OK;
+            }
+            // rebuild the pair tables of the first form (the workspace was reused)
+            FormChoice f0;
+            f0.form = t->fc.form;
+            f0.no_fixed = t->fc.no_fixed;
+            return prepare(&f0, &a, &tp);
+        };
+        Timed best;
+        best.fc = fc;
+        err = select(&best);
+        if (err != ERI_OK) return err;
+        // Where fixed point is not surely the faster one, the FP64 tile is timed too,
+        // once per signature: fewer than 81 primitive quartets each, or (ss| on a side.
+        // 20000 quartets, ms, FP64 against fixed point: K = 2 (pp|ss) 0.199 / 0.225, (dd|ss)
+        // 0.433 / 0.488, (pp|pp) 0.558 / 0.446; K = 3 (ff|ss) 3.81 / 5.39, (dd|ss) 1.26 / 1.06;
+        // elsewhere 0.46 to 0.99 times FP64 for K = 3 and 4, (ps|ps) to (dp|dp).
+        const int KB0 = (best.fc.form & 1) ? KK : KB, KK0 = (best.fc.form & 1) ? KB : KK;
+        if (best.fc.fixed && best.tuned && g_fixed_mode == ERI_FIXED_RULE && g_form_mask.load() == 0xF &&
+            ((int64_t)KB * KK < kFixSmallPrims || cls.la + cls.lb == 0 || cls.lc + cls.ld == 0) &&
+            lookup_fp64_faster(cls, KB0, KK0, kind) < 0) {
+            Timed fp64;
+            fp64.fc.no_fixed = 1;
+            err = prepare(&fp64.fc, &a, &tp);
+            if (err == ERI_OK) err = select(&fp64);
+            if (err != ERI_OK) return err;
+            // (fixed point has to make up for the second pass over its pair tables,
+            // about 40 us a call, and for what the timings scatter; an FP64 recursion
+            // form, of the larger error, has to be 10 % faster than a plain one)
+            const float w = fp64.fc.form >= 2 && best.fc.form < 2 ? 1.1f : 1.0f;
+            const bool faster = fp64.tuned && w * fp64.ms * (float)nqq < 1.05f * best.ms * (float)nqq + 0.04f;
+            remember_fp64_faster(cls, KB0, KK0, kind, faster);
+            if (faster) {
+                best = fp64;
             } else {
-                // rebuild the pair tables of the first form (the workspace was reused)
                 FormChoice f0;
-                f0.form = fc.form;
+                f0.form = best.fc.form;
                 err = prepare(&f0, &a, &tp);
                 if (err != ERI_OK) return err;
             }
         }
-        if (tuned) {
-            tp = best;
+        fc = best.fc;
+        if (best.tuned) {
+            tp = best.tile;
             set_tile(a, tp);
             a.ntiles = (nqq + tp.TQ - 1) / tp.TQ;
             from_tuner = true;
@@ -1746,11 +1845,11 @@ extern "C" int eri_last_arithmetic(int32_t* arithmetic)
     return ERI_OK;
 }
 
-extern "C" int eri_set_fixed(int32_t allowed)
+extern "C" int eri_set_fixed(int32_t mode)
 {
-    if (allowed != 0 && allowed != 1) return ERI_EINVAL;
-    const int prev = g_allow_fixed;
-    g_allow_fixed = allowed;
+    if (mode < ERI_FIXED_NEVER || mode > ERI_FIXED_ALWAYS) return ERI_EINVAL;
+    const int prev = g_fixed_mode;
+    g_fixed_mode = mode;
     return prev;
 }
 

@@ -167,6 +167,7 @@ struct PairTables {
 // kernel's bra), bit 1 = horizontal-recursion form.
 struct FormChoice {
     int form = -1;    // in: a form to force, or -1 (remembered, else modelled); out: the form used
+    int no_fixed = 0; // in: 1 keeps to the FP64 tile
     int alt = -1;     // out: the modelled-cheapest feasible form of the other kind (plain vs HRR), or -1
     int cached = 0;   // out: 1 when the form was remembered from an earlier timing
     int key = 0;      // out: the arithmetic (XF_*) the form is remembered under: what the class may take,

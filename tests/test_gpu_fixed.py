@@ -16,6 +16,14 @@ from gpu_helpers import assert_close, nc, oracle_blocks, to_device
 
 pytestmark = pytest.mark.gpu
 
+
+@pytest.fixture(autouse=True)
+def _wherever_it_can():
+    """The fixed-point tile wherever its precision allows, whatever would be faster."""
+    eri.eri_set_fixed(eri.ERI_FIXED_ALWAYS)
+    yield
+    eri.eri_set_fixed(eri.ERI_FIXED_RULE)
+
 # class, primitives per shell: K_ket = 4 (even), 9 (odd), 16 (past one fold), 25 and 36 for s shells (several
 # folds); L = 1..6 in fixed point, 7 and 8 in FP64; a component-pair list of one column, pairs and single columns
 CASES = [((1, 0, 0, 0), 2), ((0, 1, 1, 0), 3), ((1, 1, 1, 0), 4), ((1, 1, 1, 1), 3), ((2, 1, 1, 1), 3),
@@ -133,7 +141,7 @@ def test_orders_above_six_keep_the_fp64_tile(cls):
     assert _sample_error(out[:24], oracle_blocks(cls, basis, bra, ket, q[:24], prec="ld")) < 5e-15
 
 
-@pytest.mark.parametrize("cls,K,nq", [((1, 1, 1, 0), 3, 20011), ((2, 1, 2, 0), 2, 16384), ((2, 2, 1, 1), 2, 16385)])
+@pytest.mark.parametrize("cls,K,nq", [((1, 1, 1, 0), 3, 20011), ((2, 1, 1, 1), 3, 16384), ((2, 2, 1, 1), 2, 16385)])
 def test_timed_tiles_and_form_against_oracle(cls, K, nq):
     """Batches long enough to be timed: the tile shape and the form come from the timing; the second call, which
     uses what the first remembered, gives the same bits."""
@@ -151,7 +159,7 @@ def test_timed_tiles_and_form_against_oracle(cls, K, nq):
 
 
 def test_callers_choice_of_the_fp64_tile():
-    """eri_set_fixed(False) keeps this thread's batches on the FP64 tile; both agree to round-off."""
+    """ERI_FIXED_NEVER keeps this thread's batches on the FP64 tile; both agree to round-off."""
     cls, nq = (1, 1, 1, 0), 4001
     basis, pools = synth.class_sweep_pools(seed=15, lmax=1, pool=32, K=3, cube=4.0)
     bra, ket, q = synth.class_sweep_batch(pools, cls, seed=16, npairs=40, nq=nq)
@@ -159,14 +167,33 @@ def test_callers_choice_of_the_fp64_tile():
     db = eri.DeviceBasis(basis)
     fixed = eri.eri_batch(cls, db, b, k, qq).cpu().numpy()
     assert eri.eri_last_arithmetic() == eri.ERI_ARITH_FIXED
-    assert eri.eri_set_fixed(False) is True
-    try:
-        fp64 = eri.eri_batch(cls, db, b, k, qq).cpu().numpy()
-        assert eri.eri_last_arithmetic() == eri.ERI_ARITH_FP64
-    finally:
-        assert eri.eri_set_fixed(True) is False
+    assert eri.eri_set_fixed(eri.ERI_FIXED_NEVER) == eri.ERI_FIXED_ALWAYS
+    fp64 = eri.eri_batch(cls, db, b, k, qq).cpu().numpy()
+    assert eri.eri_last_arithmetic() == eri.ERI_ARITH_FP64
     assert_close(fixed, fp64, what="fixed point against FP64")
     assert not np.array_equal(fixed, fp64)
+
+
+@pytest.mark.parametrize("cls,K,ratio,nq,fixed", [
+    ((1, 1, 1, 0), 2, 3.0, 16383, False), ((2, 1, 2, 1), 2, 3.0, 9400, False),  # few primitive quartets, not timed
+    ((2, 2, 0, 0), 3, 2.0, 2000, False), ((1, 0, 0, 0), 3, 2.0, 4000, False),  # the models
+    ((1, 1, 1, 1), 3, 2.0, 8000, True), ((2, 1, 1, 1), 4, 1.5, 4000, True),
+    ((3, 3, 0, 0), 2, 3.0, 20000, False),  # timed against the FP64 tile
+    ((1, 1, 1, 0), 3, 2.0, 20000, True)])
+def test_rule_takes_the_faster_tile(cls, K, ratio, nq, fixed):
+    """Batches on which the two tiles' times differ by a tenth and more: the rule, and the timing, pick the faster."""
+    eri.eri_set_fixed(eri.ERI_FIXED_RULE)
+    basis, pools = synth.class_sweep_pools(seed=3, lmax=max(cls), pool=256, K=K,
+                                           exps_fn=lambda rng, k: 0.2 * ratio ** np.arange(k))
+    bra, ket, q = synth.class_sweep_batch(pools, cls, seed=4, npairs=1024, nq=nq)
+    b, k, qq = to_device(bra, ket, q)
+    db = eri.DeviceBasis(basis)
+    for _ in range(2):
+        out = eri.eri_batch(cls, db, b, k, qq)
+        assert eri.eri_last_arithmetic() == (eri.ERI_ARITH_FIXED if fixed else eri.ERI_ARITH_FP64)
+    pick = np.r_[0:6, nq - 6:nq]
+    got = out.cpu().numpy().reshape(-1, nq).T[pick]
+    assert_close(got, oracle_blocks(cls, basis, bra, ket, q[pick]), what=f"{cls} K={K}")
 
 
 # in a process of its own: the library keeps its tables and workspace
@@ -188,9 +215,9 @@ db = eri.DeviceBasis(basis)
 out = torch.empty(nq * nc(2) * nc(1) * nc(1), dtype=torch.float64, device="cuda")
 eri.eri_set_forms(1)
 if leave < 1 << 30:  # the FP64 tile's tables are there already
-    eri.eri_set_fixed(False)
+    eri.eri_set_fixed(eri.ERI_FIXED_NEVER)
     eri.eri_batch(cls, db, b, k, qq, out=out)
-    eri.eri_set_fixed(True)
+eri.eri_set_fixed(eri.ERI_FIXED_ALWAYS)
 torch.cuda.synchronize()
 held = torch.empty(torch.cuda.mem_get_info()[0] - leave, dtype=torch.uint8, device="cuda")
 eri.eri_batch(cls, db, b, k, qq, out=out)

@@ -12,6 +12,14 @@ from gpu_helpers import THREADS, assert_close, oracle_blocks, to_device
 pytestmark = pytest.mark.gpu
 
 
+@pytest.fixture(autouse=True)
+def _wherever_it_can():
+    """The fixed-point tile wherever its precision allows, whatever would be faster."""
+    eri.eri_set_fixed(eri.ERI_FIXED_ALWAYS)
+    yield
+    eri.eri_set_fixed(eri.ERI_FIXED_RULE)
+
+
 def _shells(atoms, l, exps, rng):
     return [(a, l, list(z), list(rng.uniform(0.5, 1.0, len(z)) * synth.norm_coef(np.asarray(z), l)))
             for a, z in zip(atoms, exps)]
@@ -61,13 +69,11 @@ def _both_tiles(cls, basis, bra, ket, q, n):
     b, k, qq = to_device(bra, ket, q)
     db = eri.DeviceBasis(basis)
     out = []
-    for fixed in (True, False):
-        eri.eri_set_fixed(fixed)
-        try:
-            out.append(eri.eri_batch(cls, db, b, k, qq).cpu().numpy().reshape(-1, len(q)).T[:n])
-        finally:
-            eri.eri_set_fixed(True)
-        assert eri.eri_last_arithmetic() == (eri.ERI_ARITH_FIXED if fixed else eri.ERI_ARITH_FP64)
+    for mode, arithmetic in ((eri.ERI_FIXED_ALWAYS, eri.ERI_ARITH_FIXED), (eri.ERI_FIXED_NEVER, eri.ERI_ARITH_FP64)):
+        eri.eri_set_fixed(mode)
+        out.append(eri.eri_batch(cls, db, b, k, qq).cpu().numpy().reshape(-1, len(q)).T[:n])
+        assert eri.eri_last_arithmetic() == arithmetic
+    eri.eri_set_fixed(eri.ERI_FIXED_ALWAYS)
     return out[0], out[1], _reference(cls, basis, bra, ket, q[:n])
 
 

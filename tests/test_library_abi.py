@@ -111,11 +111,11 @@ def test_arithmetic_selector_without_gpu():
     import paper_2506_12501_gb300 as eri
     L = eri.lib()
     assert L.eri_last_arithmetic(None) == eri.ERI_EINVAL
-    assert L.eri_set_fixed(2) == eri.ERI_EINVAL and L.eri_set_fixed(-1) == eri.ERI_EINVAL
-    assert eri.eri_set_fixed(False) is True
+    assert L.eri_set_fixed(3) == eri.ERI_EINVAL and L.eri_set_fixed(-1) == eri.ERI_EINVAL
+    assert eri.eri_set_fixed(eri.ERI_FIXED_NEVER) == eri.ERI_FIXED_RULE
     seen = []
-    t = threading.Thread(target=lambda: seen.append(eri.eri_set_fixed(True)))
+    t = threading.Thread(target=lambda: seen.append(eri.eri_set_fixed(eri.ERI_FIXED_ALWAYS)))
     t.start()
     t.join()
-    assert seen == [True]
-    assert eri.eri_set_fixed(True) is False
+    assert seen == [eri.ERI_FIXED_RULE]
+    assert eri.eri_set_fixed(eri.ERI_FIXED_RULE) == eri.ERI_FIXED_NEVER
