@@ -254,7 +254,7 @@ struct PairArgs {
 };
 
 constexpr int kPairThreads = 128;
-constexpr int64_t kPairWarpSlots = 8192;  // at most this many slots take a warp each (twice as many for 1000 terms)
+constexpr double kPairWarpSlots = 640.0;  // times sqrt(terms): at most this many slots take a warp each
 constexpr int kEax = (kLmax + 3) * (kLmax + 3) * (2 * kLmax + 5);  // per-axis E table bound (adjoint shifts)
 constexpr int kEfw = (kLmax + 1) * (kLmax + 1) * (2 * kLmax + 1);  // without the shifts (also the HRR form's)
 
@@ -457,15 +457,17 @@ __global__ void __launch_bounds__(kPairThreads) pair_kernel_t(PairArgs a)
 // takes three per slot
 static void launch_pair(const PairArgs& p, int grid, cudaStream_t st)
 {
-    // A warp per slot where the slots are few for one thread each (time in us of
-    // one thread | one warp per slot): 1000 slots of (pp| 26 | 12, 2048 of (dd|
-    // 93 | 36, 9216 of (dd| 94 | 87, 18432 of (dp| 57 | 149, of (dd| 94 | 164;
-    // longest lists: 2048 of (ff| 917 | 92, 9216 of (ff| 1036 | 460.  Lists of fewer
-    // than 16 terms leave most lanes idle.
+    // A warp per slot where the slots are few for one thread each: one thread takes the
+    // same time for any number of slots up to the chip's threads, warps queue from about
+    // 3000 on.  Calls of one quartet, us, one thread | one warp per slot: (pp|, 33 terms,
+    // 1000 slots 99 | 87, 3000 98 | 95, 4500 99 | 105, 8192 103 | 124; (dp|, 108, 6000
+    // 136 | 126, 8192 132 | 140; (dd|, 336, 8192 240 | 182, 16384 242 | 276; (ff|, 1920,
+    // 16384 984 | 646: they cross near 640 sqrt(terms).  Lists of fewer than 16 terms
+    // leave most lanes idle.
     const int64_t slots = p.npairs * p.KS;
     if (p.ax)
         pair_kernel_t<true, false><<<(int)std::min<int64_t>(3LL * grid, 24LL * sm_count()), kPairThreads, 0, st>>>(p);
-    else if (p.T >= 16 && slots <= (p.T >= 1000 ? 2 : 1) * kPairWarpSlots)
+    else if (p.T >= 16 && (double)slots <= kPairWarpSlots * std::sqrt((double)p.T))
         pair_kernel_t<false, true><<<(int)std::max<int64_t>(1, std::min<int64_t>((32 * slots + kPairThreads - 1) / kPairThreads, 16LL * sm_count())),
                                      kPairThreads, 0, st>>>(p);
     else

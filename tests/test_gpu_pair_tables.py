@@ -11,7 +11,8 @@ from gpu_helpers import assert_close, oracle_blocks, to_device
 pytestmark = pytest.mark.gpu
 
 
-@pytest.mark.parametrize("cls,K,limit", [((1, 1, 0, 0), 1, 8192), ((1, 1, 1, 0), 3, 8192 // 9), ((3, 3, 0, 0), 1, 16384)])
+# limit: the last number of bra pairs that take warps, 640 sqrt(terms) slots for 33 and 1920 terms
+@pytest.mark.parametrize("cls,K,limit", [((1, 1, 0, 0), 1, 3676), ((1, 1, 1, 0), 3, 3676 // 9), ((3, 3, 0, 0), 1, 28043)])
 def test_warp_and_thread_tables_agree(cls, K, limit):
     basis, pools = synth.class_sweep_pools(seed=11, lmax=max(cls), pool=40, K=K, cube=3.0)
     bra, ket, _ = synth.class_sweep_batch(pools, cls, seed=12, npairs=37, nq=1)
