@@ -445,7 +445,7 @@ __device__ __forceinline__ void fix_recursion_c(const long long (&F)[L + 1], con
     });
 }
 
-// Stage A of one primitive quartet into its column of R, relative to 2^g.
+// Stage A of one primitive quartet into its column of R, relative to 2^g (L > 0).
 template <int LMAX, int FIXED>
 __device__ __forceinline__ void fix_aux_item(int Lr, const FixPrim& p, const FixPrim& q, int f,
                                              const long long* __restrict__ tab, const long long* __restrict__ far,
@@ -458,21 +458,16 @@ __device__ __forceinline__ void fix_aux_item(int Lr, const FixPrim& p, const Fix
     FixBase b;
     fix_base<LMAX>(L, p, q, f, tab, far, F, b);
     fix_factors<LMAX>(L, b, sigma, rmu, g, phi, sh);
-    if constexpr (FIXED && LMAX == 0) {
-        *reinterpret_cast<int2*>(R) = fix_limbs<kLimbR>(fix_finish(F[0], phi[0], sh[0]));
-    } else {
-        int x1[3], x0s[3];
+    int x1[3], x0s[3];
 #pragma unroll
-        for (int i = 0; i < 3; ++i) {
-            x1[i] = (int)((b.x[i] + (1LL << 28)) >> 29);
-            x0s[i] = (int)((unsigned)(int)(b.x[i] - ((long long)x1[i] << 29)) << 3);
-        }
-        if constexpr (FIXED) {
-            fix_recursion_c<LMAX>(F, x1, x0s, phi, sh, R, NIs);
-        } else {
-            fix_recursion(L, F, x1, x0s, phi, sh, st, ord, R, NIs, G, j, on);
-        }
+    for (int i = 0; i < 3; ++i) {
+        x1[i] = (int)((b.x[i] + (1LL << 28)) >> 29);
+        x0s[i] = (int)((unsigned)(int)(b.x[i] - ((long long)x1[i] << 29)) << 3);
     }
+    if constexpr (FIXED)
+        fix_recursion_c<LMAX>(F, x1, x0s, phi, sh, R, NIs);
+    else
+        fix_recursion(L, F, x1, x0s, phi, sh, st, ord, R, NIs, G, j, on);
 }
 
 // Shared-memory tables of a class and tile shape (stage_fixed_tables).
@@ -726,7 +721,6 @@ __device__ void tile_fixed(const FwdArgs& a, int64_t q0, int nqt, double* sm, do
                     NIs, G, lane & (G - 1), on);
             };
             switch (regs ? ct.L : -1) {
-                case 0: run(IntC<0>(), IntC<1>()); break;
                 case 1: run(IntC<1>(), IntC<1>()); break;
                 case 2: run(IntC<2>(), IntC<1>()); break;
                 case 3: run(IntC<3>(), IntC<1>()); break;

@@ -95,6 +95,74 @@ int main() {
             worst = std::max(worst, fabs((double)(sqrtl(rho) * R[N] * powl(mu * powl(2, sigma), -N) * powl(2, -gg))));
     }
     printf("distance 0 %.9f\n", worst);
+    // each order's axis entry at a distance, relative to its multipole sqrt(pi)/2 N!/r^(N+1), in the tile's
+    // Hermite unit (s r >= 1.1 sqrt(8)), beside the same recursion in doubles
+    for (int L = 1; L <= 6; ++L) {
+        std::vector<int64_t> tab((size_t)kFixBoysRows * fix_boys_words(L), 0), far(kFixFarWords);
+        fix_far_constants(L, far.data());
+        auto boys = [&](int M, Q T, Q* F) {
+            Q t = 1.0L / (2 * M + 1), sum = t;
+            for (int k = 1; k < 5000 && t > sum * 1e-25L; ++k) { t *= 2 * T / (2 * M + 2 * k + 1); sum += t; }
+            F[M] = expl(-T) * sum;
+            for (int m = M - 1; m >= 0; --m) F[m] = (2 * T * F[m + 1] + expl(-T)) / (2 * m + 1);
+        };
+        const double Ts[] = {4.5, 9, 30, 100, 300};
+        const int W = kBoysMtab + 2, per = kFixBoysInvStep / kBoysInvStep;
+        std::vector<Q> master((size_t)kBoysGrid * W, 0);
+        for (double T : Ts)
+            for (int j = (int)(T * kFixBoysInvStep) - 3; j <= (int)(T * kFixBoysInvStep) + 3; ++j) {
+                const int c = (j + per / 2) / per;
+                boys(kBoysMtab, (Q)c / kBoysInvStep, &master[(size_t)c * W]);
+                master[(size_t)c * W + kBoysMtab + 1] = expl(-(Q)c / kBoysInvStep);
+                fix_boys_row(master.data(), L, j, tab.data() + (size_t)j * fix_boys_words(L));
+            }
+        Q e[7] = {0}, e64[7] = {0};
+        for (int it = 0; it < 4000; ++it) {
+            const double T0 = it % 6 < 5 ? Ts[it % 6] + uni(-2, 2) / kFixBoysInvStep : pow(10, uni(2.6, 4));
+            const double zp = pow(10, uni(-1, 2)), zq = pow(10, uni(-1, 2)), rho0 = zp * zq / (zp + zq);
+            FixPrim p = prim(zp), q = prim(zq);
+            const double P = uni(-6, 6), C = P - sqrt(T0 / rho0);
+            p.x[0] = fix_coordinate(P, 50);
+            q.x[0] = fix_coordinate(C, 50);
+            const Q r = ((Q)p.x[0] - (Q)q.x[0]) / powl(2, 50), rho = 1 / (1 / (Q)zp + 1 / (Q)zq), T = rho * r * r;
+            const double mu = uni(1, 2), fr = (double)r;
+            const int sigma = (ilogb(2.42 / (mu * mu) * std::min(rho0, 4 / (fr * fr))) + 2) >> 1;
+            const int gg = fix_bound(L, (float)rho0, (float)(fr * fr), sigma, (float)(1 / mu));
+            long long F[11], phi[11], R[7];
+            int sh[11];
+            FixBase B;
+            fix_base<10>(L, p, q, 50, (const long long*)tab.data(), (const long long*)far.data(), F, B);
+            fix_factors<10>(L, B, sigma, (long long)(0x1p62L / (Q)mu), gg, phi, sh);
+            const int x1 = (int)((B.x[0] + (1LL << 28)) >> 29), x0 = (int)((B.x[0] - ((long long)x1 << 29)) * 8);
+            Q FQ[kBoysMtab + 1], c[7];
+            double d[7];
+            if (T > 400) {
+                const Q eT = expl(-T);
+                FQ[0] = 0.5L * sqrtl(3.14159265358979323846264338327950288L / T);
+                for (int m = 0; m < L; ++m) FQ[m + 1] = ((2 * m + 1) * FQ[m] - eT) / (2 * T);
+            } else
+                boys(L, T, FQ);
+            auto f64 = [&](int n) { double v = sqrt((double)rho); for (int i = 0; i < n; ++i) v *= -2 * (double)rho; return v * (double)FQ[n]; };
+            R[0] = F[L]; c[0] = sqrtl(rho) * powl(-2 * rho, L) * FQ[L]; d[0] = f64(L);
+            for (int n = L - 1; n >= 0; --n) {
+                for (int t = L - n; t >= 1; --t) {
+                    R[t] = t > 1 ? fix_step(x1, x0, R[t - 1], t - 1, R[t - 2]) : fix_step(x1, x0, R[t - 1]);
+                    c[t] = r * c[t - 1] + (t > 1 ? (t - 1) * c[t - 2] : 0);
+                    d[t] = fr * d[t - 1] + (t > 1 ? (t - 1) * d[t - 2] : 0);
+                }
+                R[0] = F[n]; c[0] = sqrtl(rho) * powl(-2 * rho, n) * FQ[n]; d[0] = f64(n);
+            }
+            Q pole = 0.886226925452758013649L / r;
+            for (int N = 0; N <= L; ++N, pole *= N / r) {
+                const Q v = (Q)fix_finish(R[N], phi[N], sh[N]) * powl(2, gg - 62) * powl(mu * powl(2, sigma), N);
+                e[N] += powl((v - c[N]) / pole, 2);
+                e64[N] += powl((d[N] - c[N]) / pole, 2);
+            }
+        }
+        double ratio = 0;
+        for (int N = 0; N <= L; ++N) ratio = std::max(ratio, (double)sqrtl(e[N] / e64[N]));
+        printf("order%d 0 %.4f\n", L, ratio);
+    }
     // the squared distance of centres at the far end of the admitted coordinates
     double off = 0;
     for (int it = 0; it < 2000; ++it) {
@@ -151,6 +219,13 @@ def test_coincident_centres_stay_inside_the_limbs(figures, L):
 def test_every_distance_stays_inside_the_bound(figures):
     # rounding the bound up to a power of two leaves the margin where the bound is attained
     assert 0.9 < figures["distance"][1] < 1 - 2.0 ** -32
+
+
+@pytest.mark.parametrize("L", range(1, 7))
+def test_every_order_keeps_its_digits_at_a_distance(figures, L):
+    """The root mean square error of each order, over the order's own size: no larger than in doubles (the integrals
+    of one-centre pairs are multipoles of a single order, however small beside order 0)."""
+    assert figures[f"order{L}"][1] < 1.0
 
 
 def test_distance_of_centres_at_the_end_of_the_range(figures):
