@@ -38,11 +38,13 @@
 // Precision: FP64 transforms round every product and sum at 2^-53 of its own
 // size; here every operand is rounded at 2^-60 or 2^-61 of the largest the
 // sum may hold.  The difference between the two is how far the bound lies above
-// the sum, which grows with the spread of exponents inside a pair:
-// (largest / smallest zeta)^((l1 + l2) / 2).  Batches whose pairs exceed
-// 2^kFixSpreadBits there run the FP64 tile (fixed_eligible in eri_fwd.cu).
-// Below it the transforms' error, simulated against 64-bit mantissas over the
-// class and exponent ranges of the tests, is 0.2 to 1.3 times the FP64 one's.
+// the sum, which grows with the spread of exponents inside a pair,
+// (largest / smallest zeta)^((l1 + l2) / 2), and with the order.  Batches beyond
+// 2^kFixSpreadBits or kFixLmax run the FP64 tile (fixed_eligible, prepare_batch
+// in eri_fwd.cu); within them the relative 2-norm error over a batch is 0.4 to 1.2
+// times the FP64 tile's ((dp|dp) with three primitives up to 1.7 in a 1.5-bohr
+// cube, 1.0 in a 12-bohr one).  That is the error of blocks: an entry far below
+// the others of its column, over short distances, keeps fewer digits than FP64.
 #pragma once
 
 #include <climits>
@@ -54,8 +56,13 @@
 
 namespace eri {
 
-// log2 of the largest spread factor of a pair for the fixed-point tile
-constexpr float kFixSpreadBits = 6.0f;
+// log2 of the largest spread factor of a pair for the fixed-point tile.  Relative
+// 2-norm error against the oracle, fixed point over FP64, plain form, one and two
+// centres a pair in cubes of 1.5 and 4 bohr | 12 bohr: 2.4 bits and less 0.6 to 1.06 |
+// 0.8 to 1.04; 4.0 (pp|pp) 0.5 to 1.07 | 1.01; 4.8 (dp|pp) 0.98 to 1.02, (dp|dp) 1.1 to 1.7 |
+// 1.0; 6.0 (pp|pp) 1.0 to 4.0 | 1.06, (dp|pp) 1.0 to 2.1 | 1.0, (dp|dp) 1.4 to 4.6 | 1.09; 7.0
+// (dp|dp) 3.3 to 10 | 1.3; 8.0 (pp|pp) 1.7 to 27 | 3.4.
+constexpr float kFixSpreadBits = 5.0f;
 // Largest order the tile takes.  Above it one exponent for the integrals of all
 // orders costs more than the FP64 tile's roundings: relative 2-norm error against
 // the oracle, fixed point over FP64, plain form, K = 2 of ratio 3, pairs of two

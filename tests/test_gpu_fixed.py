@@ -124,6 +124,24 @@ def test_wide_exponents_and_non_finite_primitives_keep_the_fp64_tile():
     assert bad.any() and np.isnan(out[bad]).all() and np.isfinite(out[~bad]).all()
 
 
+@pytest.mark.parametrize("ratio,fixed", [(30.0, True), (34.0, False), (60.0, False)])
+def test_spread_beyond_five_bits_keeps_the_fp64_tile(ratio, fixed):
+    """(pp|pp), K = 2: a pair's exponents spread by log2(ratio) = 4.9, 5.1 and 5.9 bits, in a small cube, where spread
+    costs most (at 5.9 bits the fixed-point tile's error was four times the FP64 tile's 5e-16)."""
+    cls, nq = (1, 1, 1, 1), 10240
+    basis, pools = synth.class_sweep_pools(seed=23, lmax=1, pool=32, K=2, cube=1.5,
+                                           exps_fn=lambda rng, K: 0.2 * np.array([1.0, ratio]))
+    bra, ket, q = synth.class_sweep_batch(pools, cls, seed=24, npairs=60, nq=nq)
+    b, k, qq = to_device(bra, ket, q)
+    eri.eri_set_forms(1)
+    try:
+        out = eri.eri_batch(cls, eri.DeviceBasis(basis), b, k, qq).cpu().numpy().reshape(-1, nq).T
+    finally:
+        eri.eri_set_forms(0)
+    assert eri.eri_last_arithmetic() == (eri.ERI_ARITH_FIXED if fixed else eri.ERI_ARITH_FP64)
+    assert _sample_error(out[:240], oracle_blocks(cls, basis, bra, ket, q[:240], prec="ld")) < 1e-15
+
+
 @pytest.mark.parametrize("cls", [(3, 2, 1, 1), (2, 2, 2, 1), (3, 3, 1, 1), (3, 2, 2, 2), (3, 2, 3, 2)])
 def test_orders_above_six_keep_the_fp64_tile(cls):
     """Contracted classes of order 7 to 10: FP64 tile, whose error in the plain form stays near 1e-15 on these pairs
