@@ -218,7 +218,8 @@ class ClockSampler:
                 "samples": len(sm), "power_w_max": max(pw) if pw else None}
 
 
-KERNEL_SOURCES = ("eri_fwd.cu", "eri_tile.cuh", "eri_device.cuh", "eri_internal.h", "eri_tables.cu")
+KERNEL_SOURCES = ("eri_fwd.cu", "eri_tile.cuh", "eri_fixed.cuh", "eri_fixaux.cuh", "eri_device.cuh", "eri_internal.h",
+                  "eri_tables.cu")
 
 
 def kernel_source_sha():
@@ -611,6 +612,7 @@ def run_library(args):
     stream = torch.cuda.current_stream()
     forms = {}
     tiles = {}
+    arithmetic = {}
 
     def step(timing=None):
         for cls, (b, k, q) in dev_batches.items():
@@ -621,6 +623,7 @@ def run_library(args):
             eri.eri_batch(cls, db, b, k, q, out=outs[cls], precision=prec)
             forms[cls] = eri.eri_last_form()
             tiles[cls] = eri.eri_last_tile()
+            arithmetic[cls] = eri.eri_last_arithmetic()
             if timing is not None:
                 e1.record(stream)
                 timing[cls].append((e0, e1))
@@ -663,28 +666,42 @@ def run_library(args):
     value = job_rate(world, nq_step, args.steps, total_ms)
 
     per_class = {}
+    class_ms = {}
     for cls in batches:
-        ms = statistics.median(a.elapsed_time(b) for a, b in timing[cls])
+        ms = class_ms[cls] = statistics.median(a.elapsed_time(b) for a, b in timing[cls])
         qps = nq_class / (ms / 1e3)
         per_class["".join(map(str, cls))] = {
             "ms": round(ms, 4), "qps": round(qps),
             "form": ("swapped " if forms[cls][0] else "") + ("hrr" if forms[cls][1] else "plain"),
             "tile": "TQ{tq} IC{ic} x{threads}".format(**tiles[cls]),
+            "arithmetic": ("fp64", "split", "fixed")[arithmetic[cls]],
             "gflops": round(sparse[cls] * qps / 1e9, 1),
             "frac": round(sparse[cls] * qps / 1e9 / FP64_PEAK_GFLOPS, 4),
             "frac_dense": round(dense[cls] * qps / 1e9 / FP64_PEAK_GFLOPS, 4)}
     emit_detail("per_class", {"note": "qps = quartets/s; gflops and frac from the sparse FP64 count of the form "
-                                      "that ran; frac_dense from the dense-GEMM count",
+                                      "that ran (of a class in fixed point: FP64 equivalents, done on "
+                                      "the integer pipe); frac_dense from the dense-GEMM count",
                               "per_class": per_class, "step_ms": [round(x, 3) for x in step_ms]}, rank)
     fwd_launches, fwd_ms = prof[eri.PROF_FWD]
-    flops_per_step = sum(sparse[c] * nq_class for c in batches)
     dense_per_step = sum(dense[c] * nq_class for c in batches)
-    fwd_gflops = flops_per_step * args.steps / (fwd_ms / 1e3) / 1e9 if fwd_ms > 0 else None
+    # the FP64 pipe bounds the classes on the FP64 tile only; a class in fixed point does its products on the integer
+    # pipe, and its FP64-equivalent rate says nothing about either
+    on_fp64 = [c for c in batches if arithmetic[c] != eri.ERI_ARITH_FIXED]
+    on_fixed = [c for c in batches if arithmetic[c] == eri.ERI_ARITH_FIXED]
+
+    def class_gflops(classes):
+        ms = sum(class_ms[c] for c in classes)
+        return sum(sparse[c] * nq_class for c in classes) / (ms / 1e3) / 1e9 if ms > 0 else None
+    fwd_gflops = class_gflops(on_fp64)
     roofline = {"bound": "alu", "kernel": "fwd_kernel", "achieved": fwd_gflops, "peak": FP64_PEAK_GFLOPS,
                 "unit": "GFLOP/s", "frac": (fwd_gflops / FP64_PEAK_GFLOPS) if fwd_gflops else None,
+                "classes": len(on_fp64), "step_share": sum(class_ms[c] for c in on_fp64) / sum(class_ms.values()),
+                "fixed_point": {"kernel": "fwd_fixed_kernel", "classes": len(on_fixed),
+                                "fp64_equivalent_gflops": class_gflops(on_fixed)},
                 "traffic": profile_traffic(),
                 "peak_source": "derived: FP64 FMA pipe, 152 SMs x 2 DFMA/clk x 2 flop x 2.07 GHz",
-                "flops": "sparse FP64 count of the implemented sequence, FMA = 2",
+                "flops": "sparse FP64 count of the implemented sequence, FMA = 2, over whole calls of the classes "
+                         "that run the FP64 tile",
                 "ms_per_launch": round(fwd_ms / max(fwd_launches, 1), 4),
                 "frac_dense_formulation": round(dense_per_step * args.steps / (fwd_ms / 1e3) / 1e9 /
                                                 FP64_PEAK_GFLOPS, 3) if fwd_ms else None}
