@@ -39,12 +39,13 @@
 // size; here every operand is rounded at 2^-60 or 2^-61 of the largest the
 // sum may hold.  The difference between the two is how far the bound lies above
 // the sum, which grows with the spread of exponents inside a pair,
-// (largest / smallest zeta)^((l1 + l2) / 2), and with the order.  Batches beyond
-// 2^kFixSpreadBits or kFixLmax run the FP64 tile (fixed_eligible, prepare_batch
-// in eri_fwd.cu); within them the relative 2-norm error over a batch is 0.4 to 1.2
-// times the FP64 tile's ((dp|dp) with three primitives up to 1.7 in a 1.5-bohr
-// cube, 1.0 in a 12-bohr one).  That is the error of blocks: an entry far below
-// the others of its column, over short distances, keeps fewer digits than FP64.
+// (largest / smallest zeta)^((l1 + l2) / 2), and with the order.  So does the FP64
+// tile's error with the distance inside a pair, which its recursion forms
+// magnify.  fixed_eligible (eri_fwd.cu) admits what measured no larger a relative
+// 2-norm error over a batch than the FP64 tile in the form that would have run:
+// order 6 and 5 bits of spread anywhere, order 8 and 6 bits where some pair's
+// centres lie kFixWide apart.  These are errors of blocks: an entry far below the
+// others of its column, over short distances, keeps fewer digits than FP64.
 #pragma once
 
 #include <climits>
@@ -56,21 +57,25 @@
 
 namespace eri {
 
-// log2 of the largest spread factor of a pair for the fixed-point tile.  Relative
-// 2-norm error against the oracle, fixed point over FP64, plain form, one and two
-// centres a pair in cubes of 1.5 and 4 bohr | 12 bohr: 2.4 bits and less 0.6 to 1.06 |
-// 0.8 to 1.04; 4.0 (pp|pp) 0.5 to 1.07 | 1.01; 4.8 (dp|pp) 0.98 to 1.02, (dp|dp) 1.1 to 1.7 |
-// 1.0; 6.0 (pp|pp) 1.0 to 4.0 | 1.06, (dp|pp) 1.0 to 2.1 | 1.0, (dp|dp) 1.4 to 4.6 | 1.09; 7.0
-// (dp|dp) 3.3 to 10 | 1.3; 8.0 (pp|pp) 1.7 to 27 | 3.4.
-constexpr float kFixSpreadBits = 5.0f;
-// Largest order the tile takes.  Above it one exponent for the integrals of all
-// orders costs more than the FP64 tile's roundings: relative 2-norm error against
-// the oracle, fixed point over FP64, plain form, K = 2 of ratio 3, pairs of two
-// centres in cubes of 1.5 | 4 | 8 bohr: (fd|pp), order 7, 3.4 | 2.1 | 1.2; (dd|dp), 7,
-// 2.3 | 1.6 | 1.1; (ff|pp), 8, 2.9 | 3.4 | 1.8; (dd|dd), 8, 1.6 | 1.9 | 1.2.  Order 6: (dp|dp) 0.97 |
-// 0.99 | 1.0, (dd|pp) 0.63 | 0.89 | 1.0; three primitives, the widest it takes, (dp|dp)
-// 1.5 | 1.1 | 1.0.  Order 5 and less: 0.6 to 1.02.
-constexpr int kFixLmax = 6;
+// log2 of the largest spread factor of a pair, and the largest order, for the
+// fixed-point tile: anywhere, and where a pair's centres lie kFixWide bohr apart.
+// Relative 2-norm error against the long double oracle, fixed point over FP64 in the
+// form that either would run, pairs of two centres (and half of one centre):
+//  cube of, bohr              1.5          4            8     12
+//  2.4 bits, (dp|dp), K = 2   0.8 (0.9)    0.7 (1.0)    0.9   1.0 (1.0)
+//  4.8 bits, (dp|dp), K = 3   1.1 (1.6)    0.7 (1.1)    0.5   1.0 (1.0)
+//  5.9 bits, (pp|pp), K = 2   2.7 (2.2)    0.9 (1.0)    1.0   1.3 (1.0)
+//            (dp|dp), K = 2   4.5 (6.0)    1.4 (2.1)    1.1   1.1 (1.2)
+//  order 7,  (dd|dp), K = 3   3.4 (4.1)    1.2 (1.6)    0.4   0.4 (1.0)
+//            (fd|pp), K = 2   2.6 (2.0)    1.2 (1.2)    0.6   0.8 (1.0)
+//  order 8,  (dd|dd), K = 3   3.7 (3.4)    1.5 (2.0)    1.1   0.4 (0.6)
+//            (ff|pp), K = 2   3.7 (2.9)    1.3 (1.2)    0.4   0.4 (0.7)
+//  order 9,  (fd|dd), K = 2                9.4          4.8   2.2 (2.1)
+//  order 10, (fd|fd), K = 2                13           8.7   7.6 (6.8)
+// (order 5 and less, 4.8 bits and less, both tiles in the plain form: 0.4 to 1.02)
+constexpr float kFixSpreadBits = 5.0f, kFixSpreadBitsWide = 6.0f;
+constexpr int kFixLmaxNear = 6, kFixLmax = 8;
+constexpr float kFixWide = 8.0f;
 static_assert(kFixLmax <= kFixAuxLmax, "order of the fixed-point auxiliary integrals");
 // products per low-limb accumulator between folds: each below 2^28 2^31.  Even:
 // the ket transform reads its operands in aligned pairs from each multiple on.
@@ -78,7 +83,7 @@ constexpr int kFixFold = 14;
 static_assert(kFixFold % 2 == 0, "pairs of ket primitives stay 16-byte aligned");
 
 // T = rho r^2 from which the Hermite unit follows the distance: s r >= 1.1 sqrt(8) = 3.1,
-// at most twice that, keeps N! / (s r)^N between 2^-7 and 1 for N <= 6
+// at most twice that, keeps N! / (s r)^N between 2^-7 and 2^3 for N <= 8
 constexpr float kFixFarT = 4.0f;
 // bits a bra column may lose to the shift of X before its quartet forms the limbs itself
 constexpr int kFixWeakBits = 4;

@@ -60,9 +60,10 @@ struct PrepassArgs {
     const int32_t* shell_off;
     const double* exps;
     int* kmin;   // optional [2]: INT_MAX less the smallest primitive-pair count K1 K2 over bra (ket) pairs
-    // optional [6]: the largest zeta_max / zeta_min of a bra (ket) pair (float
+    // optional [7]: the largest zeta_max / zeta_min of a bra (ket) pair (float
     // bits), 1 if a primitive lies outside the fixed-point tile's range, the
-    // largest |coordinate| and the largest zeta of a bra (ket) pair (float bits)
+    // largest |coordinate|, the largest zeta of a bra (ket) pair and the largest
+    // distance of a pair's centres (float bits)
     int* spread;
     const double* coefs;
 };
@@ -76,10 +77,16 @@ __device__ __forceinline__ bool fix_range(double z, double c)
 
 // zeta_max / zeta_min over the primitive pairs of shells s1, s2 (s2 < 0: the
 // unit function); *bad set where a primitive or centre is out of range, *far
-// raised to the largest |coordinate|, *zmax the largest zeta
-__device__ float pair_spread(const PrepassArgs& a, int s1, int s2, bool* bad, float* far, float* zmax)
+// raised to the largest |coordinate|, *wide to the distance of the centres, *zmax
+// the largest zeta
+__device__ float pair_spread(const PrepassArgs& a, int s1, int s2, bool* bad, float* far, float* wide, float* zmax)
 {
-    float lo = 0.f, hi = 0.f;
+    float lo = 0.f, hi = 0.f, r2 = 0.f;
+    for (int x = 0; x < 3 && s2 >= 0; ++x) {
+        const float d = (float)(a.centres[3 * a.shell_atom[s1] + x] - a.centres[3 * a.shell_atom[s2] + x]);
+        r2 = fmaf(d, d, r2);
+    }
+    *wide = fmaxf(*wide, sqrtf(r2));
     for (int c = 0; c < 2; ++c) {
         const int s = c ? s2 : s1;
         if (s < 0) continue;
@@ -140,7 +147,7 @@ __global__ void prepass_kernel(PrepassArgs a)
 {
     const int64_t n = max(max(a.nbra, a.nket), a.nq);
     // this thread's largest values, reduced per warp at the end
-    int kmax[4] = {0, 0, 0, 0}, kmin[2] = {0, 0}, risk[2] = {0, 0}, ratio[2] = {0, 0}, zeta[2] = {0, 0}, coord = 0;
+    int kmax[4] = {0, 0, 0, 0}, kmin[2] = {0, 0}, risk[2] = {0, 0}, ratio[2] = {0, 0}, zeta[2] = {0, 0}, coord = 0, apart = 0;
     for (int64_t i = blockIdx.x * (int64_t)blockDim.x + threadIdx.x; i < n; i += (int64_t)gridDim.x * blockDim.x) {
 #pragma unroll
         for (int side = 0; side < 2; ++side) {
@@ -180,8 +187,9 @@ __global__ void prepass_kernel(PrepassArgs a)
                     const int K1 = a.shell_K[s1], K2 = unit ? 1 : a.shell_K[s2];
                     if (K1 >= 1 && K1 <= kKmax && K2 >= 1 && K2 <= kKmax) {
                         bool bad = false;
-                        float far = 0.f, zmax;
-                        const float r = pair_spread(a, s1, unit ? -1 : s2, &bad, &far, &zmax);
+                        float far = 0.f, wide = 0.f, zmax;
+                        const float r = pair_spread(a, s1, unit ? -1 : s2, &bad, &far, &wide, &zmax);
+                        apart = max(apart, __float_as_int(wide));
                         zeta[side] = max(zeta[side], __float_as_int(zmax));
                         ratio[side] = max(ratio[side], __float_as_int(r));  // r >= 1: int order = float order
                         if (bad) a.spread[2] = 1;
@@ -214,7 +222,9 @@ __global__ void prepass_kernel(PrepassArgs a)
         warp_max_into(&a.spread[side], ratio[side]);
         warp_max_into(&a.spread[4 + side], zeta[side]);
     }
-    if (a.spread) warp_max_into(&a.spread[3], coord);
+    if (!a.spread) return;
+    warp_max_into(&a.spread[3], coord);
+    warp_max_into(&a.spread[6], apart);
 }
 
 // ---------------------------------------------------------------------------
@@ -805,16 +815,20 @@ static int dev_err_to_code(int e)
 static size_t align_up(size_t n) { return (n + 255) & ~size_t(255); }
 
 // Whether a batch of class cls may run the fixed-point tile: every primitive
-// in its range, and no pair whose exponents spread further than the scales
-// allow (eri_fixed.cuh).  info: PrepassArgs::spread.
+// in its range, and neither order nor exponents' spread beyond what its
+// precision allows (eri_fixed.cuh).  info: PrepassArgs::spread.
 static bool fixed_eligible(eri_class_t cls, const int32_t* info)
 {
     if (info[2]) return false;
+    float apart;
+    std::memcpy(&apart, &info[6], 4);
+    const bool wide = apart >= kFixWide;
+    if (cls.la + cls.lb + cls.lc + cls.ld > (wide ? kFixLmax : kFixLmaxNear)) return false;
     for (int side = 0; side < 2; ++side) {
         float r;
         std::memcpy(&r, &info[side], 4);
         const int l = side ? cls.lc + cls.ld : cls.la + cls.lb;
-        if (!(0.5f * (float)l * std::log2(r) <= kFixSpreadBits)) return false;
+        if (!(0.5f * (float)l * std::log2(r) <= (wide ? kFixSpreadBitsWide : kFixSpreadBits))) return false;
     }
     return true;
 }
@@ -956,10 +970,10 @@ int prepare_batch(eri_class_t cls, const eri_basis_t* basis, const int32_t* bra,
     if (!hinfo) return ERI_ENOMEM;
     // info lives in the status block (slots 8..16), separate from the error word:
     // [0..6] as PrepassArgs::info, [7..8] the smallest pair counts per side,
-    // [9..14] PrepassArgs::spread
+    // [9..15] PrepassArgs::spread
     int* dinfo = status + 8;
     // (one call: a small batch is bound by its launches, about 2 us each)
-    if (cudaMemsetAsync(dinfo, 0, 15 * sizeof(int), st) != cudaSuccess) return ERI_ECUDA;
+    if (cudaMemsetAsync(dinfo, 0, 16 * sizeof(int), st) != cudaSuccess) return ERI_ECUDA;
     // Where the fixed-point tile can be the faster one (GB300, ms, FP64 against fixed
     // point): contracted 4-centre classes above (ss|ss).  Not (ss|ss), 4e5 of mixed
     // degrees 5.12 / 5.37, whose tiles hold few primitive quartets; not uncontracted
@@ -991,11 +1005,11 @@ int prepare_batch(eri_class_t cls, const eri_basis_t* basis, const int32_t* bra,
     int32_t* hmapped = nullptr;
     if (cudaHostGetDevicePointer((void**)&hmapped, hinfo, 0) == cudaSuccess && hmapped) {
         count_launch();
-        info_to_host_kernel<<<1, 32, 0, st>>>(dinfo, 15, hmapped);
+        info_to_host_kernel<<<1, 32, 0, st>>>(dinfo, 16, hmapped);
         if (cudaGetLastError() != cudaSuccess) return ERI_ECUDA;
     } else {
         cudaGetLastError();
-        if (cudaMemcpyAsync(hinfo, dinfo, 15 * sizeof(int), cudaMemcpyDeviceToHost, st) != cudaSuccess)
+        if (cudaMemcpyAsync(hinfo, dinfo, 16 * sizeof(int), cudaMemcpyDeviceToHost, st) != cudaSuccess)
             return ERI_ECUDA;
     }
     if (cudaStreamSynchronize(st) != cudaSuccess) return ERI_ECUDA;
@@ -1347,19 +1361,20 @@ static bool tuned_tile(const FwdArgs& base, int split, cudaStream_t st, TilePlan
     cudaEventCreate(&e1);
     float best_ms = 3e38f;  // per quartet
     bool ok = false;
-    for (const TilePlan& tp : cands) {
+    // per quartet, over about `waves` waves of tiles (steady state) and at least
+    // kTuneQuartets quartets; 3e38: did not run
+    auto time_tile = [&](const TilePlan& tp, int waves) {
         FwdArgs a = base;
         set_tile(a, tp);
         void (*kern)(FwdArgs) = fwd_kern(split, tp.nt);
         if (cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)tp.bytes) != cudaSuccess) {
             cudaGetLastError();
-            continue;
+            return 3e38f;
         }
         int per_sm = 0;
         cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per_sm, kern, tp.nt, tp.bytes);
         const int64_t slots = (int64_t)std::max(per_sm, 1) * sm_count();
-        // about four waves of tiles (steady state), at least kTuneQuartets quartets
-        const int64_t nq = std::min(base.nq, std::max(kTuneQuartets, 4 * slots * tp.TQ));
+        const int64_t nq = std::min(base.nq, std::max(kTuneQuartets, waves * slots * tp.TQ));
         a.ntiles = (nq + tp.TQ - 1) / tp.TQ;
         const int64_t grid = std::min<int64_t>(a.ntiles, slots);
         // one warm-up launch, then the fastest of three timed ones: candidates
@@ -1379,14 +1394,35 @@ static bool tuned_tile(const FwdArgs& base, int split, cudaStream_t st, TilePlan
         }
         if (!timed) {
             cudaGetLastError();
-            continue;
+            return 3e38f;
         }
-        ms /= (float)nq;
+        return ms / (float)nq;
+    };
+    std::vector<float> first;
+    for (const TilePlan& tp : cands) {
+        const float ms = time_tile(tp, 4);
+        first.push_back(ms);
         if (ms < best_ms) {
             best_ms = ms;
             *best = tp;
             ok = true;
         }
+    }
+    if (split == XF_FIXED && ok) {
+        // fixed-point tiles of very different shapes tie in four waves and differ by
+        // 3 % over a batch ((pp|ps) K = 3, 1e5 quartets, 2.27 ms in 256 threads of 8
+        // quartets, 2.35 in 512 of 32): those within 4 % again, over 16 waves
+        const float close = 1.04f * best_ms;
+        best_ms = 3e38f;
+        for (size_t i = 0; i < cands.size(); ++i) {
+            if (first[i] > close) continue;
+            const float ms = time_tile(cands[i], 16);
+            if (ms < best_ms) {
+                best_ms = ms;
+                *best = cands[i];
+            }
+        }
+        ok = best_ms < 3e38f;
     }
     cudaEventDestroy(e0);
     cudaEventDestroy(e1);
@@ -1687,13 +1723,16 @@ static int run_forward(eri_class_t cls, const eri_basis_t* basis, const int32_t*
         err = select(&best);
         if (err != ERI_OK) return err;
         // Where fixed point is not surely the faster one, the FP64 tile is timed too,
-        // once per signature: fewer than 81 primitive quartets each, or (ss| on a side.
+        // once per signature: fewer than 81 primitive quartets each, or sides whose orders
+        // lie four apart or of which one is (ss|.
         // 20000 quartets, ms, FP64 against fixed point: K = 2 (pp|ss) 0.199 / 0.225, (dd|ss)
-        // 0.433 / 0.488, (pp|pp) 0.558 / 0.446; K = 3 (ff|ss) 3.81 / 5.39, (dd|ss) 1.26 / 1.06;
+        // 0.433 / 0.488, (pp|pp) 0.558 / 0.446; K = 3 (ff|ss) 3.81 / 5.39, (dd|ss) 1.26 / 1.06,
+        // (ff|ps) 5.21 / 5.65, (fd|ps) 4.15 / 4.34, (ff|ds) 11.0 / 10.9 (16384);
         // elsewhere 0.46 to 0.99 times FP64 for K = 3 and 4, (ps|ps) to (dp|dp).
         const int KB0 = (best.fc.form & 1) ? KK : KB, KK0 = (best.fc.form & 1) ? KB : KK;
         if (best.fc.fixed && best.tuned && g_fixed_mode == ERI_FIXED_RULE && g_form_mask.load() == 0xF &&
-            ((int64_t)KB * KK < kFixSmallPrims || cls.la + cls.lb == 0 || cls.lc + cls.ld == 0) &&
+            ((int64_t)KB * KK < kFixSmallPrims || cls.la + cls.lb == 0 || cls.lc + cls.ld == 0 ||
+             std::abs(cls.la + cls.lb - cls.lc - cls.ld) >= 4) &&
             lookup_fp64_faster(cls, KB0, KK0, kind) < 0) {
             Timed fp64;
             fp64.fc.no_fixed = 1;

@@ -124,6 +124,28 @@ def test_wide_exponents_and_non_finite_primitives_keep_the_fp64_tile():
     assert bad.any() and np.isnan(out[bad]).all() and np.isfinite(out[~bad]).all()
 
 
+@pytest.mark.parametrize("cls,ratio,fixed", [((2, 2, 2, 1), 3.0, True), ((2, 2, 2, 2), 3.0, True), ((3, 2, 1, 1), 3.0, True),
+                                             ((1, 1, 1, 1), 60.0, True), ((3, 2, 2, 2), 3.0, False),
+                                             ((1, 1, 1, 1), 70.0, False)])
+def test_wide_pairs_admit_order_eight_and_six_bits(cls, ratio, fixed):
+    """Pairs of centres up to 20 bohr apart: the tile takes order 8 and 6 bits of spread, where its error over the
+    batch is no larger than the FP64 tile's in the form that runs (to 1.3 for the samples of 120 blocks)."""
+    nq = 16384
+    basis, pools = synth.class_sweep_pools(seed=25, lmax=max(cls), pool=64, K=2, cube=12.0,
+                                           exps_fn=lambda rng, K: 0.2 * np.array([1.0, ratio]))
+    bra, ket, q = synth.class_sweep_batch(pools, cls, seed=26, npairs=60, nq=nq)
+    b, k, qq = to_device(bra, ket, q)
+    db = eri.DeviceBasis(basis)
+    ref = oracle_blocks(cls, basis, bra, ket, q[:120], prec="ld")
+    error = []
+    for mode in (eri.ERI_FIXED_ALWAYS, eri.ERI_FIXED_NEVER):
+        eri.eri_set_fixed(mode)
+        out = eri.eri_batch(cls, db, b, k, qq).cpu().numpy().reshape(-1, nq).T
+        assert eri.eri_last_arithmetic() == (eri.ERI_ARITH_FIXED if fixed and not error else eri.ERI_ARITH_FP64)
+        error.append(_sample_error(out[:120], ref))
+    assert error[0] <= 1.3 * error[1], error
+
+
 @pytest.mark.parametrize("ratio,fixed", [(30.0, True), (34.0, False), (60.0, False)])
 def test_spread_beyond_five_bits_keeps_the_fp64_tile(ratio, fixed):
     """(pp|pp), K = 2: a pair's exponents spread by log2(ratio) = 4.9, 5.1 and 5.9 bits, in a small cube, where spread
@@ -144,8 +166,8 @@ def test_spread_beyond_five_bits_keeps_the_fp64_tile(ratio, fixed):
 
 @pytest.mark.parametrize("cls", [(3, 2, 1, 1), (2, 2, 2, 1), (3, 3, 1, 1), (3, 2, 2, 2), (3, 2, 3, 2)])
 def test_orders_above_six_keep_the_fp64_tile(cls):
-    """Contracted classes of order 7 to 10: FP64 tile, whose error in the plain form stays near 1e-15 on these pairs
-    (in fixed point it was up to 3.4 times that at order 7 and 8, 1e-14 above)."""
+    """Contracted classes of order 7 to 10, centres within 7 bohr: FP64 tile, whose error in the plain form stays near
+    1e-15 on these pairs (in fixed point it was up to 3.4 times that at order 7 and 8, 1e-14 above)."""
     nq = 9382
     basis, pools = synth.class_sweep_pools(seed=3, lmax=3, pool=64, K=2, cube=4.0)
     bra, ket, q = synth.class_sweep_batch(pools, cls, seed=4, npairs=50, nq=nq)
