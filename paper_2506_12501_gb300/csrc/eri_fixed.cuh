@@ -514,15 +514,17 @@ inline size_t fix_table_bytes(const ClassTables& ct)
            2 * (2 * ct.Tab + 2 * ct.Tcd + ct.nhb * ct.nhk + ct.nhl + 2 * ct.nkpair + 2 * ct.nbpair);
 }
 
-// The tile's integer scratch: per (quartet, bra primitive) sigma, the bound g
-// (then its distance to the quartet's largest G), sigma_i - sigma, and flags: bit 0
-// the ket's E change there, bit 1 the quartet forms its bra limbs itself; per bra
-// primitive whether any quartet's E change; per quartet G and the largest rho for its distance; per (quartet, ket column)
-// the exponent H (largest sigma) and its distance to the current sigma's; per
-// (quartet, bra column) the exponent F.
+// The tile's scratch: ints, per (quartet, bra primitive) sigma and the bound g;
+// per bra primitive whether any quartet's ket E change there; per quartet G, the
+// largest exponent of the bounds, and the largest rho for its distance (a float);
+// per (quartet, ket column) the exponent H (largest sigma) and its distance to the
+// current sigma's.  Then 16-bit words (two tiles of some shapes only just share an
+// SM), per (quartet, bra primitive) sigma_i - sigma, and flags: bit 0 the ket's E
+// change there, bit 1 the quartet forms its bra limbs itself; per (quartet, bra
+// column) the exponent F.
 __host__ __device__ __forceinline__ int fix_scratch_ints(int TQ, int KB, int nab, int ncd)
 {
-    return 4 * TQ * KB + KB + 2 * TQ + 2 * TQ * ncd + TQ * nab;
+    return 2 * TQ * KB + KB + 2 * TQ + 2 * TQ * ncd + (2 * TQ * KB + TQ * nab + 1) / 2;
 }
 
 constexpr int kFixRegL = 4;  // auxiliary integrals in registers up to this order
@@ -543,14 +545,14 @@ __device__ void tile_fixed(const FwdArgs& a, int64_t q0, int nqt, double* sm, do
     int64_t* s_qq = reinterpret_cast<int64_t*>(sm + a.o_dj);
     int* s_sig = reinterpret_cast<int*>(sm + a.o_fx);
     int* s_g = s_sig + TQ * KB;
-    int* s_ds = s_g + TQ * KB;
-    int* s_ch = s_ds + TQ * KB;
-    int* s_any = s_ch + TQ * KB;
+    int* s_any = s_g + TQ * KB;
     int* s_G = s_any + KB;
-    int* s_dh = s_G + TQ;
+    float* s_lim = reinterpret_cast<float*>(s_G + TQ);
+    int* s_dh = s_G + 2 * TQ;
     int* s_H = s_dh + TQ * ncd;
-    int* s_F = s_H + TQ * ncd;
-    float* s_lim = reinterpret_cast<float*>(s_F + TQ * nab);
+    int16_t* s_ds = reinterpret_cast<int16_t*>(s_H + TQ * ncd);
+    int16_t* s_ch = s_ds + TQ * KB;
+    int16_t* s_F = s_ch + TQ * KB;
     const int lgTQ = 31 - __clz(TQ);  // TQ is a power of two
     const FastDiv d_ncd(ncd), d_kb(KB);
     __shared__ int s_kmax[2], s_next;
@@ -638,11 +640,11 @@ __device__ void tile_fixed(const FwdArgs& a, int64_t q0, int nqt, double* sm, do
         s_ds[idx] = on ? fix_sigma(sPb[idx].zeta, a.fx_c) - sg : 0;
         s_g[idx] = -1000;
     }
+    __syncthreads();
     for (int idx = tid; idx < TQ * ncd; idx += NT) {
         const int q = d_ncd.div(idx);
-        s_H[idx] = q < nqt ? norm_exp(q, idx - q * ncd, sigma_of(q, 0)) : 0;
+        s_H[idx] = q < nqt ? norm_exp(q, idx - q * ncd, s_sig[q * KB]) : 0;
     }
-    __syncthreads();
     // whether quartet q forms its bra limbs itself; lo: the smallest sigma_i - sigma
     auto own_limbs = [&](int q, int* lo) {
         int hi = 0;
