@@ -6,6 +6,11 @@
 // magnitudes are known beforehand, so they run here on 64-bit fixed-point
 // numbers, three multiply-adds per product; so do the auxiliary integrals (eri_fixaux.cuh).
 // The E products and the epilogue stay FP64.
+// What bounds it: no pipe.  (pp|ps) and (dp|pp), K = 3: issue slots 37 and 40 % busy,
+// the IMAD pipe 39 and 43 %, with the four warps a scheduler that 128 registers
+// leave; of 10 cycles an instruction 3 to 3.6 are barriers between the stages, 2 the
+// latency of dependent integer operations.  1e5 quartets of (pp|ps): FP64 tile 3.5 ms,
+// this one 2.26; 6.5e4 of (dp|pp): 10.7 and 8.1.
 //
 // Scales (all powers of two, so scaling rounds nothing):
 //  * Hermite orders carry a length: for bra primitive i a unit s = mu 2^sigma
@@ -85,7 +90,10 @@ static_assert(kFixFold % 2 == 0, "pairs of ket primitives stay 16-byte aligned")
 // T = rho r^2 from which the Hermite unit follows the distance: s r >= 1.1 sqrt(8) = 3.1,
 // at most twice that, keeps N! / (s r)^N between 2^-7 and 2^3 for N <= 8
 constexpr float kFixFarT = 4.0f;
-// bits a bra column may lose to the shift of X before its quartet forms the limbs itself
+// bits a bra column may lose to the shift of X before its quartet forms the limbs
+// itself (shifted throughout, components of (dp|ps) with one-centre bra pairs came out
+// 1.9e-11 of themselves off with bra exponents 2e3 times the ket's, 5.4e-9 with 1e5
+// times; FP64 4e-16)
 constexpr int kFixWeakBits = 4;
 
 template <int N>
